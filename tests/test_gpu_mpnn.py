@@ -169,3 +169,35 @@ def test_trained_proposal_against_random_and_idi_starts():
     idi = np.array(idi)
     assert np.all(idi > 0.56), idi
     assert fr.mean() > 0.92 * idi.mean(), (fr, idi)
+
+
+@pytest.mark.parametrize("hidden,layers", [(4, 1), (12, 2), (36, 3), (100, 2), (128, 1)])
+@pytest.mark.parametrize("n", [1, 63, 64, 65, 257])
+def test_tiles_and_widths_match_oracle(n, hidden, layers):
+    """Node tiles of 64, chunks of 256 and every kind of width (a warp's fraction, not a power of two, the
+    largest): inference, loss and gradient against FP64.  Bounds as above: FP32 dot products of at most 2 x 128
+    terms (2^-24 x 256 = 1.5e-5 of the sum of magnitudes, which is a few units here) and FP32 node sums."""
+    g = gg.er_graph(n, min(1.0, 6.0 / n), 50 + n) if n > 1 else gg.from_edges(1, [], [])
+    G = deco.graph_from(g)
+    m = deco.Mpnn(hidden, layers, 5)
+    theta = (m.get_params() + np.random.default_rng(n).normal(scale=0.05, size=m.n_params)).astype(np.float32)
+    m.set_params(theta)
+    t64 = theta.astype(np.float64)
+    h = torch.zeros(n, device=DEV)
+    m.infer(G, h, feat_seed=8)
+    o, _ = M.forward(t64, g, M.features(g, 8), hidden, layers)
+    np.testing.assert_allclose(h.cpu().numpy(), np.tanh(o), rtol=0, atol=3e-5)
+    z = gg.random_binary(n, 1, 7)[:, 0]
+    zd = torch.from_numpy(z).to(DEV)
+    grad = torch.zeros(m.n_params, device=DEV)
+    L, gref = M.loss_grad(t64, g, M.features(g, 8), z, hidden=hidden, layers=layers)
+    assert m.loss_grad(G, zd, grad, feat_seed=8) == pytest.approx(L, rel=1e-5, abs=1e-7)
+    assert m.loss_grad(G, zd, None, feat_seed=8) == pytest.approx(L, rel=1e-5, abs=1e-7)
+    assert np.max(np.abs(grad.cpu().numpy() - gref)) <= 1e-4 * np.max(np.abs(gref)) + 1e-6
+    # several steps in one call take the same path as single steps
+    ref = deco.Mpnn(hidden, layers, 5)
+    ref.set_params(theta)
+    m.set_params(theta)
+    one = [ref.train_step(G, zd, lr=1e-3, feat_seed=8) for _ in range(3)]
+    np.testing.assert_allclose(m.train(G, zd, 3, lr=1e-3, feat_seed=8), one, rtol=1e-12)
+    np.testing.assert_array_equal(m.get_params(), ref.get_params())
