@@ -143,7 +143,7 @@ extern "C" int deco_eval_cuts(const deco_graph* g, int32_t B, const uint8_t* z, 
   int rc = check_graph(g);
   if (rc) return rc;
   if (B < 1 || !z || !cuts) { set_error("bad arguments"); return DECO_ERR_ARG; }
-  return launch_cut_bytes(g, B, z, cuts, as_stream(stream));
+  return cut_bytes(g, B, z, cuts, as_stream(stream));
 }
 
 extern "C" int deco_eval_cut(const deco_graph* g, const uint8_t* z, int64_t* cut_out) {
@@ -159,7 +159,7 @@ extern "C" int deco_eval_cut(const deco_graph* g, const uint8_t* z, int64_t* cut
     int64_t* dc = nullptr;
     if ((rc = s.alloc(&dz, (size_t)g->n)) || (rc = s.alloc(&dc, sizeof(int64_t)))) return rc;
     DECO_CUDA_TRY(cudaMemcpyAsync(dz, z, (size_t)g->n, cudaMemcpyHostToDevice, st));
-    if ((rc = launch_cut_bytes(g, 1, dz, dc, st))) return rc;
+    if ((rc = cut_bytes(g, 1, dz, dc, st))) return rc;
     DECO_CUDA_TRY(cudaMemcpyAsync(&c, dc, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
   }
   DECO_CUDA_TRY(cudaStreamSynchronize(st));

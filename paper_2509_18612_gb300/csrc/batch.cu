@@ -73,39 +73,6 @@ void philox_host(uint32_t c[4], uint32_t k0, uint32_t k1) {
 double u01_host(uint32_t x) { return (2.0 * (double)(x >> 9) + 1.0) * 5.9604644775390625e-8; }
 
 // ---- per-graph bookkeeping kernels
-constexpr int GCUT_ROWS = 32;   // rows per warp
-
-__global__ void k_cut_graphs(int32_t n, int32_t B, int32_t W, const int32_t* row_ptr, const int32_t* col_idx,
-                             const int32_t* wint, const uint32_t* zbits, const int32_t* gid, int64_t* cuts) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int32_t k = blockIdx.y;
-  const int64_t r0 = warp * GCUT_ROWS;
-  if (r0 >= n) return;
-  const int32_t r1 = (int32_t)std::min<int64_t>(n, r0 + GCUT_ROWS);
-  const int32_t b = k * 32 + lane;
-  long long acc = 0;
-  int32_t cg = gid[r0];
-  for (int32_t v = (int32_t)r0; v < r1; ++v) {
-    const int32_t g = gid[v];
-    if (g != cg) {
-      if (b < B && acc) atomicAdd(reinterpret_cast<unsigned long long*>(cuts + (size_t)cg * B + b), (unsigned long long)acc);
-      acc = 0;
-      cg = g;
-    }
-    const uint32_t zv = zbits[(size_t)v * W + k];
-    int32_t racc = 0;
-    for (int32_t e = row_ptr[v]; e < row_ptr[v + 1]; ++e) {
-      const int32_t u = col_idx[e];
-      if (u <= v) continue;
-      const uint32_t x = (zv ^ zbits[(size_t)u * W + k]) >> lane & 1u;
-      racc += wint ? (int32_t)x * wint[e] : (int32_t)x;
-    }
-    acc += racc;
-  }
-  if (b < B && acc) atomicAdd(reinterpret_cast<unsigned long long*>(cuts + (size_t)cg * B + b), (unsigned long long)acc);
-}
-
 // one block per graph: lowest index among the maximal cuts
 __global__ void k_argmax_graphs(int32_t B, const int64_t* cuts, int32_t* best) {
   __shared__ long long sv[256];
@@ -705,10 +672,7 @@ extern "C" int deco_solve_batch(const deco_batch* b, int32_t B, const deco_param
             return e2;
         }
         if ((e2 = launch_pack(U, B, lift, ld, p->precision, ybuf[cur], zbits, st))) return e2;
-        ce = cudaMemsetAsync(cuts, 0, sizeof(int64_t) * (size_t)G * B, st);
-        if (ce != cudaSuccess) return cuda_fail(ce, "memset cuts");
-        dim3 grid((unsigned)((((int64_t)n + GCUT_ROWS - 1) / GCUT_ROWS + 7) / 8), (unsigned)W);
-        k_cut_graphs<<<grid, 256, 0, st>>>(n, B, W, U->row_ptr, U->col_idx, U->wint, zbits, b->gid, cuts);
+        if ((e2 = launch_cut_graphs(U, B, zbits, b->goff, G, cuts, st))) return e2;
         k_argmax_graphs<<<G, 256, 0, st>>>(B, cuts, best_idx);
         k_record_graphs<<<(G + 127) / 128, 128, 0, st>>>(G, B, cuts, best_idx, d_round, rec_cut, rec_round, improved);
         k_extract_graphs<<<(n + 255) / 256, 256, 0, st>>>(n, W, zbits, b->gid, best_idx, improved, rbz, bz);

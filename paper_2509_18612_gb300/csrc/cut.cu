@@ -1,17 +1,27 @@
 // Rounding, integer cut evaluation and argmax over starting points
 // (the rounding and selection steps of Alg. 1 / Alg. 2; Eq. 5, Eq. 11, Eq. 1).
 //
-//  pack:   one warp per (row, 32 starting points); lane b forms z_{v,b} from
-//          the iterate and __ballot_sync packs the 32 bits into one word.
-//  cut:    one warp per (row block, word); lane b accumulates
-//          w_uv * ((z_v xor z_u) >> b & 1) over the neighbours u > v of its
-//          rows (each unordered edge once), in integers; the block reduces and
-//          issues one 64-bit atomic per starting point.  Integer atomics are
-//          associative, so the result is exact and run-to-run identical.
+//  pack:   one thread per (row, 8 starting points) reads their columns as
+//          16-byte vectors and writes 8 bits; blocks whose rows are not
+//          16-byte aligned, and lifts above 4, take one warp per (row, 32
+//          starting points) and a ballot.
+//  cut:    warps take equal ranges of the stored entries, a lane per entry:
+//          the words z_v xor z_u of 32 entries form a 32 x 32 bit matrix that
+//          the warp transposes, so that lane b counts starting point b with
+//          one popc (weights: one per bit of |w| and sign).  Entries with
+//          u > v count (each unordered edge once), in integers; the block
+//          reduces and issues one 64-bit atomic per starting point.  Integer
+//          sums are exact in any order.
 //  argmax: one block; lowest index among the maximal cuts.
+#include <algorithm>
+
+#include "api_util.cuh"
 #include "deco_internal.cuh"
 
 namespace deco {
+
+int device_sm_count();
+
 namespace {
 
 template <int PREC>
@@ -44,59 +54,195 @@ __global__ void k_pack(int32_t n, int32_t B, int32_t lift, int32_t ld, int32_t W
   if (lane == 0) zbits[(size_t)v * W + k] = word;
 }
 
-constexpr int CUT_BLOCK = 256;
-
-// zb(v, k): word k of row v, either from packed bits or from a byte matrix.
-struct BitsSrc {
-  const uint32_t* zbits;  // n x W
-  int32_t W;
-  __device__ __forceinline__ uint32_t word(int32_t v, int32_t k) const {
-    return __ldg(zbits + (size_t)v * W + k);
-  }
-};
-struct BytesSrc {
-  const uint8_t* z;  // n x B
-  int32_t B;
-  __device__ __forceinline__ uint32_t word(int32_t v, int32_t k) const {
-    // lane-independent word assembled from 32 bytes (used only by deco_eval_cuts)
-    uint32_t w = 0;
-    const int32_t b0 = k * 32;
-    for (int i = 0; i < 32 && b0 + i < B; ++i) w |= (z[(size_t)v * B + b0 + i] ? 1u : 0u) << i;
-    return w;
-  }
-};
-
-template <typename Src>
-__global__ void __launch_bounds__(CUT_BLOCK) k_cut(int32_t n, int32_t B, int32_t W,
-                                                   const int32_t* row_ptr, const int32_t* col_idx,
-                                                   const int32_t* wint, Src src, int64_t* cuts) {
-  __shared__ long long part[CUT_BLOCK / 32][32];
-  const int lane = threadIdx.x & 31;
-  const int wib = threadIdx.x >> 5;
-  const int32_t k = blockIdx.y;                      // word (32 starting points)
-  const int64_t warps_total = (int64_t)gridDim.x * (CUT_BLOCK / 32);
-  long long acc = 0;
-  for (int64_t v64 = (int64_t)blockIdx.x * (CUT_BLOCK / 32) + wib; v64 < n; v64 += warps_total) {
-    const int32_t v = (int32_t)v64;
-    const uint32_t zv = src.word(v, k);
-    const int32_t e0 = __ldg(row_ptr + v), e1 = __ldg(row_ptr + v + 1);
-    int32_t racc = 0;   // |sum| <= sum |w| over the row <= 2^24 (checked at creation)
-    // neighbours are sorted: skip u < v, keep u > v (each unordered edge once)
-    for (int32_t e = e0; e < e1; ++e) {
-      const int32_t u = __ldg(col_idx + e);
-      if (u <= v) continue;
-      const uint32_t x = (zv ^ src.word(u, k)) >> lane & 1u;
-      racc += wint ? (int32_t)x * __ldg(wint + e) : (int32_t)x;
+// Byte q of row v: starting points 8q ... 8q + 7, i.e. columns 8 q LIFT ... of
+// the row, 16-byte aligned (ld % 8 == 0).  A vector may reach past column C
+// but not past ld; points >= B give 0.  Bound by HBM: 10^6 rows of 128 BF16
+// columns in 64 us (4.2 TB/s); a warp per word, 2 bytes a lane, took 456.
+template <int PREC, int LIFT>
+__global__ void __launch_bounds__(256) k_pack_vec(int32_t n, int32_t B, int32_t ld, int32_t W, const void* y,
+                                                  uint8_t* zbytes) {
+  constexpr int VN = PREC == DECO_PREC_BF16 ? 8 : 4;    // values of a vector
+  constexpr int NV = 8 * LIFT / VN;                     // vectors of 8 points
+  const int64_t total = (int64_t)n * W * 4, step = (int64_t)gridDim.x * blockDim.x;
+  const int32_t W4 = W * 4;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += step) {
+    const int32_t v = (int32_t)(i / W4), q = (int32_t)(i % W4);
+    uint32_t bits = 0;
+    const int32_t c0 = 8 * q * LIFT;
+    const uint4* src = reinterpret_cast<const uint4*>(static_cast<const char*>(y) +
+                                                      ((size_t)v * ld + c0) * (PREC == DECO_PREC_BF16 ? 2 : 4));
+    uint4 raw[NV];
+#pragma unroll
+    for (int h = 0; h < NV; ++h) {
+      raw[h] = make_uint4(0u, 0u, 0u, 0u);
+      if (c0 + h * VN < B * LIFT) raw[h] = __ldg(src + h);
     }
-    acc += racc;
+    float val[8 * LIFT];
+#pragma unroll
+    for (int h = 0; h < NV; ++h) {
+      const uint32_t u[4] = {raw[h].x, raw[h].y, raw[h].z, raw[h].w};
+#pragma unroll
+      for (int k = 0; k < VN; ++k) {
+        if (PREC == DECO_PREC_FP32) val[h * VN + k] = __uint_as_float(u[k % 4]);
+        else val[h * VN + k] = (k & 1) ? bf16hi(u[k / 2]) : bf16lo(u[k / 2]);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      bool bit;
+      if (LIFT == 1) {
+        bit = val[k] > 0.0f;                             // Eq. 5: strict
+      } else {
+        float s = 0.0f;
+#pragma unroll
+        for (int l = 0; l < LIFT; ++l) s += val[k * LIFT + l];
+        bit = s >= 0.0f;                                 // Eq. 11: non-strict
+      }
+      if (bit && 8 * q + k < B) bits |= 1u << k;
+    }
+    zbytes[i] = (uint8_t)bits;
   }
-  part[wib][lane] = acc;
+}
+
+// 0/1 bytes (n x B, any nonzero byte counts as 1) to bits: a warp per (row, word)
+__global__ void k_bytes_to_bits(int32_t n, int32_t B, int32_t W, const uint8_t* z, uint32_t* bits) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < (int64_t)n * W; i += warps) {
+    const int32_t v = (int32_t)(i / W), b = (int32_t)(i % W) * 32 + lane;
+    const uint32_t word = __ballot_sync(0xFFFFFFFFu, b < B && z[(size_t)v * B + b] != 0);
+    if (lane == 0) bits[i] = word;
+  }
+}
+
+// lane b of the result holds, at bit e, bit b of lane e's x
+__device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
+#pragma unroll
+  for (int s = 16; s >= 1; s >>= 1) {
+    const uint32_t m = s == 16 ? 0x0000FFFFu : s == 8 ? 0x00FF00FFu : s == 4 ? 0x0F0F0F0Fu : s == 2 ? 0x33333333u
+                                                                                                   : 0x55555555u;
+    const uint32_t y = __shfl_xor_sync(0xFFFFFFFFu, x, s);
+    x = (lane & s) ? ((x & ~m) | ((y >> s) & m)) : ((x & m) | ((y & m) << s));
+  }
+  return x;
+}
+
+constexpr int CUT_BLOCK = 256;
+constexpr int CUT_U = 2;   // batches of 32 entries in flight per warp
+
+// Cuts of the starting points of V words (word group blockIdx.y) over the
+// rows of graph blockIdx.z (goff: first rows; null: all n rows), added to
+// cuts[graph B + b].  Bound by the latency of the gathered words and the
+// transposes' issue slots: 10^6 nodes, degree 10, 128 starting points in
+// 108 us; a warp per row that walked its neighbours one by one took 1 059.
+template <int V, bool WT>
+__global__ void __launch_bounds__(CUT_BLOCK) k_cut(int32_t n, int32_t B, int32_t W, const int32_t* __restrict__ row_ptr,
+                                                   const int32_t* __restrict__ col_idx, const int32_t* __restrict__ wint,
+                                                   int wbits, const uint32_t* __restrict__ zbits,
+                                                   const int32_t* __restrict__ goff, int64_t* cuts) {
+  __shared__ long long part[CUT_BLOCK / 32][32 * V];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const int32_t k0 = blockIdx.y * V, g = blockIdx.z;
+  const int32_t ra = goff ? __ldg(goff + g) : 0, rb = goff ? __ldg(goff + g + 1) : n;
+  const int64_t Ea = __ldg(row_ptr + ra), Eb = __ldg(row_ptr + rb);
+  const int64_t warps = (int64_t)gridDim.x * (CUT_BLOCK / 32);
+  const int64_t per = ((Eb - Ea + warps - 1) / warps + 31) / 32 * 32;
+  int64_t e = Ea + ((int64_t)blockIdx.x * (CUT_BLOCK / 32) + wib) * per;
+  const int64_t E1 = min(Eb, e + per);
+  long long acc[V];
+#pragma unroll
+  for (int j = 0; j < V; ++j) acc[j] = 0;
+  if (e < E1) {
+    // the row that holds entry e: row_ptr[r] <= e < row_ptr[r + 1]
+    int32_t lo = ra, hi = rb;
+    while (hi - lo > 1) {
+      const int32_t step = (hi - lo + 31) / 32;
+      const int64_t p = lo + (int64_t)(lane + 1) * step;
+      const int cnt = __popc(__ballot_sync(0xFFFFFFFFu, p < hi && __ldg(row_ptr + p) <= e));
+      lo += cnt * step;
+      hi = min(hi, lo + step);
+    }
+    // window of 32 rows: lane i holds the end of row r + i
+    int32_t r = lo;
+    int32_t end = __ldg(row_ptr + min(r + lane + 1, rb));
+    while (e < E1) {
+      const int32_t last = __shfl_sync(0xFFFFFFFFu, end, 31);
+      if (last <= e) {
+        r += 32;
+        end = __ldg(row_ptr + min(r + lane + 1, rb));
+        continue;
+      }
+      const int64_t lim = min(E1, (int64_t)last);
+      for (; e < lim; e += 32 * CUT_U) {
+        int32_t row[CUT_U], u[CUT_U], w[CUT_U];
+#pragma unroll
+        for (int q = 0; q < CUT_U; ++q) {
+          const int64_t x = e + 32 * q + lane;
+          u[q] = -1;
+          w[q] = 1;
+          if (x < lim) {
+            u[q] = __ldg(col_idx + x);
+            if (WT) w[q] = __ldg(wint + x);
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < CUT_U; ++q) {
+          const int64_t x = e + 32 * q + lane;
+          int pos = 0;   // rows of the window that end at or before entry x
+#pragma unroll
+          for (int s = 16; s >= 1; s >>= 1)
+            if (__shfl_sync(0xFFFFFFFFu, end, pos + s - 1) <= x) pos += s;
+          row[q] = r + pos;
+        }
+        uint32_t d[CUT_U][V];
+#pragma unroll
+        for (int q = 0; q < CUT_U; ++q) {
+#pragma unroll
+          for (int j = 0; j < V; ++j) d[q][j] = 0u;
+          if (u[q] > row[q]) {
+            const uint32_t* zu = zbits + (size_t)u[q] * W + k0;
+            const uint32_t* zv = zbits + (size_t)row[q] * W + k0;
+            if (V == 4) {
+              const uint4 a = __ldg(reinterpret_cast<const uint4*>(zu)), b = __ldg(reinterpret_cast<const uint4*>(zv));
+              d[q][0] = a.x ^ b.x; d[q][1 % V] = a.y ^ b.y; d[q][2 % V] = a.z ^ b.z; d[q][3 % V] = a.w ^ b.w;
+            } else if (V == 2) {
+              const uint2 a = __ldg(reinterpret_cast<const uint2*>(zu)), b = __ldg(reinterpret_cast<const uint2*>(zv));
+              d[q][0] = a.x ^ b.x; d[q][1 % V] = a.y ^ b.y;
+            } else {
+              d[q][0] = __ldg(zu) ^ __ldg(zv);
+            }
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < CUT_U; ++q) {
+#pragma unroll
+          for (int j = 0; j < V; ++j) d[q][j] = transpose32(d[q][j], lane);
+          if (!WT) {
+#pragma unroll
+            for (int j = 0; j < V; ++j) acc[j] += __popc(d[q][j]);
+          } else {
+            for (int h = 0; h < wbits; ++h) {
+              const uint32_t pos = __ballot_sync(0xFFFFFFFFu, w[q] > 0 && ((w[q] >> h) & 1));
+              const uint32_t neg = __ballot_sync(0xFFFFFFFFu, w[q] < 0 && ((-w[q] >> h) & 1));
+#pragma unroll
+              for (int j = 0; j < V; ++j)
+                acc[j] += (long long)(__popc(d[q][j] & pos) - __popc(d[q][j] & neg)) << h;
+            }
+          }
+        }
+      }
+      e = lim;
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < V; ++j) part[wib][32 * j + lane] = acc[j];
   __syncthreads();
-  if (wib == 0) {
+  for (int x = threadIdx.x; x < 32 * V; x += CUT_BLOCK) {
     long long s = 0;
-    for (int i = 0; i < CUT_BLOCK / 32; ++i) s += part[i][lane];
-    const int32_t b = k * 32 + lane;
-    if (b < B && s != 0) atomicAdd(reinterpret_cast<unsigned long long*>(cuts + b), (unsigned long long)s);
+    for (int i = 0; i < CUT_BLOCK / 32; ++i) s += part[i][x];
+    const int32_t b = 32 * k0 + x;
+    if (b < B && s != 0)
+      atomicAdd(reinterpret_cast<unsigned long long*>(cuts + (size_t)g * B + b), (unsigned long long)s);
   }
 }
 
@@ -152,14 +298,28 @@ __global__ void k_extract(int32_t n, int32_t W, const uint32_t* zbits, const int
   if (rec->improved && best_z) best_z[v] = z;
 }
 
-int cut_grid_x(const deco_graph* g, int32_t W) {
-  int dev_sms = 152;
-  int dev = 0;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, dev);
-  int64_t want = ((int64_t)g->n + CUT_BLOCK / 32 - 1) / (CUT_BLOCK / 32);
-  int64_t cap = (int64_t)dev_sms * 8 / (W > 0 ? W : 1);
-  if (cap < dev_sms) cap = dev_sms;
-  return (int)(want < cap ? (want > 0 ? want : 1) : cap);
+template <int V>
+void launch_cut_v(const deco_graph* g, int32_t B, int32_t W, const uint32_t* zbits, const int32_t* goff, int32_t graphs,
+                  int64_t* cuts, cudaStream_t st) {
+  // enough warps to keep every SM's slots filled, at least 64 entries each
+  const int groups = W / V;
+  const int64_t want = (g->nnz / graphs + CUT_BLOCK * 2 - 1) / (CUT_BLOCK * 2);
+  const int64_t cap = std::max<int64_t>(1, (int64_t)device_sm_count() * 8 / ((int64_t)groups * graphs));
+  const dim3 grid((unsigned)std::max<int64_t>(1, std::min(want, cap)), (unsigned)groups, (unsigned)graphs);
+  int wbits = 1;
+  while (wbits < 31 && (g->max_abs_w >> wbits)) ++wbits;
+  if (g->wint)
+    k_cut<V, true><<<grid, CUT_BLOCK, 0, st>>>(g->n, B, W, g->row_ptr, g->col_idx, g->wint, wbits, zbits, goff, cuts);
+  else
+    k_cut<V, false><<<grid, CUT_BLOCK, 0, st>>>(g->n, B, W, g->row_ptr, g->col_idx, nullptr, 1, zbits, goff, cuts);
+}
+
+template <int PREC, int LIFT>
+void launch_pack_vec(const deco_graph* g, int32_t B, int32_t ld, int32_t W, const void* y, uint32_t* zbits,
+                     cudaStream_t st) {
+  const int64_t blocks = ((int64_t)g->n * W * 4 + 255) / 256;
+  k_pack_vec<PREC, LIFT><<<(unsigned)std::min<int64_t>(blocks, (int64_t)device_sm_count() * 64), 256, 0, st>>>(
+      g->n, B, ld, W, y, reinterpret_cast<uint8_t*>(zbits));
 }
 
 }  // namespace
@@ -167,6 +327,21 @@ int cut_grid_x(const deco_graph* g, int32_t W) {
 int launch_pack(const deco_graph* g, int32_t B, int32_t lift, int32_t ld, int precision,
                 const void* y, uint32_t* zbits, cudaStream_t st) {
   const int32_t W = (B + 31) / 32;
+  if (lift <= 4 && ld % 8 == 0 && reinterpret_cast<uintptr_t>(y) % 16 == 0) {
+    if (precision == DECO_PREC_BF16) {
+      if (lift == 1) launch_pack_vec<DECO_PREC_BF16, 1>(g, B, ld, W, y, zbits, st);
+      else if (lift == 2) launch_pack_vec<DECO_PREC_BF16, 2>(g, B, ld, W, y, zbits, st);
+      else if (lift == 3) launch_pack_vec<DECO_PREC_BF16, 3>(g, B, ld, W, y, zbits, st);
+      else launch_pack_vec<DECO_PREC_BF16, 4>(g, B, ld, W, y, zbits, st);
+    } else {
+      if (lift == 1) launch_pack_vec<DECO_PREC_FP32, 1>(g, B, ld, W, y, zbits, st);
+      else if (lift == 2) launch_pack_vec<DECO_PREC_FP32, 2>(g, B, ld, W, y, zbits, st);
+      else if (lift == 3) launch_pack_vec<DECO_PREC_FP32, 3>(g, B, ld, W, y, zbits, st);
+      else launch_pack_vec<DECO_PREC_FP32, 4>(g, B, ld, W, y, zbits, st);
+    }
+    DECO_CUDA_TRY(cudaGetLastError());
+    return DECO_OK;
+  }
   const int64_t threads = (int64_t)g->n * W * 32;
   const int block = 256;
   const unsigned grid = (unsigned)((threads + block - 1) / block);
@@ -176,26 +351,44 @@ int launch_pack(const deco_graph* g, int32_t B, int32_t lift, int32_t ld, int pr
   return DECO_OK;
 }
 
+int launch_cut_graphs(const deco_graph* g, int32_t B, const uint32_t* zbits, const int32_t* goff, int32_t graphs,
+                      int64_t* cuts, cudaStream_t st) {
+  const int32_t W = (B + 31) / 32;
+  DECO_CUDA_TRY(cudaMemsetAsync(cuts, 0, sizeof(int64_t) * (size_t)B * graphs, st));
+  // the widest vector of words that every row's words are aligned to
+  const uintptr_t at = reinterpret_cast<uintptr_t>(zbits);
+  for (int32_t g0 = 0; g0 < graphs; g0 += 65535) {   // grid limit
+    const int32_t gc = std::min(graphs - g0, 65535);
+    const int32_t* go = goff ? goff + g0 : nullptr;
+    int64_t* c = cuts + (size_t)g0 * B;
+    if (W % 4 == 0 && at % 16 == 0) launch_cut_v<4>(g, B, W, zbits, go, gc, c, st);
+    else if (W % 2 == 0 && at % 8 == 0) launch_cut_v<2>(g, B, W, zbits, go, gc, c, st);
+    else launch_cut_v<1>(g, B, W, zbits, go, gc, c, st);
+    DECO_CUDA_TRY(cudaGetLastError());
+  }
+  return DECO_OK;
+}
+
 int launch_cut_bits(const deco_graph* g, int32_t B, const uint32_t* zbits, int64_t* cuts,
                     cudaStream_t st) {
+  return launch_cut_graphs(g, B, zbits, nullptr, 1, cuts, st);
+}
+
+int launch_bytes_to_bits(int32_t n, int32_t B, const uint8_t* z, uint32_t* bits, cudaStream_t st) {
   const int32_t W = (B + 31) / 32;
-  DECO_CUDA_TRY(cudaMemsetAsync(cuts, 0, sizeof(int64_t) * (size_t)B, st));
-  dim3 grid(cut_grid_x(g, W), W);
-  BitsSrc src{zbits, W};
-  k_cut<BitsSrc><<<grid, CUT_BLOCK, 0, st>>>(g->n, B, W, g->row_ptr, g->col_idx, g->wint, src, cuts);
+  const int64_t blocks = ((int64_t)n * W + 7) / 8;
+  k_bytes_to_bits<<<(unsigned)std::min<int64_t>(blocks, (int64_t)device_sm_count() * 64), 256, 0, st>>>(n, B, W, z,
+                                                                                                       bits);
   DECO_CUDA_TRY(cudaGetLastError());
   return DECO_OK;
 }
 
-int launch_cut_bytes(const deco_graph* g, int32_t B, const uint8_t* z, int64_t* cuts,
-                     cudaStream_t st) {
-  const int32_t W = (B + 31) / 32;
-  DECO_CUDA_TRY(cudaMemsetAsync(cuts, 0, sizeof(int64_t) * (size_t)B, st));
-  dim3 grid(cut_grid_x(g, W), W);
-  BytesSrc src{z, B};
-  k_cut<BytesSrc><<<grid, CUT_BLOCK, 0, st>>>(g->n, B, W, g->row_ptr, g->col_idx, g->wint, src, cuts);
-  DECO_CUDA_TRY(cudaGetLastError());
-  return DECO_OK;
+int cut_bytes(const deco_graph* g, int32_t B, const uint8_t* z, int64_t* cuts, cudaStream_t st) {
+  Scratch s(st);
+  uint32_t* bits = nullptr;
+  int rc = s.alloc(&bits, sizeof(uint32_t) * (size_t)g->n * ((B + 31) / 32));
+  if (rc || (rc = launch_bytes_to_bits(g->n, B, z, bits, st))) return rc;
+  return launch_cut_bits(g, B, bits, cuts, st);
 }
 
 int launch_argmax(int32_t B, const int64_t* cuts, int32_t* best, cudaStream_t st) {

@@ -216,8 +216,13 @@ int launch_pack(const deco_graph* g, int32_t B, int32_t lift, int32_t ld, int pr
                 const void* y, uint32_t* zbits, cudaStream_t st);
 int launch_cut_bits(const deco_graph* g, int32_t B, const uint32_t* zbits, int64_t* cuts,
                     cudaStream_t st);
-int launch_cut_bytes(const deco_graph* g, int32_t B, const uint8_t* z, int64_t* cuts,
-                     cudaStream_t st);
+// the same per graph of a disjoint union: graph i's rows are goff[i] ... goff[i + 1] - 1 (device), its cuts at i B
+int launch_cut_graphs(const deco_graph* g, int32_t B, const uint32_t* zbits, const int32_t* goff, int32_t graphs,
+                      int64_t* cuts, cudaStream_t st);
+// n x B bytes (nonzero = 1) to n x ceil(B/32) words
+int launch_bytes_to_bits(int32_t n, int32_t B, const uint8_t* z, uint32_t* bits, cudaStream_t st);
+// cuts of byte columns, through a packed scratch copy
+int cut_bytes(const deco_graph* g, int32_t B, const uint8_t* z, int64_t* cuts, cudaStream_t st);
 int launch_argmax(int32_t B, const int64_t* cuts, int32_t* best, cudaStream_t st);
 // 1-flip local search on bit-packed columns (n x ceil(B/32) words), in place;
 // gains: n x 32 ceil(B/32) int32 scratch, changed: max_rounds + 1 int32 scratch

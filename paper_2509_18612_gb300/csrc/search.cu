@@ -84,15 +84,7 @@ __global__ void k_greedy(int32_t n, int32_t B, const int32_t* row_ptr, const int
   }
 }
 
-// bytes (n x B) <-> bits (n x W words, bit b % 32 of word b / 32)
-__global__ void k_bytes_to_bits(int32_t n, int32_t B, int32_t W, const uint8_t* z, uint32_t* bits) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (int64_t)n * W) return;
-  const int32_t v = (int32_t)(i / W), k = (int32_t)(i % W);
-  uint32_t w = 0;
-  for (int c = 0; c < 32 && 32 * k + c < B; ++c) w |= (z[(size_t)v * B + 32 * k + c] ? 1u : 0u) << c;
-  bits[i] = w;
-}
+// bits (n x W words, bit b % 32 of word b / 32) -> bytes (n x B)
 __global__ void k_bits_to_bytes(int32_t n, int32_t B, int32_t W, const uint32_t* bits, uint8_t* z) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (int64_t)n * B) return;
@@ -203,7 +195,7 @@ extern "C" int deco_greedy(const deco_graph* g, int32_t B, uint64_t seed, uint8_
     k_greedy<<<blocks_for((int64_t)B * 32, 128), 128, 0, st>>>(g->n, B, g->row_ptr, g->col_idx, g->wint, order, z);
     DECO_CUDA_TRY(cudaGetLastError());
   }
-  return launch_cut_bytes(g, B, z, cuts, st);
+  return cut_bytes(g, B, z, cuts, st);
 }
 
 extern "C" int deco_local_search(const deco_graph* g, int32_t B, uint8_t* z, int32_t max_rounds, int64_t* cuts,
@@ -223,12 +215,12 @@ extern "C" int deco_local_search(const deco_graph* g, int32_t B, uint8_t* z, int
       (rc = s.alloc(&changed, sizeof(int32_t) * (size_t)(max_rounds + 1))))
     return rc;
   if (g->n > 0) {
-    k_bytes_to_bits<<<blocks_for((int64_t)g->n * W, 256), 256, 0, st>>>(g->n, B, W, z, bits);
+    if ((rc = launch_bytes_to_bits(g->n, B, z, bits, st))) return rc;
     if ((rc = launch_local_search(g, B, bits, max_rounds, gains, changed, st))) return rc;
     k_bits_to_bytes<<<blocks_for((int64_t)g->n * B, 256), 256, 0, st>>>(g->n, B, W, bits, z);
     DECO_CUDA_TRY(cudaGetLastError());
   }
-  if (cuts && (rc = launch_cut_bytes(g, B, z, cuts, st))) return rc;
+  if (cuts && (rc = launch_cut_bits(g, B, bits, cuts, st))) return rc;
   if (rounds) {
     std::vector<int32_t> h((size_t)max_rounds + 1, 0);
     DECO_CUDA_TRY(cudaMemcpyAsync(h.data(), changed, sizeof(int32_t) * h.size(), cudaMemcpyDeviceToHost, st));

@@ -191,3 +191,68 @@ def test_smem_probe_rate_is_plausible():
     for width in (8, 16):
         gbs = deco.deco_probe_smem_rate(width, 1 << 14)
         assert 0.1 * derived < gbs < 1.1 * derived, (width, gbs)
+
+
+CUT_GRAPHS = {
+    "star": lambda rng: gg.from_edges(700, np.zeros(699, int), np.arange(1, 700)),      # one hub row, 699 short rows
+    "gaps": lambda rng: gg.from_edges(500, [3, 400, 401], [499, 401, 499]),             # windows of empty rows
+    "er": lambda rng: gg.er_graph(333, 0.03, 5),
+    "signed": lambda rng: _weighted(gg.er_graph(257, 0.05, 6), rng.choice([-1.0, 1.0], 100000)),
+    "large weights": lambda rng: _weighted(gg.ba_graph(150, 4, 7), rng.choice([-2.0 ** 20, 2.0 ** 20, 3.0, -77.0], 100000)),
+}
+
+
+def _weighted(g, w):
+    u, v, _ = g.edges()
+    if np.abs(w).max() > 1000:     # a row's |w| may sum to 2^24 at most
+        deg = np.diff(g.row_ptr)
+        w = np.where(np.maximum(deg[u], deg[v]) < 16, w[:u.size], 5.0)
+    return gg.from_edges(g.n, u, v, w[:u.size])
+
+
+@pytest.mark.parametrize("B", [1, 31, 32, 33, 64, 96, 128, 130])
+@pytest.mark.parametrize("name", list(CUT_GRAPHS))
+def test_cut_sums_over_entry_ranges_are_exact(name, B):
+    # word vectors of 1, 2 and 4, ragged last words, hub rows, empty windows, every bit of the weights; the same
+    # vectors as bytes, and from a word buffer that is only 4-byte aligned
+    rng = np.random.default_rng(B)
+    g = CUT_GRAPHS[name](rng)
+    G = deco.graph_from(g)
+    W = (B + 31) // 32
+    Y = rng.uniform(-1, 1, size=(g.n, (B + 7) // 8 * 8)).astype(np.float32)
+    Z = (Y[:, :B] > 0).astype(np.uint8)
+    ref = O.cut_values(g, Z)
+    cuts = torch.zeros(B, dtype=torch.int64, device=DEV)
+    buf = torch.full((g.n * W + 1,), -1, dtype=torch.int32, device=DEV)
+    for off in (0, 1):
+        zbits = buf[off:off + g.n * W]
+        deco.deco_round_cut(G, B, 1, Y.shape[1], deco.DECO_PREC_FP32, torch.from_numpy(Y).to(DEV), zbits, cuts)
+        np.testing.assert_array_equal(cuts.cpu().numpy(), ref)
+    words = zbits.cpu().numpy().view(np.uint32).reshape(g.n, W)
+    bits = ((words[:, :, None] >> np.arange(32, dtype=np.uint32)) & 1).reshape(g.n, 32 * W)
+    np.testing.assert_array_equal(bits[:, :B], Z)
+    assert not bits[:, B:].any()
+    deco.deco_eval_cuts(G, B, torch.from_numpy(Z * np.uint8(3)).to(DEV), cuts)   # any nonzero byte is 1
+    np.testing.assert_array_equal(cuts.cpu().numpy(), ref)
+
+
+@pytest.mark.parametrize("precision", [deco.DECO_PREC_FP32, deco.DECO_PREC_BF16])
+@pytest.mark.parametrize("lift", [1, 2, 3, 4, 5])
+@pytest.mark.parametrize("pad", [0, 3, 8])
+def test_rounding_by_vectors_equals_rounding_by_columns(lift, pad, precision):
+    # rows whose length is a multiple of 8 are read as vectors, others column by column; what lies past the last
+    # column (here: 7) must not count
+    n, B = 70, 37
+    C = B * lift
+    ld = (C + 7) // 8 * 8 + pad
+    y = torch.full((n, ld), 7.0, device=DEV, dtype=torch.bfloat16 if precision else torch.float32)
+    y[:, :C] = (torch.randint(-2, 3, (n, C), device=DEV, generator=torch.Generator(device=DEV).manual_seed(lift)) / 2).to(y.dtype)
+    zbits = torch.zeros(n * 2, dtype=torch.int32, device=DEV)
+    cuts = torch.zeros(B, dtype=torch.int64, device=DEV)
+    deco.deco_round_cut(deco.graph_from(gg.er_graph(n, 0.1, 3)), B, lift, ld, precision, y, zbits, cuts)
+    s = y[:, :C].float().cpu().numpy().reshape(n, B, lift).sum(2)     # halves: exact in any order
+    Z = s > 0 if lift == 1 else s >= 0
+    words = zbits.cpu().numpy().view(np.uint32).reshape(n, 2)
+    bits = ((words[:, :, None] >> np.arange(32, dtype=np.uint32)) & 1).reshape(n, 64)
+    np.testing.assert_array_equal(bits[:, :B], Z.astype(np.uint32))
+    assert not bits[:, B:].any()
