@@ -151,3 +151,38 @@ def test_budget_solve_stops_on_time_and_resumes():
     # resume from the first call's assignment: never below it
     r2, z2, n2 = deco.deco_solve_budget(G, 128, sched, p, 7, budget_ms=0.0, warm=z0)
     assert r2.best_cut >= r0.best_cut and r2.best_cut == O.cut_value(g, z2)
+
+
+def _hub_graph(n, hubs, deg, seed):
+    rng = np.random.default_rng(seed)
+    u = np.concatenate([np.full(deg, h) for h in range(hubs)] + [rng.integers(hubs, n, 2 * n)])
+    v = np.concatenate([rng.permutation(np.arange(hubs, n))[:deg] for _ in range(hubs)] + [rng.integers(hubs, n, 2 * n)])
+    keep = u != v
+    return gg.from_edges(n, u[keep], v[keep])
+
+
+@pytest.mark.parametrize("n", [2, 31, 32, 33, 40, 65])
+@pytest.mark.parametrize("weights", [False, True])
+def test_greedy_windows_of_vertices(n, weights):
+    # windows of 32 vertices, neighbours loaded 8 vertices ahead, across the ends of windows and orderings
+    g = signed_graph(n, 0.5, n) if weights else gg.er_graph(n, 0.5, n)
+    B = 33
+    z = torch.zeros(n * B, dtype=torch.uint8, device=DEV)
+    cuts = torch.zeros(B, dtype=torch.int64, device=DEV)
+    deco.deco_greedy(deco.graph_from(g), B, 9, z, cuts)
+    Zr, cr = O.greedy_batch(g, B, 9)
+    np.testing.assert_array_equal(z.cpu().numpy().reshape(n, B), Zr)
+    np.testing.assert_array_equal(cuts.cpu().numpy(), cr)
+
+
+@pytest.mark.parametrize("n,deg", [(400, 40), (400, 64), (400, 65), (700, 300), (240000, 70)])
+def test_greedy_long_rows_and_sides_outside_shared_memory(n, deg):
+    # rows of more than 32 and 64 entries; 240 000 sides do not fit in shared memory
+    g = _hub_graph(n, 3, deg, n + deg)
+    B = 2 if n > 1000 else 9
+    z = torch.zeros(n * B, dtype=torch.uint8, device=DEV)
+    cuts = torch.zeros(B, dtype=torch.int64, device=DEV)
+    deco.deco_greedy(deco.graph_from(g), B, 31, z, cuts)
+    Zr, cr = O.greedy_batch(g, B, 31)
+    np.testing.assert_array_equal(z.cpu().numpy().reshape(n, B), Zr)
+    np.testing.assert_array_equal(cuts.cpu().numpy(), cr)
