@@ -225,9 +225,11 @@ int launch_bytes_to_bits(int32_t n, int32_t B, const uint8_t* z, uint32_t* bits,
 int cut_bytes(const deco_graph* g, int32_t B, const uint8_t* z, int64_t* cuts, cudaStream_t st);
 int launch_argmax(int32_t B, const int64_t* cuts, int32_t* best, cudaStream_t st);
 // 1-flip local search on bit-packed columns (n x ceil(B/32) words), in place;
-// gains: n x 32 ceil(B/32) int32 scratch, changed: max_rounds + 1 int32 scratch
-int launch_local_search(const deco_graph* g, int32_t B, uint32_t* zbits, int32_t max_rounds, int32_t* gains,
-                        int32_t* changed, cudaStream_t st);
+// gains: local_search_words words of scratch, changed: max_rounds + 1 int32
+// scratch; kernels (or null) counts the launches
+size_t local_search_words(const deco_graph* g, int32_t B);
+int launch_local_search(const deco_graph* g, int32_t B, uint32_t* zbits, int32_t max_rounds, uint32_t* gains,
+                        int32_t* changed, int64_t* kernels, cudaStream_t st);
 
 // Phase bookkeeping of deco_solve: best of the phase, global best record.
 struct BestRecord {

@@ -16,11 +16,15 @@
 //    pairwise non-adjacent, so the cut grows by the sum of their gains; the
 //    search ends at a 1-flip local optimum or after max_rounds rounds.  A
 //    device flag per round lets the remaining rounds return at once.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "api_util.cuh"
 #include "deco_internal.cuh"
 #include "slab.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace deco {
 
@@ -47,117 +51,155 @@ struct Feistel {
   }
 };
 
-// order[b n + k] = pi_b(k).  A thread walks one item after another, so that a
-// warp is not held by its longest walk: 5 000 x 256 items 133 us, one item per
-// thread 129.
-__global__ void k_orders(Feistel F, int32_t B, int32_t* order) {
-  const int64_t total = (int64_t)F.n * B, step = (int64_t)gridDim.x * blockDim.x;
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= total) return;
-  uint32_t b = (uint32_t)(i / F.n), x = (uint32_t)(i % F.n);
+// order[b n + k] = pi_b(k).  TABLE: the round function of run b takes 2^h
+// values of R in each of the 4 rounds, so the block tabulates them (4 x 2^h
+// Philox calls instead of four per step of every walk) in shared memory.  A
+// thread walks one item after another, so that a warp is not held by its
+// longest walk.  Measured, 5 000 x 256 items: 19 us; Philox in every step 129.
+constexpr int ORDER_MAX_H = 12;   // 4 x 2^12 16-bit words: 32 KB
+
+template <bool TABLE>
+__global__ void __launch_bounds__(256) k_orders(Feistel F, int32_t B, int32_t* order) {
+  extern __shared__ uint16_t tab[];
+  const uint32_t b = blockIdx.x, half = F.mask + 1u;
+  if (TABLE) {
+    for (uint32_t i = threadIdx.x; i < 4u * half; i += blockDim.x)
+      tab[i] = (uint16_t)(philox4x32_10(make_uint4(i & F.mask, b, i >> F.h, STREAM_ORDER), F.k0, F.k1).x & F.mask);
+    __syncthreads();
+  }
+  const uint32_t step = gridDim.y * blockDim.x;
+  uint32_t k = blockIdx.y * blockDim.x + threadIdx.x;
+  if (k >= F.n) return;
+  uint32_t x = k;
   for (;;) {
     // a cycle of the bijection on [0, 4^h) passes through [0, n): every walk ends
-    x = F.net(x, b);
+    if (TABLE) {
+      uint32_t L = x >> F.h, R = x & F.mask;
+#pragma unroll
+      for (uint32_t i = 0; i < 4; ++i) {
+        const uint32_t t = R;
+        R = L ^ tab[i * half + R];
+        L = t;
+      }
+      x = (L << F.h) | R;
+    } else {
+      x = F.net(x, b);
+    }
     if (x >= F.n) continue;
-    order[i] = (int32_t)x;
-    i += step;
-    if (i >= total) return;
-    b = (uint32_t)(i / F.n);
-    x = (uint32_t)(i % F.n);
+    order[(size_t)b * F.n + k] = (int32_t)x;
+    if (F.n - k <= step) return;
+    x = k += step;
   }
 }
 
-// One run (one warp, one block) places its vertices in order.  Bound by the
-// chain of n dependent placements; everything that does not depend on the
-// sides is loaded ahead of it: the orders and row bounds a window of 32
-// vertices ahead (one per lane), the first 64 neighbours GREEDY_AHEAD
-// vertices ahead.  SMEM: the sides (2: not placed) live in shared memory, a
-// byte per vertex, and a placement is a shared load, a warp reduction and a
-// shared store; at the end they go to the run's part of `order`, which it has
-// consumed (4 n bytes of stride).  Else (a graph whose sides do not fit) the
-// sides are column b of z, in global memory.  Measured, n = 5 000, degree 10,
-// 256 runs: 1.07 ms; with the whole chain of loads in each placement 4.28.
-constexpr int GREEDY_AHEAD = 8;
+// One run per block places its vertices in order: warp 0 places, warp 1 loads
+// ahead of it.  Bound by the chain of n dependent placements: a shared load of
+// the neighbours' sides (2: not placed), a warp reduction, a shared store.
+// Warp 1 fills the list of the next GREEDY_WIN vertices (vertex, row, first 64
+// entries) in shared memory while warp 0 works on this one; longer rows are
+// read in place.  SMEM: the sides live in shared memory, a byte per vertex, and
+// go to the run's part of `order` at the end, which it has consumed (4 n bytes of
+// stride); else (a graph whose sides do not fit) they are column b of z.
+// Measured, n = 5 000, degree 10, 256 runs: 0.49 ms; loading ahead from the same
+// warp 1.07, with the whole chain of loads in each placement 4.28.
+constexpr int GREEDY_WIN = 16;
+
+template <bool WT>
+struct GreedyWindow {
+  int4 row[GREEDY_WIN];                                  // vertex, first entry, entries
+  int32_t u[GREEDY_WIN][64];                             // neighbours (-1: none)
+  int32_t w[WT ? GREEDY_WIN : 1][64];
+};
 
 template <bool WT, bool SMEM>
-__global__ void __launch_bounds__(32) k_greedy(int32_t n, int32_t B, const int32_t* __restrict__ row_ptr,
+__global__ void __launch_bounds__(64) k_greedy(int32_t n, int32_t B, const int32_t* __restrict__ row_ptr,
                                                const int32_t* __restrict__ col_idx, const int32_t* __restrict__ wint,
                                                int32_t* order, uint8_t* z) {
   extern __shared__ __align__(16) uint8_t sides[];
-  const int lane = threadIdx.x;
+  __shared__ GreedyWindow<WT> win[2];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int32_t b = blockIdx.x;
   int32_t* const ord = order + (size_t)b * n;
-  if (SMEM) {
-    for (int i = lane; i < (n + 3) / 4; i += 32) reinterpret_cast<uint32_t*>(sides)[i] = 0x02020202u;
-    __syncwarp();
-  }
-  auto side = [&](int32_t u) -> int { return SMEM ? sides[u] : z[(size_t)u * B + b]; };
-  // w of the entry if its vertex is in S-bar (placing v in S cuts it), -w if in S, 0 if not placed
-  auto vote = [&](int32_t u, int32_t w) -> int32_t {
-    const int s = u >= 0 ? side(u) : 2;
-    return s == 0 ? w : s == 1 ? -w : 0;
+  if (SMEM)
+    for (int i = threadIdx.x; i < (n + 3) / 4; i += 64) reinterpret_cast<uint32_t*>(sides)[i] = 0x02020202u;
+  // rows of the window after the next, one per lane (warp 1)
+  int32_t v = -1, e0 = 0, d = 0;
+  auto rows = [&](int32_t k) {
+    v = lane < GREEDY_WIN && k + lane < n ? ord[k + lane] : -1;
+    e0 = v >= 0 ? __ldg(row_ptr + v) : 0;
+    d = v >= 0 ? __ldg(row_ptr + v + 1) - e0 : 0;
   };
-  struct Ahead { int32_t u[2], w[2]; };
-  Ahead q[GREEDY_AHEAD];
-  auto fetch = [&](int32_t e0, int32_t d, Ahead& a) {
+  auto fill = [&](GreedyWindow<WT>& g) {
+    if (lane < GREEDY_WIN) g.row[lane] = make_int4(v, e0, d, 0);
+    int32_t u[GREEDY_WIN][2], w[WT ? GREEDY_WIN : 1][2];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      a.u[h] = -1;
-      a.w[h] = 1;
-      if (32 * h + lane < d) {
-        a.u[h] = __ldg(col_idx + e0 + 32 * h + lane);
-        if (WT) a.w[h] = __ldg(wint + e0 + 32 * h + lane);
-      }
-    }
-  };
-  // window of 32 vertices, one per lane: vertex, first entry, entries (0 past n)
-  int32_t v = lane < n ? ord[lane] : -1, vn = -1;
-  int32_t e0 = v >= 0 ? __ldg(row_ptr + v) : 0, d = v >= 0 ? __ldg(row_ptr + v + 1) - e0 : 0, e0n = 0, dn = 0;
+    for (int j = 0; j < GREEDY_WIN; ++j) {
+      const int32_t ej = __shfl_sync(0xFFFFFFFFu, e0, j), dj = __shfl_sync(0xFFFFFFFFu, d, j);
 #pragma unroll
-  for (int i = 0; i < GREEDY_AHEAD; ++i)
-    fetch(__shfl_sync(0xFFFFFFFFu, e0, i), __shfl_sync(0xFFFFFFFFu, d, i), q[i]);
-  for (int32_t k0 = 0; k0 < n; k0 += 32) {
-    vn = k0 + 32 + lane < n ? ord[k0 + 32 + lane] : -1;
-#pragma unroll 1
-    for (int j0 = 0; j0 < 32; j0 += GREEDY_AHEAD) {
-      if (k0 + j0 >= n) break;
-      if (j0 == GREEDY_AHEAD) {
-        e0n = vn >= 0 ? __ldg(row_ptr + vn) : 0;
-        dn = vn >= 0 ? __ldg(row_ptr + vn + 1) - e0n : 0;
-      }
-#pragma unroll
-      for (int i = 0; i < GREEDY_AHEAD; ++i) {
-        const int j = j0 + i;
-        if (k0 + j < n) {
-          const int32_t vv = __shfl_sync(0xFFFFFFFFu, v, j), dd = __shfl_sync(0xFFFFFFFFu, d, j);
-          int32_t t = vote(q[i].u[0], q[i].w[0]);
-          if (dd > 32) t += vote(q[i].u[1], q[i].w[1]);
-          if (dd > 64) {
-            const int32_t ee = __shfl_sync(0xFFFFFFFFu, e0, j);
-            for (int32_t x = 64 + lane; x < dd; x += 32)
-              t += vote(__ldg(col_idx + ee + x), WT ? __ldg(wint + ee + x) : 1);
-          }
-          // |sum| <= sum of the row's |w| <= 2^24 (checked when the graph is created)
-          const int32_t sum = __reduce_add_sync(0xFFFFFFFFu, t);
-          if (lane == 0) {
-            if (SMEM) sides[vv] = sum >= 0 ? 1 : 0;
-            else z[(size_t)vv * B + b] = sum >= 0 ? 1 : 0;
-          }
-          __syncwarp();   // the next vertices read this side
+      for (int h = 0; h < 2; ++h) {
+        u[j][h] = -1;
+        if (WT) w[WT ? j : 0][h] = 0;
+        if (32 * h + lane < dj) {
+          u[j][h] = __ldg(col_idx + ej + 32 * h + lane);
+          if (WT) w[WT ? j : 0][h] = __ldg(wint + ej + 32 * h + lane);
         }
-        // vertex j + GREEDY_AHEAD: of this window, or of the next
-        const int ja = j + GREEDY_AHEAD;
-        if (ja < 32) fetch(__shfl_sync(0xFFFFFFFFu, e0, ja), __shfl_sync(0xFFFFFFFFu, d, ja), q[i]);
-        else fetch(__shfl_sync(0xFFFFFFFFu, e0n, ja - 32), __shfl_sync(0xFFFFFFFFu, dn, ja - 32), q[i]);
       }
     }
-    v = vn;
-    e0 = e0n;
-    d = dn;
+#pragma unroll
+    for (int j = 0; j < GREEDY_WIN; ++j)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        g.u[j][32 * h + lane] = u[j][h];
+        if (WT) g.w[WT ? j : 0][32 * h + lane] = w[WT ? j : 0][h];
+      }
+  };
+  if (warp == 1) {
+    rows(0);
+    fill(win[0]);
+    rows(GREEDY_WIN);
+  }
+  __syncthreads();
+  for (int32_t k0 = 0, s = 0; k0 < n; k0 += GREEDY_WIN, s ^= 1) {
+    if (warp == 1) {
+      fill(win[s ^ 1]);
+      rows(k0 + 2 * GREEDY_WIN);
+    } else {
+      const GreedyWindow<WT>& g = win[s];
+      const int cnt = min(GREEDY_WIN, n - k0);
+      auto vote = [&](int32_t u, int32_t w) -> int32_t {
+        // w if the neighbour is in S-bar (placing v in S cuts the edge), -w if in S, 0 if not placed
+        const int x = u >= 0 ? (SMEM ? sides[u] : z[(size_t)u * B + b]) : 2;
+        return x == 0 ? w : x == 1 ? -w : 0;
+      };
+      int4 r = g.row[0];
+      int32_t u0 = g.u[0][lane], w0 = WT ? g.w[0][lane] : 1;
+      for (int j = 0; j < cnt; ++j) {
+        const int4 cur = r;
+        const int32_t u = u0, w = w0;
+        const int jn = j + 1 < cnt ? j + 1 : j;
+        int32_t t = vote(u, w);
+        r = g.row[jn];                                    // the next vertex's list, meanwhile
+        u0 = g.u[jn][lane];
+        if (WT) w0 = g.w[WT ? jn : 0][lane];
+        if (cur.z > 32) {
+          t += vote(g.u[j][32 + lane], WT ? g.w[WT ? j : 0][32 + lane] : 1);
+          for (int32_t x = 64 + lane; x < cur.z; x += 32)
+            t += vote(__ldg(col_idx + cur.y + x), WT ? __ldg(wint + cur.y + x) : 1);
+        }
+        // |sum| <= sum of the row's |w| <= 2^24 (checked when the graph is created)
+        const int32_t sum = __reduce_add_sync(0xFFFFFFFFu, t);
+        if (lane == 0) {
+          if (SMEM) sides[cur.x] = sum >= 0 ? 1 : 0;
+          else z[(size_t)cur.x * B + b] = sum >= 0 ? 1 : 0;
+        }
+        __syncwarp();   // the next vertices read this side
+      }
+    }
+    __syncthreads();
   }
   if (SMEM) {
     uint8_t* out = reinterpret_cast<uint8_t*>(ord);
-    for (int i = lane; i < n; i += 32) out[i] = sides[i];
+    for (int i = threadIdx.x; i < n; i += 64) out[i] = sides[i];
   }
 }
 
@@ -244,26 +286,332 @@ __global__ void k_ls_flip(int32_t n, int32_t W, int32_t B, const int32_t* row_pt
   }
 }
 
+// ---- unit and +-1 weights: gains as bit planes.  A word's 32 columns are
+// worked on together: the neighbours on the side that a flip would lose are
+// counted by ripple-carry adders over bit planes (plane p holds bit p of every
+// column's count), positive gains are kept as NP planes, and two nodes' gains
+// compare in two operations a plane.  A thread owns a (row, word).
+template <int NP>
+__device__ __forceinline__ void planes_load(const uint32_t* p, uint32_t* g) {
+#pragma unroll
+  for (int h = 0; h < NP / 4; ++h) {
+    const uint4 q = __ldcg(reinterpret_cast<const uint4*>(p) + h);
+    g[4 * h] = q.x; g[4 * h + 1] = q.y; g[4 * h + 2] = q.z; g[4 * h + 3] = q.w;
+  }
+}
+
+template <int NP>
+__device__ __forceinline__ void planes_store(uint32_t* p, const uint32_t* g) {
+#pragma unroll
+  for (int h = 0; h < NP / 4; ++h)
+    __stcg(reinterpret_cast<uint4*>(p) + h, make_uint4(g[4 * h], g[4 * h + 1], g[4 * h + 2], g[4 * h + 3]));
+}
+
+// counts: add 1 to the columns of x
+template <int NP>
+__device__ __forceinline__ void ls_count(uint32_t* c, uint32_t x) {
+#pragma unroll
+  for (int p = 0; p < NP; ++p) {
+    const uint32_t t = c[p] & x;
+    c[p] ^= x;
+    x = t;
+  }
+}
+
+// g = d - 2 c where that is positive (columns `cols`), else 0; returns the columns with a positive gain
+template <int NP>
+__device__ __forceinline__ uint32_t ls_gain(const uint32_t* c, int32_t d, uint32_t cols, uint32_t* g) {
+  uint32_t borrow = 0u, any = 0u;
+#pragma unroll
+  for (int p = 0; p <= NP; ++p) {
+    const uint32_t a = p < NP && ((d >> p) & 1) ? 0xFFFFFFFFu : 0u, b = p ? c[p > 0 ? p - 1 : 0] : 0u;
+    if (p < NP) g[p < NP ? p : 0] = a ^ b ^ borrow;
+    borrow = (~a & (b | borrow)) | (b & borrow);
+  }
+#pragma unroll
+  for (int p = 0; p < NP; ++p) {
+    g[p] &= ~borrow & cols;
+    any |= g[p];
+  }
+  return any;
+}
+
+// columns where gu > g, or gu == g and `lower` (the other node has the lower index)
+template <int NP>
+__device__ __forceinline__ uint32_t ls_beats(const uint32_t* gu, const uint32_t* g, bool lower) {
+  uint32_t beats = lower ? 0xFFFFFFFFu : 0u;
+#pragma unroll
+  for (int p = 0; p < NP; ++p) beats = (gu[p] & ~g[p]) | (~(gu[p] ^ g[p]) & beats);
+  return beats;
+}
+
+// col: index, or index | sign bit of a +-1 graph.  zk: the word column, row u at zk[u W].
+template <int NP>
+__device__ __forceinline__ void ls_gain_row(int32_t v, int32_t W, const int32_t* __restrict__ row_ptr,
+                                            const uint32_t* __restrict__ col, const uint32_t* zk, uint32_t cols,
+                                            uint32_t* gains) {
+  const int32_t e0 = __ldg(row_ptr + v), e1 = __ldg(row_ptr + v + 1);
+  const uint32_t zv = zk[(size_t)v * W];
+  uint32_t c[NP], g[NP];
+#pragma unroll
+  for (int p = 0; p < NP; ++p) c[p] = 0u;
+  for (int32_t e = e0; e < e1; e += 8) {
+    uint32_t u[8], x[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) u[q] = __ldg(col + min(e + q, e1 - 1));
+#pragma unroll
+    for (int q = 0; q < 8; ++q) x[q] = zk[(size_t)(u[q] & 0x7FFFFFFFu) * W];
+    // columns where the entry is lost to a flip: the other side of a +1, the same side of a -1
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      ls_count<NP>(c, e + q < e1 ? x[q] ^ zv ^ ((u[q] & 0x80000000u) ? 0xFFFFFFFFu : 0u) : 0u);
+  }
+  ls_gain<NP>(c, e1 - e0, cols, g);
+  planes_store<NP>(gains + (size_t)v * NP, g);
+}
+
+// flips row v's columns whose positive gain no neighbour beats; true if any
+template <int NP>
+__device__ __forceinline__ bool ls_flip_row(int32_t v, int32_t W, const int32_t* __restrict__ row_ptr,
+                                            const uint32_t* __restrict__ col, const uint32_t* gains, uint32_t* zk) {
+  uint32_t g[NP], left = 0u;
+  planes_load<NP>(gains + (size_t)v * NP, g);
+#pragma unroll
+  for (int p = 0; p < NP; ++p) left |= g[p];
+  if (!left) return false;
+  const int32_t e1 = __ldg(row_ptr + v + 1);
+  for (int32_t e = __ldg(row_ptr + v); e < e1 && left; e += 4) {
+    uint32_t gu[4][NP];
+    int32_t u[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) u[q] = (int32_t)(__ldg(col + min(e + q, e1 - 1)) & 0x7FFFFFFFu);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) planes_load<NP>(gains + (size_t)u[q] * NP, gu[q]);
+    // a repeated last entry changes nothing
+#pragma unroll
+    for (int q = 0; q < 4; ++q) left &= ~ls_beats<NP>(gu[q], g, u[q] < v);
+  }
+  if (!left) return false;
+  zk[(size_t)v * W] ^= left;
+  return true;
+}
+
+__device__ __forceinline__ uint32_t word_columns(int32_t B, int32_t k) {
+  return B - 32 * k >= 32 ? 0xFFFFFFFFu : (1u << (B - 32 * k)) - 1u;
+}
+
+// All rounds of one word in one cluster of LS_CLUSTER CTAs (columns are
+// independent of one another), so the word stops at its own optimum.  CTA i
+// owns a range of rows, holds their entries in shared memory (16-bit index |
+// sign) and a copy of the word's column of z and of its positive-gain masks,
+// which the owners of the rows update in all CTAs through distributed shared
+// memory; a cluster barrier ends each half round.  Only gains of neighbours
+// that have a positive gain in a column still open are read (L2).  Bound by
+// the latency of the half rounds.  Measured, n = 5 000, degree 10, 256 columns,
+// rounded vectors: 94 us; with z and all gains read through L2 275, a launch
+// per half round of 32 integer gains a word 780.
+constexpr int LS_CLUSTER = 8;
+
+struct LsSmem {
+  size_t z, pos, rp, ent, total;   // byte offsets
+};
+__host__ __device__ inline LsSmem ls_smem(int32_t n, int32_t entries) {
+  LsSmem L;
+  const int32_t own = (n + LS_CLUSTER - 1) / LS_CLUSTER;
+  L.z = 0;
+  L.pos = L.z + (size_t)n * 4;
+  L.rp = L.pos + (size_t)n * 4;
+  L.ent = L.rp + (size_t)(own + 1) * 4;
+  L.total = L.ent + ((size_t)entries * 2 + 15) / 16 * 16;
+  return L;
+}
+
+template <int NP>
+__global__ void __cluster_dims__(LS_CLUSTER, 1, 1) __launch_bounds__(1024)
+    k_ls_cluster(int32_t n, int32_t W, int32_t B, const int32_t* __restrict__ row_ptr,
+                 const uint32_t* __restrict__ col, uint32_t* zb, uint32_t* gains, int32_t max_rounds,
+                 int32_t* changed, int32_t max_entries) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ int32_t s_any[2][LS_CLUSTER];
+  cg::cluster_group cluster = cg::this_cluster();
+  const LsSmem L = ls_smem(n, max_entries);
+  uint32_t* const z = reinterpret_cast<uint32_t*>(smem + L.z);
+  uint32_t* const pos = reinterpret_cast<uint32_t*>(smem + L.pos);
+  int32_t* const rp = reinterpret_cast<int32_t*>(smem + L.rp);
+  uint16_t* const ent = reinterpret_cast<uint16_t*>(smem + L.ent);
+  const int rank = (int)cluster.block_rank(), tid = threadIdx.x, nt = blockDim.x;
+  const int32_t k = blockIdx.x / LS_CLUSTER, own = (n + LS_CLUSTER - 1) / LS_CLUSTER;
+  const int32_t ra = min(n, rank * own), rows = min(n, ra + own) - ra;
+  uint32_t* const gk = gains + (size_t)k * n * NP;
+  const uint32_t cols = word_columns(B, k);
+  const int32_t ebase = __ldg(row_ptr + ra);
+  for (int32_t i = tid; i <= rows; i += nt) rp[i] = __ldg(row_ptr + ra + i) - ebase;
+  const int32_t entries = __ldg(row_ptr + ra + rows) - ebase;
+  for (int32_t i = tid; i < entries; i += nt) {
+    const uint32_t c = __ldg(col + ebase + i);
+    ent[i] = (uint16_t)((c & 0x7FFFu) | (c >> 31 << 15));
+  }
+  for (int32_t v = tid; v < n; v += nt) z[v] = zb[(size_t)v * W + k];
+  // the same word of every CTA of the cluster
+  auto put = [&](uint32_t* at, uint32_t x) {
+#pragma unroll
+    for (int q = 0; q < LS_CLUSTER; ++q) *cluster.map_shared_rank(at, q) = x;
+  };
+  cluster.sync();
+  for (int32_t r = 0; r < max_rounds; ++r) {
+    for (int32_t i = tid; i < rows; i += nt) {
+      const int32_t e0 = rp[i], d = rp[i + 1] - e0;
+      const uint32_t zv = z[ra + i];
+      uint32_t c[NP], g[NP];
+#pragma unroll
+      for (int p = 0; p < NP; ++p) c[p] = 0u;
+#pragma unroll 4
+      for (int32_t e = 0; e < d; ++e) {
+        const uint32_t u = ent[e0 + e];
+        ls_count<NP>(c, z[u & 0x7FFFu] ^ zv ^ ((u & 0x8000u) ? 0xFFFFFFFFu : 0u));
+      }
+      const uint32_t any = ls_gain<NP>(c, d, cols, g);
+      put(pos + ra + i, any);
+      if (any) planes_store<NP>(gk + (size_t)(ra + i) * NP, g);
+    }
+    cluster.sync();
+    bool flipped = false;
+    for (int32_t i = tid; i < rows; i += nt) {
+      const int32_t v = ra + i;
+      uint32_t left = pos[v];
+      if (!left) continue;
+      uint32_t g[NP];
+      planes_load<NP>(gk + (size_t)v * NP, g);
+      const int32_t e1 = rp[i + 1];
+      for (int32_t e = rp[i]; e < e1 && left; e += 4) {
+        uint32_t gu[4][NP];
+        int32_t u[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          u[q] = ent[min(e + q, e1 - 1)] & 0x7FFF;
+          if (pos[u[q]] & left) {
+            planes_load<NP>(gk + (size_t)u[q] * NP, gu[q]);
+          } else {
+            u[q] = n;   // no open column to compare: a gain of 0, and not the lower index
+#pragma unroll
+            for (int p = 0; p < NP; ++p) gu[q][p] = 0u;
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) left &= ~ls_beats<NP>(gu[q], g, u[q] < v);
+      }
+      if (!left) continue;
+      flipped = true;
+      put(z + v, z[v] ^ left);
+    }
+    const int block_any = __syncthreads_or(flipped ? 1 : 0);
+    if (tid < LS_CLUSTER) *cluster.map_shared_rank(&s_any[r & 1][rank], tid) = block_any;
+    cluster.sync();
+    int32_t sum = 0;
+#pragma unroll
+    for (int i = 0; i < LS_CLUSTER; ++i) sum |= s_any[r & 1][i];
+    if (!sum) break;   // the same in every CTA of the cluster
+    if (rank == 0 && tid == 0) changed[r + 1] = 1;
+  }
+  for (int32_t i = tid; i < rows; i += nt) zb[(size_t)(ra + i) * W + k] = z[ra + i];
+}
+
+// one half round of all words per launch (graphs with more rows than a cluster covers well)
+template <int NP>
+__global__ void __launch_bounds__(128) k_ls_gain_planes(int32_t n, int32_t W, int32_t B,
+                                                        const int32_t* __restrict__ row_ptr,
+                                                        const uint32_t* __restrict__ col, const uint32_t* zb,
+                                                        uint32_t* gains, const int32_t* run) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (int64_t)n * W || !*run) return;
+  const int32_t v = (int32_t)(i % n), k = (int32_t)(i / n);
+  ls_gain_row<NP>(v, W, row_ptr, col, zb + k, word_columns(B, k), gains + (size_t)k * n * NP);
+}
+template <int NP>
+__global__ void __launch_bounds__(128) k_ls_flip_planes(int32_t n, int32_t W, const int32_t* __restrict__ row_ptr,
+                                                        const uint32_t* __restrict__ col, const uint32_t* gains,
+                                                        uint32_t* zb, const int32_t* run, int32_t* next) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (int64_t)n * W || !*run) return;
+  const int32_t v = (int32_t)(i % n), k = (int32_t)(i / n);
+  if (ls_flip_row<NP>(v, W, row_ptr, col, gains + (size_t)k * n * NP, zb + k)) *next = 1;
+}
+
 unsigned blocks_for(int64_t threads, int per) { return (unsigned)((threads + per - 1) / per); }
 
 }  // namespace
 
+// Bit planes of a positive gain (at most the row's degree), 0: the weights or
+// the degrees do not allow them and the gains are kept as integers.
+static int ls_planes(const deco_graph* g) {
+  if (g->wmode == W_GENERAL) return 0;
+  if (g->max_deg < 16) return 4;
+  if (g->max_deg < 256) return 8;
+  return g->max_deg < 65536 ? 16 : 0;
+}
+
+size_t local_search_words(const deco_graph* g, int32_t B) {
+  const int np = ls_planes(g);
+  return (size_t)g->n * ((B + 31) / 32) * (np ? np : 32);
+}
+
+template <int NP>
+static int run_planes(const deco_graph* g, int32_t B, uint32_t* zbits, int32_t max_rounds, uint32_t* gains,
+                      int32_t* changed, int64_t* kernels, cudaStream_t st) {
+  const int32_t W = (B + 31) / 32, n = g->n;
+  const uint32_t* col = g->wmode == W_SIGN ? g->col_sw : reinterpret_cast<const uint32_t*>(g->col_idx);
+  // one cluster per word while its rows fit on chip (n of about 20 000 at
+  // degree 10; the launches of the other form alone cost 2 x 2.2 us a round)
+  int32_t entries = 0;
+  const int32_t own = (n + LS_CLUSTER - 1) / LS_CLUSTER;
+  for (int q = 0; q < LS_CLUSTER; ++q)
+    entries = std::max(entries, g->h_row_ptr[std::min(n, (q + 1) * own)] - g->h_row_ptr[std::min(n, q * own)]);
+  const size_t smem = ls_smem(n, entries).total;
+  if (n <= 32768 && smem + 1024 <= (size_t)slab_max_smem()) {
+    const int nt = own <= 256 ? 256 : own <= 512 ? 512 : 1024;
+    DECO_CUDA_TRY(cudaFuncSetAttribute(k_ls_cluster<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_ls_cluster<NP><<<(unsigned)W * LS_CLUSTER, nt, smem, st>>>(n, W, B, g->row_ptr, col, zbits, gains, max_rounds,
+                                                                 changed, entries);
+    DECO_CUDA_TRY(cudaGetLastError());
+    if (kernels) *kernels += 1;
+    return DECO_OK;
+  }
+  const int64_t threads = (int64_t)n * W;
+  for (int32_t r = 0; r < max_rounds; ++r) {
+    k_ls_gain_planes<NP><<<blocks_for(threads, 128), 128, 0, st>>>(n, W, B, g->row_ptr, col, zbits, gains, changed + r);
+    k_ls_flip_planes<NP><<<blocks_for(threads, 128), 128, 0, st>>>(n, W, g->row_ptr, col, gains, zbits, changed + r,
+                                                                   changed + r + 1);
+  }
+  DECO_CUDA_TRY(cudaGetLastError());
+  if (kernels) *kernels += 2 * (int64_t)max_rounds;
+  return DECO_OK;
+}
+
 // The rounds of the local search on bit-packed columns (stream-ordered).
-// gains: n x 32W int32 scratch; changed: max_rounds + 1 int32 scratch.
-int launch_local_search(const deco_graph* g, int32_t B, uint32_t* zbits, int32_t max_rounds, int32_t* gains,
-                        int32_t* changed, cudaStream_t st) {
+// gains: local_search_words(g, B) words of scratch; changed: max_rounds + 1
+// int32 scratch, changed[r] nonzero where round r flipped (r >= 1).
+int launch_local_search(const deco_graph* g, int32_t B, uint32_t* zbits, int32_t max_rounds, uint32_t* gains,
+                        int32_t* changed, int64_t* kernels, cudaStream_t st) {
   const int32_t W = (B + 31) / 32;
   if (max_rounds <= 0 || g->n == 0) return DECO_OK;
   DECO_CUDA_TRY(cudaMemsetAsync(changed, 0, sizeof(int32_t) * (size_t)(max_rounds + 1), st));
   DECO_CUDA_TRY(cudaMemsetAsync(changed, 1, sizeof(int32_t), st));   // round 0 runs (any nonzero word)
+  switch (ls_planes(g)) {
+    case 4: return run_planes<4>(g, B, zbits, max_rounds, gains, changed, kernels, st);
+    case 8: return run_planes<8>(g, B, zbits, max_rounds, gains, changed, kernels, st);
+    case 16: return run_planes<16>(g, B, zbits, max_rounds, gains, changed, kernels, st);
+    default: break;
+  }
   const int64_t threads = (int64_t)g->n * W;
+  int32_t* gi = reinterpret_cast<int32_t*>(gains);
   for (int32_t r = 0; r < max_rounds; ++r) {
-    k_ls_gain<<<blocks_for(threads, 128), 128, 0, st>>>(g->n, W, g->row_ptr, g->col_idx, g->wint, zbits, gains,
+    k_ls_gain<<<blocks_for(threads, 128), 128, 0, st>>>(g->n, W, g->row_ptr, g->col_idx, g->wint, zbits, gi,
                                                         changed + r);
-    k_ls_flip<<<blocks_for(threads, 128), 128, 0, st>>>(g->n, W, B, g->row_ptr, g->col_idx, gains, zbits,
-                                                        changed + r, changed + r + 1);
+    k_ls_flip<<<blocks_for(threads, 128), 128, 0, st>>>(g->n, W, B, g->row_ptr, g->col_idx, gi, zbits, changed + r,
+                                                        changed + r + 1);
   }
   DECO_CUDA_TRY(cudaGetLastError());
+  if (kernels) *kernels += 2 * (int64_t)max_rounds;
   return DECO_OK;
 }
 
@@ -291,21 +639,18 @@ extern "C" int deco_greedy(const deco_graph* g, int32_t B, uint64_t seed, uint8_
   const int32_t n = g->n, W = (B + 31) / 32;
   uint32_t* bits = nullptr;
   if ((rc = s.alloc(&bits, sizeof(uint32_t) * (size_t)n * W))) return rc;
-  const int64_t items = (int64_t)n * B;
-  k_orders<<<(unsigned)std::min<int64_t>((items + 255) / 256, (int64_t)device_sm_count() * 8), 256, 0, st>>>(F, B,
-                                                                                                            order);
+  const dim3 ogrid((unsigned)B, (unsigned)std::min((n + 1023) / 1024, device_sm_count()));
+  if (F.h <= ORDER_MAX_H) k_orders<true><<<ogrid, 256, sizeof(uint16_t) * (4u << F.h), st>>>(F, B, order);
+  else k_orders<false><<<ogrid, 256, 0, st>>>(F, B, order);
   DECO_CUDA_TRY(cudaGetLastError());
   const size_t smem = ((size_t)n + 15) / 16 * 16;
-  const bool fits = smem <= (size_t)slab_max_smem();
+  // the sides, beside the two windows of loaded rows
+  const bool fits = smem + sizeof(GreedyWindow<true>) * 2 <= (size_t)slab_max_smem();
   auto fn = g->wint ? (fits ? k_greedy<true, true> : k_greedy<true, false>)
                     : (fits ? k_greedy<false, true> : k_greedy<false, false>);
-  if (fits) {
-    if (smem > 48 * 1024)
-      DECO_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  } else {
-    DECO_CUDA_TRY(cudaMemsetAsync(z, 2, (size_t)n * B, st));
-  }
-  fn<<<(unsigned)B, 32, fits ? smem : 0, st>>>(n, B, g->row_ptr, g->col_idx, g->wint, order, z);
+  if (fits) DECO_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  else DECO_CUDA_TRY(cudaMemsetAsync(z, 2, (size_t)n * B, st));
+  fn<<<(unsigned)B, 64, fits ? smem : 0, st>>>(n, B, g->row_ptr, g->col_idx, g->wint, order, z);
   DECO_CUDA_TRY(cudaGetLastError());
   if (fits) {
     const int64_t tiles = (int64_t)((n + 31) / 32) * W;
@@ -328,15 +673,15 @@ extern "C" int deco_local_search(const deco_graph* g, int32_t B, uint8_t* z, int
   const int32_t W = (B + 31) / 32;
   Scratch s(st);
   uint32_t* bits = nullptr;
-  int32_t* gains = nullptr;
+  uint32_t* gains = nullptr;
   int32_t* changed = nullptr;
   if ((rc = s.alloc(&bits, sizeof(uint32_t) * (size_t)g->n * W)) ||
-      (rc = s.alloc(&gains, sizeof(int32_t) * (size_t)g->n * 32 * W)) ||
+      (rc = s.alloc(&gains, sizeof(uint32_t) * local_search_words(g, B))) ||
       (rc = s.alloc(&changed, sizeof(int32_t) * (size_t)(max_rounds + 1))))
     return rc;
   if (g->n > 0) {
     if ((rc = launch_bytes_to_bits(g->n, B, z, bits, st))) return rc;
-    if ((rc = launch_local_search(g, B, bits, max_rounds, gains, changed, st))) return rc;
+    if ((rc = launch_local_search(g, B, bits, max_rounds, gains, changed, nullptr, st))) return rc;
     k_bits_to_bytes<<<blocks_for((int64_t)g->n * B, 256), 256, 0, st>>>(g->n, B, W, bits, z);
     DECO_CUDA_TRY(cudaGetLastError());
   }

@@ -113,10 +113,10 @@ extern "C" int deco_solve(const deco_graph* g, int32_t B, const deco_phase* phas
     if ((rc = s.alloc(&pbz, (size_t)n)) || (rc = s.alloc(&bz, (size_t)n))) return rc;
     if ((rc = s.alloc(&h, sizeof(float) * n)) || (rc = s.alloc(&side, (size_t)n))) return rc;
     if ((rc = s.alloc(&flag, sizeof(int32_t)))) return rc;
-    int32_t* ls_gains = nullptr;
+    uint32_t* ls_gains = nullptr;
     int32_t* ls_changed = nullptr;
     if (p->local_search > 0) {
-      if ((rc = s.alloc(&ls_gains, sizeof(int32_t) * (size_t)n * 32 * W)) ||
+      if ((rc = s.alloc(&ls_gains, sizeof(uint32_t) * local_search_words(g, B))) ||
           (rc = s.alloc(&ls_changed, sizeof(int32_t) * ((size_t)p->local_search + 1))))
         return rc;
     }
@@ -205,8 +205,7 @@ extern "C" int deco_solve(const deco_graph* g, int32_t B, const deco_phase* phas
         if (e) return e;
         if (p->local_search > 0) {
           // 1-flip polish of the rounded vectors (off by default)
-          if ((e = launch_local_search(g, B, zbits, p->local_search, ls_gains, ls_changed, st))) return e;
-          kernels += 2 * (int64_t)p->local_search;
+          if ((e = launch_local_search(g, B, zbits, p->local_search, ls_gains, ls_changed, &kernels, st))) return e;
         }
         if ((e = launch_cut_bits(g, B, zbits, cut_out, st))) return e;
         if ((e = launch_phase_finish(g, B, k, first_eval, cut_out, zbits, idx, rec, phase_best, bz, st))) return e;

@@ -186,3 +186,34 @@ def test_greedy_long_rows_and_sides_outside_shared_memory(n, deg):
     Zr, cr = O.greedy_batch(g, B, 31)
     np.testing.assert_array_equal(z.cpu().numpy().reshape(n, B), Zr)
     np.testing.assert_array_equal(cuts.cpu().numpy(), cr)
+
+
+SEARCH_GRAPHS = {
+    "degree 15 (4 planes)": lambda: gg.er_graph(16, 1.0, 0),
+    "degree 16 (8 planes)": lambda: gg.er_graph(17, 1.0, 0),
+    "degree 300 (16 planes)": lambda: _hub_graph(600, 2, 300, 1),
+    "signed": lambda: signed_graph(900, 0.02, 3, (-1.0, 1.0)),
+    "signed hubs": lambda: _sign(_hub_graph(500, 2, 280, 2)),
+    "several rows per thread": lambda: gg.er_graph_avg_degree(20000, 6.0, 4),
+    "a launch per half round": lambda: gg.er_graph_avg_degree(33000, 5.0, 5),
+    "launches, signed": lambda: _sign(gg.er_graph_avg_degree(33000, 5.0, 6)),
+}
+
+
+def _sign(g):
+    u, v, _ = g.edges()
+    return gg.from_edges(g.n, u, v, np.random.default_rng(g.n).choice([-1.0, 1.0], size=u.size))
+
+
+@pytest.mark.parametrize("name", list(SEARCH_GRAPHS))
+@pytest.mark.parametrize("B,rounds", [(1, 2), (32, 100), (45, 100)])
+def test_local_search_bit_planes_match_oracle(name, B, rounds):
+    g = SEARCH_GRAPHS[name]()
+    Z = (np.random.default_rng(B).random((g.n, B)) < 0.5).astype(np.uint8)
+    z = torch.from_numpy(Z.reshape(-1).copy()).to(DEV)
+    cuts = torch.zeros(B, dtype=torch.int64, device=DEV)
+    r = deco.deco_local_search(deco.graph_from(g), B, z, rounds, cuts)
+    Zr, rr = O.local_search(g, Z, rounds)
+    np.testing.assert_array_equal(z.cpu().numpy().reshape(g.n, B), Zr)
+    np.testing.assert_array_equal(cuts.cpu().numpy(), O.cut_values(g, Zr))
+    assert r == rr
