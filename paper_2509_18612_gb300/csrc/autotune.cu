@@ -66,6 +66,7 @@ extern "C" int deco_autotune(const deco_graph* g, int32_t C, int32_t precision, 
         cands.push_back(DECO_KERNEL_GLOBAL | (s << 16) | DECO_KERNEL_PIPELINED | DECO_KERNEL_PIPE_ENTRIES(e) |
                         DECO_KERNEL_PIPE_STAGES(1) | DECO_KERNEL_PIPE_MIXED_ADD | DECO_KERNEL_PIPE_WIDE);
   }
+  cands.push_back(DECO_KERNEL_ONCHIP);   // the planner's own on-chip form (the row-vector form where it is estimated faster)
   for (int k = 1; k <= 8; k *= 2)
     for (int t = 1; t <= 2; ++t)
       for (int x = 1; x <= 2; ++x) {
@@ -77,7 +78,7 @@ extern "C" int deco_autotune(const deco_graph* g, int32_t C, int32_t precision, 
   for (int k = 1; k <= 8; k *= 2) cands.push_back(DECO_KERNEL_ONCHIP | (k << 8) | (2 << 12) | (2 << 14) | DECO_KERNEL_LEAN);
   // every on-chip shape also in the row-pair form (a half-warp per row)
   for (size_t i = 0, n0 = cands.size(); i < n0; ++i)
-    if ((cands[i] & 0x3) == DECO_KERNEL_ONCHIP) cands.push_back(cands[i] | DECO_KERNEL_ROW_PAIRS);
+    if ((cands[i] & 0x3) == DECO_KERNEL_ONCHIP && cands[i] != DECO_KERNEL_ONCHIP) cands.push_back(cands[i] | DECO_KERNEL_ROW_PAIRS);
   // dense tensor-core kernel: BF16 blocks of graphs with at least n^2 / 64 entries
   if (precision == DECO_PREC_BF16 && (double)g->nnz * 64.0 >= (double)g->n * (double)g->n)
     for (int k = 1; k <= 8; k *= 2) cands.push_back(DECO_KERNEL_DENSE | (k << 8));

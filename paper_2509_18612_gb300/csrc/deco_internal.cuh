@@ -104,6 +104,27 @@ struct StreamShape {
   int fe = 0;          // entries per item fixed at compile time (8 or 12, two stages), or 0
 };
 
+namespace deco {
+// On-chip image of one graph for `lpr` lanes (16-byte vectors) per row.  The
+// rows are sorted by entries (ties: +1 entries of a +-1 graph, then index) and
+// cut into slices of 32 / lpr; position p of the order is row p of the
+// shared-memory replica, position n a row of zeros.
+//   table  nslices x {first list chunk, + entries, - entries, first weight}:
+//          the largest counts among the slice's rows
+//   lists  chunks of 8 entries: for every row of the slice 8 16-bit vector
+//          offsets (lpr x position) into the replica; the + chunks, then the
+//          - chunks; entries past a row's own count name the zero row
+//   wts    8 floats per row and chunk (general integral weights only)
+struct RowsImage {
+  int lpr = 0;
+  int32_t n = 0, nslices = 0;
+  int32_t list16 = 0, wts16 = 0;   // 16-byte units of the lists / the weights
+  uint32_t* data = nullptr;        // device: table, lists, weights, then order (n int32)
+  int32_t longest = 0;             // entries of the longest slice
+  int64_t padded = 0;              // entries of all slices, padding included
+};
+}  // namespace deco
+
 // The opaque handle of the ABI.
 struct deco_graph {
   int32_t n = 0;
@@ -121,6 +142,8 @@ struct deco_graph {
   std::vector<SlabImage> images;    // on-chip CSR images, one per cluster size used
   std::deque<StreamImage> streams;  // record streams of the pipelined step kernel, one per launch shape
                                     // (a deque: phase plans keep pointers to them while others are added)
+  std::deque<deco::RowsImage> rows;         // images of the row-vector on-chip form, one per slab width used
+  std::vector<deco::RowsImage> rows_sizes;  // their sizes for every slab width (planning), nothing on the device
   __nv_bfloat16* dense = nullptr;   // dense BF16 copy of A for the tensor-core kernel (built on first use)
   int32_t dense_ld = 0;             // its row stride, round_up(n, 128)
   struct Tuning {

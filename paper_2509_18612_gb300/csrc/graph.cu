@@ -47,6 +47,7 @@ static void free_graph(deco_graph* g) {
   if (!g) return;
   for (auto& im : g->images) cudaFree(im.data);
   for (auto& im : g->streams) free_stream_image(im);
+  for (auto& im : g->rows) cudaFree(im.data);
   cudaFree(g->dense);
   cudaFree(g->row_ptr);
   cudaFree(g->col_idx);

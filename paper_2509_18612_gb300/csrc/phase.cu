@@ -61,6 +61,34 @@ static double onchip_cost(int64_t own_nnz, int32_t own, int32_t n, int k, int wa
   return per_cta * waves;
 }
 
+// Estimates in SM cycles of one step, for the choice between the on-chip
+// forms.  k_slab: gathers, and for a cluster the exchange of the whole replica
+// and its barriers.  Fitted to the measured steps of five graphs of 700 - 1000
+// rows and degree 4 - 48 (FP32 k = 8: 5 500 - 12 500 cycles, k = 4: 7 200 -
+// 18 900; BF16 k = 8: 6 800 - 15 600), within 10 %.
+static double slab_cycles(int64_t own_nnz, int32_t own, int32_t n, int k, int waves, int prec) {
+  const bool bf = prec == DECO_PREC_BF16;
+  if (k == 1) return waves * ((bf ? 2.0 : 1.5) * (double)own_nnz + 20.0 * own);
+  const double gather = k == 8 ? (bf ? 2.0 : 1.6) : (bf ? 1.7 : 1.35);
+  return waves * (gather * (double)own_nnz + 3.0 * n + (k == 8 ? 2500.0 : 3600.0) + (bf ? 1100.0 : 0.0));
+}
+// k_rows: several CTAs may share an SM; they then share its shared-memory pipe
+static double rows_step_cycles(const RowsImage& im, int prec, int items, int max_smem) {
+  double pipe = 0.0;
+  const double alone = rows_cycles(im, &pipe);
+  const size_t smem = rows_smem_bytes(im, prec, true, true);
+  const int threads = rows_threads(im.n, im.lpr);
+  const int per_sm = std::max(1, std::min((int)((max_smem + 2048) / (smem + 1024)), 1024 / threads));
+  const int sms = device_sm_count();
+  const int waves = (items + sms * per_sm - 1) / (sms * per_sm);
+  const int share = std::min(per_sm, (items + sms - 1) / sms);
+  return waves * std::max(alone, share * pipe + 350.0);
+}
+// one launch of the per-step kernel: the launch, and its gathers at ~4.5 TB/s
+static double step_cycles(const deco_graph* g, int32_t C, int prec) {
+  return 5500.0 + (double)g->nnz * C * (prec == DECO_PREC_BF16 ? 2.0 : 4.0) / 4.5e12 * 2.07e9;
+}
+
 bool valid_selector(int kernel) {
   const int kind = kernel & 0x3, k = (kernel >> 8) & 0xF, t = (kernel >> 12) & 0x3, x = (kernel >> 14) & 0x3;
   const int s = (kernel >> 16) & 0x7;
@@ -177,6 +205,8 @@ int plan_phase(const deco_graph* g, int32_t C, int32_t ld, int prec, int force, 
   // the row-pair form is also the cost model's choice (measured faster on
   // every on-chip shape of the benchmark); the autotuner times both forms
   const bool want_pairs = ((force >> 21) & 1) != 0 || (force & 0x3) == DECO_KERNEL_AUTO;
+  // without modifiers the on-chip form is the planner's choice too
+  const bool any_form = force == DECO_KERNEL_AUTO || force == DECO_KERNEL_ONCHIP;
   force &= 0x3;
   if (force == DECO_KERNEL_DENSE) {
     // BF16 blocks only; an FP32 block (e.g. the FP32 polish) is planned as AUTO
@@ -215,7 +245,7 @@ int plan_phase(const deco_graph* g, int32_t C, int32_t ld, int prec, int force, 
   const int max_smem = slab_max_smem();
   const int items = (C + cols - 1) / cols;
   const int sms = device_sm_count();
-  double best = 0.0;
+  double best = 0.0, slab_best = 0.0;
   // the replica alone must fit before any split is worth sizing
   const bool replica_fits = (size_t)g->n * 128 + 4096 <= (size_t)max_smem;
   for (int k = 1; k <= SLAB_MAX_CLUSTER && aligned && replica_fits; k *= 2) {
@@ -230,7 +260,9 @@ int plan_phase(const deco_graph* g, int32_t C, int32_t ld, int prec, int force, 
     const size_t smem = slab_smem_bytes(g->n, max_own, (int)max_words, prec, want_lean);
     if (smem > (size_t)max_smem) continue;
     const int per_sm = std::max(1, std::min(4, (int)((size_t)(max_smem + 1024) / (smem + 1024))));
-    const int waves = (int)((items * (int64_t)k + (int64_t)sms * per_sm - 1) / ((int64_t)sms * per_sm));
+    // clusters are placed within a GPC: 16 clusters of 8 take two waves although 128 SMs would hold them
+    const int64_t held = std::max(1, std::min(slab_resident_clusters(k), sms / k)) * (int64_t)per_sm;
+    const int waves = (int)((items + held - 1) / held);
     const double cost = onchip_cost(max_edges, max_own, g->n, k, waves);
     if (plan->kernel != KERNEL_ONCHIP || cost < best) {
       best = cost;
@@ -239,12 +271,32 @@ int plan_phase(const deco_graph* g, int32_t C, int32_t ld, int prec, int force, 
       plan->max_own = max_own;
       plan->max_img_words = (int32_t)max_words;
       plan->items = items;
+      slab_best = slab_cycles(max_edges, max_own, g->n, k, waves, prec);
     }
   }
   if (force == DECO_KERNEL_ONCHIP && plan->kernel != KERNEL_ONCHIP) {
     set_error("the on-chip kernel does not fit this graph (n=%d, nnz=%lld, ld=%d)", g->n,
               (long long)g->nnz, ld);
     return DECO_ERR_UNSUPPORTED;
+  }
+  if (any_form && aligned && (size_t)(g->n + 1) * 32 <= (size_t)max_smem) {
+    // the row-vector form, where its estimate is the lowest over its slab widths
+    double least = plan->kernel == KERNEL_ONCHIP ? slab_best : step_cycles(g, C, prec);
+    std::lock_guard<std::mutex> lock(g_image_mutex);
+    auto& sizes = const_cast<deco_graph*>(g)->rows_sizes;
+    if (sizes.empty())
+      rows_measure(g->h_row_ptr.data(), g->h_w.empty() ? nullptr : g->h_w.data(), g->wmode, 0, g->n, &sizes);
+    for (const RowsImage& im : sizes) {
+      if (rows_smem_bytes(im, prec, true, true) > (size_t)max_smem) continue;
+      const int w = im.lpr * (prec == DECO_PREC_BF16 ? 8 : 4);
+      const double t = rows_step_cycles(im, prec, (C + w - 1) / w, max_smem);
+      if (t < least) {
+        least = t;
+        plan->kernel = KERNEL_ROWS;
+        plan->rows_lpr = im.lpr;
+        plan->items = (C + w - 1) / w;
+      }
+    }
   }
   return DECO_OK;
 }
@@ -291,6 +343,10 @@ int PhaseRunner::prepare(const deco_graph* g_, int32_t C_, int32_t ld_, int prec
     std::lock_guard<std::mutex> lock(g_image_mutex);
     // the record streams live with the graph, like the on-chip CSR images
     return stream_image(const_cast<deco_graph*>(g), plan.stream, &plan.rec);
+  }
+  if (plan.kernel == KERNEL_ROWS) {
+    std::lock_guard<std::mutex> lock(g_image_mutex);
+    return rows_image(const_cast<deco_graph*>(g), plan.rows_lpr, &plan.rows);
   }
   if (plan.kernel != KERNEL_ONCHIP) return DECO_OK;
   {
@@ -347,6 +403,34 @@ int PhaseRunner::run(void* y[2], int& cur, float* v, int32_t steps, int objectiv
     p.max_img_words = plan.image.max_words;
     p.flag = flag;
     int rc = launch_slab(p, plan.items, prec, g->wmode, st);
+    if (rc) return rc;
+    if (kernels) *kernels += 1;
+    return DECO_OK;
+  }
+  if (plan.kernel == KERNEL_ROWS) {
+    RowsParams p{};
+    p.g0 = rows_graph(*plan.rows);
+    p.g0.ld = ld;
+    p.g0.C = C;
+    p.g0.dnet = g->dnet;
+    p.g0.y = y[cur];
+    p.g0.v = v;
+    p.g0.alpha_cols = alpha_cols;
+    p.g0.steps_cols = steps_cols;
+    p.lpr = plan.rows_lpr;
+    p.threads = rows_threads(g->n, plan.rows_lpr);
+    const bool lap = objective == DECO_OBJ_LAPLACIAN, momv = mu != 0.0f;
+    p.smem = (uint32_t)rows_smem_bytes(*plan.rows, prec, lap, momv);
+    p.steps = steps;
+    const float fac = objective == DECO_OBJ_MULTILINEAR01 ? 2.0f : 1.0f;
+    p.alpha = fac * alpha;
+    p.afac = fac;
+    p.mu = mu;
+    p.objective = objective;
+    p.load_v = load_v ? 1 : 0;
+    p.store_v = store_v ? 1 : 0;
+    p.flag = flag;
+    const int rc = launch_rows(p, plan.items, prec, g->wmode, st);
     if (rc) return rc;
     if (kernels) *kernels += 1;
     return DECO_OK;

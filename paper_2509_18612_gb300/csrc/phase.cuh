@@ -4,11 +4,12 @@
 
 #include "deco_internal.cuh"
 #include "dense_tc.cuh"
+#include "rows.cuh"
 #include "slab.cuh"
 
 namespace deco {
 
-enum KernelKind { KERNEL_GLOBAL = 0, KERNEL_ONCHIP = 1, KERNEL_DENSE = 2 };
+enum KernelKind { KERNEL_GLOBAL = 0, KERNEL_ONCHIP = 1, KERNEL_DENSE = 2, KERNEL_ROWS = 3 };
 
 struct PhasePlan {
   int kernel = KERNEL_GLOBAL;
@@ -25,6 +26,8 @@ struct PhasePlan {
   int items = 0;                 // column slabs
   int32_t max_own = 0, max_img_words = 0;
   SlabImage image;               // on-chip CSR image (owned by the graph)
+  int rows_lpr = 0;              // row-vector on-chip kernel: vectors of a slab row
+  const RowsImage* rows = nullptr;   // its image (owned by the graph)
   int ks = 1;                    // dense kernel: contraction split over a cluster (per-step launches)
   int32_t kpad = 0, cpad = 0;    // dense kernel: padded n and C
   bool dpersist = false;         // dense kernel: one persistent launch per phase

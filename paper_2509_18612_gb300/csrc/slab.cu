@@ -27,6 +27,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 #include <vector>
 
@@ -558,6 +559,34 @@ int slab_max_smem() {
     v = 227 * 1024;
   }
   return v - 1024;   // room for the kernel's static shared memory (mbarrier)
+}
+
+int slab_resident_clusters(int k) {
+  static std::atomic<int> held[SLAB_MAX_CLUSTER + 1];   // every thread finds the same value
+  if (k < 1 || k > SLAB_MAX_CLUSTER) return 1;
+  if (held[k] == 0) {
+    auto fn = k_slab<DECO_PREC_FP32, W_UNIT, 1024, false, true>;
+    const size_t smem = (size_t)slab_max_smem();
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(k * 64), 1, 1);
+    cfg.blockDim = dim3(1024, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)k;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess || n < 1) {
+      cudaGetLastError();
+      n = std::max(1, 152 / k);
+    }
+    held[k] = n;
+  }
+  return held[k];
 }
 
 // Row split of one graph into k parts by cost(r) = row_ptr[r] + 2 r.

@@ -54,6 +54,8 @@ struct SlabParams {
 
 size_t slab_smem_bytes(int max_n, int max_own, int max_img_words, int prec, bool lean = false);
 int slab_max_smem();
+// clusters of k CTAs that the GPU holds at once with one CTA per SM
+int slab_resident_clusters(int k);
 // one thread waits, with k_slab's bounded exchange wait, on an mbarrier that
 // never completes; sets bit 1 of *flag when the wait gives up
 int launch_wait_probe_slab(int32_t* flag, cudaStream_t st);

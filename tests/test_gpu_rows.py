@@ -1,0 +1,87 @@
+"""The row-vector form of the on-chip kernel (the planner's choice for graphs
+with short rows or few starts) against the per-step kernel: the same FP32
+operations in the same order, so the blocks are bit-identical.
+
+The planner takes slab widths of 1, 2, 4 or 8 vectors by the number of
+columns: on a graph of 100 rows 64, 1 024, 3 000 and 9 000 columns take one
+width each; more columns than the GPU holds at once run in several waves."""
+import numpy as np
+import pytest
+
+import graphgen as gg
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():
+    pytest.skip("needs a GPU", allow_module_level=True)
+
+import paper_2509_18612_gb300 as deco  # noqa: E402
+
+DEV = torch.device("cuda:0")
+
+
+def _weighted(g, choices, seed):
+    u, v, _ = g.edges()
+    return gg.from_edges(g.n, u, v, np.random.default_rng(seed).choice(np.array(choices), size=u.size))
+
+
+GRAPHS = {
+    "one": lambda: gg.from_edges(1, [], []),
+    "31": lambda: gg.er_graph(31, 0.3, 1),
+    "33": lambda: gg.er_graph(33, 0.9, 2),                       # rows of 24 ... 32 entries: whole chunks of 8
+    "er100": lambda: gg.er_graph(100, 0.1, 0),
+    "isolated": lambda: gg.from_edges(90, [0, 1, 2, 5], [1, 2, 3, 9]),
+    "hubs": lambda: gg.ba_graph(1025, 4, 7),                     # one slice more than 32 warps hold, long rows
+    "torus": lambda: gg.torus_graph(40, 20, 3),                  # +-1: both lists, 0 ... 4 entries
+    "sign": lambda: _weighted(gg.er_graph(257, 0.05, 3), [-1.0, 1.0], 1),
+    "weights": lambda: _weighted(gg.ba_graph(300, 4, 5), [-3.0, 2.0, 7.0], 2),
+    "long": lambda: gg.er_graph_avg_degree(2300, 5.0, 4),        # beyond the 128-byte slabs: AUTO only
+}
+
+
+@pytest.mark.parametrize("name", list(GRAPHS))
+@pytest.mark.parametrize("precision", [deco.DECO_PREC_FP32, deco.DECO_PREC_BF16])
+@pytest.mark.parametrize("objective,mu", [(0, 0.0), (0, 0.9), (1, 0.9), (1, 0.0)])
+@pytest.mark.parametrize("C", [1, 37, 64, 200, 1024, 3000, 9000])
+def test_row_vector_form_bitwise_equals_per_step_kernel(name, precision, objective, mu, C):
+    g = GRAPHS[name]()
+    if C > 1024 and g.n > 300:
+        pytest.skip("the widths are covered by the small graphs")
+    G = deco.graph_from(g)
+    ld = (C + 63) // 64 * 64
+    gen = torch.Generator(device=DEV).manual_seed(C)
+    y0 = (torch.rand(g.n, ld, device=DEV, generator=gen) * 2 - 1) * 0.3
+    y0 = y0.bfloat16() if precision else y0
+    v0 = torch.randn(g.n, ld, device=DEV, generator=gen) * 0.1 if mu else None
+    alpha = torch.rand(C, device=DEV, generator=gen) * 0.02
+    budget = torch.randint(0, 8, (C,), device=DEV, generator=gen, dtype=torch.int32)
+    for cols in (False, True):
+        args = deco.step_args(objective, precision, 0.01, mu, alpha_cols=alpha if cols else None,
+                              steps_cols=budget if cols else None)
+        out = []
+        for kernel in (deco.DECO_KERNEL_GLOBAL, deco.DECO_KERNEL_AUTO, deco.DECO_KERNEL_ONCHIP):
+            if kernel == deco.DECO_KERNEL_ONCHIP and g.n > 1700:
+                continue
+            y, v = y0.clone(), None if v0 is None else v0.clone()
+            for steps in (0, 3, 4):      # both replicas; state carried from call to call
+                deco.deco_run_phase(G, C, ld, y, v, steps, args, kernel=kernel)
+            out.append((y, v))
+        for y, v in out[1:]:
+            assert torch.equal(y, out[0][0])
+            assert mu == 0.0 or torch.equal(v, out[0][1])
+
+
+def test_row_vector_form_flags_nonfinite_and_keeps_limits():
+    g = GRAPHS["er100"]()
+    G = deco.graph_from(g)
+    y = torch.zeros(100, 64, device=DEV)
+    y[5, 3] = float("inf")
+    flag = torch.zeros(1, dtype=torch.int32, device=DEV)
+    deco.deco_run_phase(G, 64, 64, y, None, 1, deco.step_args(), flag=flag)
+    assert flag.item() & 1
+    # a graph beyond the 128-byte slabs is refused where the on-chip kernel is demanded, as ever
+    big = deco.graph_from(GRAPHS["long"]())
+    with pytest.raises(deco.DecoError):
+        deco.deco_run_phase(big, 64, 64, torch.zeros(2300, 64, device=DEV), None, 1, deco.step_args(),
+                            kernel=deco.DECO_KERNEL_ONCHIP)
