@@ -19,7 +19,9 @@
 #include <algorithm>
 #include <climits>
 #include <cmath>
+#include <deque>
 #include <memory>
+#include <mutex>
 #include <vector>
 
 #include "api_util.cuh"
@@ -27,6 +29,14 @@
 #include "phase.cuh"
 
 using namespace deco;
+
+// The members' images of the row-vector on-chip kernel for one slab width,
+// built once and kept with the batch.
+struct BatchRows {
+  int lpr = 0;
+  std::vector<RowsImage> images;      // data: inside `data`
+  uint32_t* data = nullptr;           // device, all members
+};
 
 struct deco_batch {
   deco_graph* U = nullptr;            // union graph
@@ -38,6 +48,9 @@ struct deco_batch {
   int32_t* gmax = nullptr;            // device, maximum degree per graph
   double* gmean = nullptr;            // device, mean degree per graph
   int32_t* gsize = nullptr;           // device, nodes per graph
+  mutable std::mutex rows_mutex;
+  mutable std::deque<BatchRows> rows;                        // one per slab width used
+  mutable std::vector<std::vector<RowsImage>> rows_sizes;    // per member: sizes for every slab width (planning)
 };
 
 namespace deco {
@@ -217,11 +230,15 @@ __global__ void k_fill_ll(int32_t n, long long v, long long* p) {
 }
 
 // One on-chip launch over a batch: item = (graph, column slab), one CTA per
-// item, every member graph's replica and CSR image on chip.  Where the
-// largest member's staging area and momentum do not fit as well, the lean
-// form keeps the momentum in global memory and refreshes the replica from L2.
+// item, every member graph's replica and image on chip: in the row-vector
+// form (k_rows, lpr > 0) or with 128-byte slabs (k_slab).  Where the largest
+// member's staging area and momentum do not fit k_slab as well, its lean form
+// keeps the momentum in global memory and refreshes the replica from L2.
 struct BatchSlab {
   bool ok = false;
+  int lpr = 0, threads = 0;          // row-vector form: vectors of a slab row, CTA size
+  uint32_t smem = 0;
+  RowsGraph* d_rows = nullptr;
   bool lean = false;
   std::vector<SlabImage> images;
   SlabGraph* d_graphs = nullptr;
@@ -231,6 +248,8 @@ struct BatchSlab {
   void release() {
     for (auto& im : images) cudaFree(im.data);
     images.clear();
+    if (d_rows) cudaFree(d_rows);
+    d_rows = nullptr;
     if (d_graphs) cudaFree(d_graphs);
     if (d_items) cudaFree(d_items);
     if (xbuf) cudaFree(xbuf);
@@ -241,9 +260,153 @@ struct BatchSlab {
   }
 };
 
-// ok stays false (nothing allocated) when a member does not fit on chip
-int batch_slab_prepare(const deco_batch* b, int32_t C, int32_t ld, int prec, void* y, float* v, bool mom_needed,
+// members in decreasing order of their work (stored entries plus rows): CTAs
+// start in item order, so the last wave holds the small graphs
+std::vector<int2> batch_items(const deco_batch* b, int32_t C, int32_t cols) {
+  const deco_graph* U = b->U;
+  std::vector<int32_t> order((size_t)b->n_graphs);
+  for (int32_t i = 0; i < b->n_graphs; ++i) order[(size_t)i] = i;
+  auto work = [&](int32_t i) {
+    const int32_t r0 = b->h_goff[i], r1 = b->h_goff[i + 1];
+    return (int64_t)(U->h_row_ptr[r1] - U->h_row_ptr[r0]) + 8LL * (r1 - r0);
+  };
+  std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t c) { return work(a) > work(c); });
+  std::vector<int2> items;
+  for (int32_t i : order)
+    for (int32_t c = 0; c < C; c += cols) items.push_back(make_int2(i, c));
+  return items;
+}
+
+// The slab width of the row-vector form for a batch of graphs that k_slab
+// holds one per CTA, or 0 where k_slab is estimated to be faster: with many
+// more items than SMs the time is the items' cycles per step over the SMs
+// (several CTAs share an SM where they fit), at least the slowest item's.
+// 48 BA graphs of 200 - 1 200 rows, 256 starts, momentum: k_slab 40.3 ms
+// a solve, rows of 1 / 2 / 4 vectors 25.8 / 22.3 / 20.1 (FP32).
+int batch_rows_shape(const deco_batch* b, int32_t C, int prec, bool lap, BatchSlab* bs) {
+  const deco_graph* U = b->U;
+  const float* w = U->h_w.empty() ? nullptr : U->h_w.data();
+  std::lock_guard<std::mutex> lock(b->rows_mutex);
+  if (b->rows_sizes.empty()) {
+    std::vector<std::vector<RowsImage>> sizes((size_t)b->n_graphs);
+    host_parallel(b->n_graphs, 8 * (int64_t)U->nnz, [&](int, int64_t i0, int64_t i1) {
+      for (int64_t i = i0; i < i1; ++i)
+        rows_measure(U->h_row_ptr.data(), w, U->wmode, b->h_goff[i], b->h_goff[i + 1] - b->h_goff[i], &sizes[(size_t)i]);
+    });
+    b->rows_sizes.swap(sizes);
+  }
+  const int sms = device_sm_count(), max_smem = slab_max_smem();
+  const int vn = prec == DECO_PREC_BF16 ? 8 : 4, resident = rows_max_threads(prec, true);
+  double least = 0.0, longest = 0.0;
+  const int64_t slabs = (C + 8 * vn - 1) / (8 * vn);
+  for (int32_t i = 0; i < b->n_graphs; ++i) {
+    const int32_t r0 = b->h_goff[i], r1 = b->h_goff[i + 1];
+    const double t = slab_cycles(U->h_row_ptr[r1] - U->h_row_ptr[r0], r1 - r0, r1 - r0, 1, 1, prec);
+    least += t * (double)slabs / sms;
+    longest = std::max(longest, t);
+  }
+  least = std::max(least, longest);
+  for (size_t l = 0; l < b->rows_sizes[0].size(); ++l) {
+    size_t smem = 0;
+    int32_t max_n = 0;
+    for (const auto& sizes : b->rows_sizes) {
+      smem = std::max(smem, rows_smem_bytes(sizes[l], prec, lap, false));
+      max_n = std::max(max_n, sizes[l].n);
+    }
+    if (smem > (size_t)max_smem) continue;
+    const int lpr = b->rows_sizes[0][l].lpr;
+    const int per_sm = std::max(1, std::min(4, (int)((max_smem + 2048) / (smem + 1024))));
+    const int64_t items = (C + lpr * vn - 1) / (lpr * vn);
+    double sum = 0.0, last = 0.0;
+    for (const auto& sizes : b->rows_sizes) {
+      double pipe = 0.0;
+      const double alone = rows_cycles(sizes[l], &pipe);
+      sum += std::max(pipe, alone / per_sm) * (double)items / sms;
+      last = std::max(last, alone);
+    }
+    const double t = std::max(sum, last);
+    if (t < least) {
+      least = t;
+      bs->lpr = lpr;
+      bs->threads = std::min(resident / per_sm / 32 * 32, rows_threads(max_n, lpr));
+      bs->smem = (uint32_t)smem;
+    }
+  }
+  return bs->lpr;
+}
+
+// images of every member for slab width lpr, built once
+int batch_rows_images(const deco_batch* b, int lpr, const BatchRows** out) {
+  const deco_graph* U = b->U;
+  const float* w = U->h_w.empty() ? nullptr : U->h_w.data();
+  std::lock_guard<std::mutex> lock(b->rows_mutex);
+  for (const auto& br : b->rows)
+    if (br.lpr == lpr) { *out = &br; return DECO_OK; }
+  BatchRows br;
+  br.lpr = lpr;
+  br.images.resize((size_t)b->n_graphs);
+  std::vector<std::vector<uint32_t>> words((size_t)b->n_graphs);
+  host_parallel(b->n_graphs, 8 * (int64_t)U->nnz, [&](int, int64_t i0, int64_t i1) {
+    for (int64_t i = i0; i < i1; ++i)
+      rows_build(U->h_row_ptr.data(), U->h_col.data(), w, U->wmode, b->h_goff[i], b->h_goff[i + 1] - b->h_goff[i], lpr,
+                 &br.images[(size_t)i], &words[(size_t)i]);
+  });
+  std::vector<uint32_t> all;
+  std::vector<size_t> at;
+  for (const auto& x : words) {
+    at.push_back(all.size());
+    all.insert(all.end(), x.begin(), x.end());
+    all.resize((all.size() + 3) / 4 * 4);   // images start on 16-byte boundaries
+  }
+  cudaError_t e = cudaMalloc((void**)&br.data, all.size() * 4);
+  if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(batch row images)");
+  e = cudaMemcpy(br.data, all.data(), all.size() * 4, cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) {
+    cudaFree(br.data);
+    return cuda_fail(e, "cudaMemcpy(batch row images)");
+  }
+  for (size_t i = 0; i < at.size(); ++i) br.images[i].data = br.data + at[i];
+  b->rows.push_back(std::move(br));
+  *out = &b->rows.back();
+  return DECO_OK;
+}
+
+int batch_rows_prepare(const deco_batch* b, int32_t C, int32_t ld, int prec, void* y, float* v,
                        const float* alpha_cols, const int32_t* steps_cols, BatchSlab* bs) {
+  const BatchRows* br = nullptr;
+  int rc = batch_rows_images(b, bs->lpr, &br);
+  if (rc) return rc;
+  std::vector<RowsGraph> hg;
+  for (int32_t i = 0; i < b->n_graphs; ++i) {
+    const size_t row0 = (size_t)b->h_goff[i];
+    RowsGraph rg = rows_graph(br->images[(size_t)i]);
+    rg.ld = ld;
+    rg.C = C;
+    rg.dnet = b->U->dnet + row0;
+    rg.y = static_cast<unsigned char*>(y) + row0 * ld * elem_size(prec);
+    rg.v = v ? v + row0 * ld : nullptr;
+    rg.alpha_cols = alpha_cols;
+    rg.steps_cols = steps_cols;
+    hg.push_back(rg);
+  }
+  const std::vector<int2> items = batch_items(b, C, bs->lpr * (prec == DECO_PREC_BF16 ? 8 : 4));
+  cudaError_t e = cudaMalloc((void**)&bs->d_rows, sizeof(RowsGraph) * hg.size());
+  if (e == cudaSuccess) e = cudaMalloc((void**)&bs->d_items, sizeof(int2) * items.size());
+  if (e == cudaSuccess) e = cudaMemcpy(bs->d_rows, hg.data(), sizeof(RowsGraph) * hg.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(bs->d_items, items.data(), sizeof(int2) * items.size(), cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) {
+    bs->release();
+    return cuda_fail(e, "batch on-chip parameters");
+  }
+  bs->n_items = (int32_t)items.size();
+  bs->ok = true;
+  return DECO_OK;
+}
+
+// ok stays false (nothing allocated) when a member does not fit on chip;
+// any_form: the row-vector form may be taken instead of k_slab
+int batch_slab_prepare(const deco_batch* b, int32_t C, int32_t ld, int prec, void* y, float* v, bool mom_needed,
+                       bool lap, bool any_form, const float* alpha_cols, const int32_t* steps_cols, BatchSlab* bs) {
   const deco_graph* U = b->U;
   const int cols = prec == DECO_PREC_BF16 ? 64 : 32;
   if (ld % cols) return DECO_OK;
@@ -251,9 +414,22 @@ int batch_slab_prepare(const deco_batch* b, int32_t C, int32_t ld, int prec, voi
   int32_t max_n = 0;
   for (int32_t i = 0; i < b->n_graphs; ++i) max_n = std::max(max_n, b->h_goff[i + 1] - b->h_goff[i]);
   if ((size_t)max_n * 128 + 4096 > (size_t)max_smem) return DECO_OK;
+  // what k_slab would take: where it does not fit, the per-step kernels run
+  int64_t max_words = 0;
+  for (int32_t i = 0; i < b->n_graphs; ++i) {
+    int32_t own = 0;
+    int64_t words = 0, edges = 0;
+    image_sizes(U, 1, &b->h_goff[i], &own, &words, &edges);
+    max_words = std::max(max_words, words);
+  }
+  if (max_words > (1 << 26)) return DECO_OK;
+  const bool staged = slab_smem_bytes(max_n, max_n, (int)max_words, prec) <= (size_t)max_smem;
+  if (!staged && (slab_smem_bytes(max_n, max_n, (int)max_words, prec, true) > (size_t)max_smem || (mom_needed && !v)))
+    return DECO_OK;
+  if (any_form && batch_rows_shape(b, C, prec, lap, bs))
+    return batch_rows_prepare(b, C, ld, prec, y, v, alpha_cols, steps_cols, bs);
   std::vector<SlabGraph> hg((size_t)b->n_graphs);
   const int32_t slabs = (C + cols - 1) / cols;
-  std::vector<int2> items;
   const size_t esz = elem_size(prec);
   for (int32_t i = 0; i < b->n_graphs; ++i) {
     const int32_t row0 = b->h_goff[i], n = b->h_goff[i + 1] - row0;
@@ -279,24 +455,10 @@ int batch_slab_prepare(const deco_batch* b, int32_t C, int32_t ld, int prec, voi
     sg.alpha_cols = alpha_cols;
     sg.steps_cols = steps_cols;
   }
-  // items in decreasing order of their graph's work (stored entries plus
-  // rows): CTAs start in item order, so the last wave holds the small graphs
-  std::vector<int32_t> order((size_t)b->n_graphs);
-  for (int32_t i = 0; i < b->n_graphs; ++i) order[(size_t)i] = i;
-  auto work = [&](int32_t i) {
-    const int32_t r0 = b->h_goff[i], r1 = b->h_goff[i + 1];
-    return (int64_t)(U->h_row_ptr[r1] - U->h_row_ptr[r0]) + 8LL * (r1 - r0);
-  };
-  std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t c) { return work(a) > work(c); });
-  for (int32_t i : order)
-    for (int32_t sl = 0; sl < slabs; ++sl) items.push_back(make_int2(i, sl * cols));
+  const std::vector<int2> items = batch_items(b, C, cols);
   bs->max_n = max_n;
   cudaError_t e = cudaSuccess;
-  if (slab_smem_bytes(max_n, bs->max_own, bs->max_words, prec) > (size_t)max_smem) {
-    if (slab_smem_bytes(max_n, bs->max_own, bs->max_words, prec, true) > (size_t)max_smem || (mom_needed && !v)) {
-      bs->release();
-      return DECO_OK;
-    }
+  if (!staged) {
     bs->lean = true;
     e = cudaMalloc((void**)&bs->xbuf, (size_t)2 * slabs * U->n * 128);
     if (e != cudaSuccess) {
@@ -556,7 +718,9 @@ extern "C" int deco_solve_batch(const deco_batch* b, int32_t B, const deco_param
       const int kind = p->kernel & 0x3;
       if ((kind == DECO_KERNEL_AUTO || kind == DECO_KERNEL_ONCHIP) &&
           (rc = batch_slab_prepare(b, B * pop->lifts[i], ld, p->precision, ybuf[0],
-                                   pop->momentum != 0.0f ? vbuf : nullptr, pop->momentum != 0.0f, alpha_cols,
+                                   pop->momentum != 0.0f ? vbuf : nullptr, pop->momentum != 0.0f,
+                                   p->objective == DECO_OBJ_LAPLACIAN,
+                                   p->kernel == DECO_KERNEL_AUTO || p->kernel == DECO_KERNEL_ONCHIP, alpha_cols,
                                    steps_cols, &lanes.back()->S)))
         return rc;
     }
@@ -633,15 +797,30 @@ extern "C" int deco_solve_batch(const deco_batch* b, int32_t B, const deco_param
         }
         if ((e2 = launch_init(il, st))) return e2;
         *kc += 3;
-        if (vbuf) {
+        Lane* L = nullptr;
+        for (auto& x : lanes) if (x->lift == lift) L = x.get();
+        if (vbuf && !(L->S.ok && L->S.lpr)) {   // the row-vector form starts and keeps its momentum on chip
           ce = cudaMemsetAsync(vbuf, 0, block_elems * sizeof(float), st);
           if (ce != cudaSuccess) return cuda_fail(ce, "memset momentum");
         }
-        Lane* L = nullptr;
-        for (auto& x : lanes) if (x->lift == lift) L = x.get();
         const bool mom = vbuf != nullptr;
         int cur = 0;
-        if (L->S.ok) {
+        if (L->S.ok && L->S.lpr) {
+          RowsParams rp{};
+          rp.graphs = L->S.d_rows;
+          rp.items = L->S.d_items;
+          rp.lpr = L->S.lpr;
+          rp.threads = L->S.threads;
+          rp.smem = L->S.smem;
+          rp.steps = pop->t_hi;
+          rp.steps_dev = d_tmax + r;
+          rp.afac = p->objective == DECO_OBJ_MULTILINEAR01 ? 2.0f : 1.0f;
+          rp.mu = pop->momentum;
+          rp.objective = p->objective;
+          rp.flag = flag;
+          if ((e2 = launch_rows(rp, L->S.n_items, p->precision, U->wmode, st))) return e2;
+          *kc += 1;
+        } else if (L->S.ok) {
           // every graph's slabs in one on-chip launch, in place in ybuf[0]
           SlabParams sp{};
           sp.graphs = L->S.d_graphs;

@@ -26,9 +26,8 @@ int device_sm_count() {
   return sms;
 }
 
-// Exact sizes of the on-chip CSR image of a split (see slab.cuh).
-static void image_sizes(const deco_graph* g, int k, const int32_t* split, int32_t* max_own,
-                        int64_t* max_words, int64_t* max_edges) {
+void image_sizes(const deco_graph* g, int k, const int32_t* split, int32_t* max_own, int64_t* max_words,
+                 int64_t* max_edges) {
   *max_own = 0;
   *max_words = 0;
   *max_edges = 0;
@@ -66,7 +65,7 @@ static double onchip_cost(int64_t own_nnz, int32_t own, int32_t n, int k, int wa
 // and its barriers.  Fitted to the measured steps of five graphs of 700 - 1000
 // rows and degree 4 - 48 (FP32 k = 8: 5 500 - 12 500 cycles, k = 4: 7 200 -
 // 18 900; BF16 k = 8: 6 800 - 15 600), within 10 %.
-static double slab_cycles(int64_t own_nnz, int32_t own, int32_t n, int k, int waves, int prec) {
+double slab_cycles(int64_t own_nnz, int32_t own, int32_t n, int k, int waves, int prec) {
   const bool bf = prec == DECO_PREC_BF16;
   if (k == 1) return waves * ((bf ? 2.0 : 1.5) * (double)own_nnz + 20.0 * own);
   const double gather = k == 8 ? (bf ? 2.0 : 1.6) : (bf ? 1.7 : 1.35);

@@ -35,6 +35,11 @@ struct PhasePlan {
 };
 
 int device_sm_count();
+// exact sizes of the on-chip CSR image of a row split (slab.cuh): the largest part's rows, 32-bit words and entries
+void image_sizes(const deco_graph* g, int k, const int32_t* split, int32_t* max_own, int64_t* max_words,
+                 int64_t* max_edges);
+// estimated SM cycles of one step of k_slab (phase.cu)
+double slab_cycles(int64_t own_nnz, int32_t own, int32_t n, int k, int waves, int prec);
 // a well-formed DECO_KERNEL_* selector (kind and the modifiers it accepts)
 bool valid_selector(int kernel);
 // recorded launch shape for (C, prec) on g, or -1

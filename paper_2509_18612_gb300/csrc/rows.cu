@@ -132,9 +132,15 @@ __device__ __forceinline__ void gather_rows(float* acc, uint32_t rep, uint32_t l
 }
 
 // PERCOL: step sizes and budgets per column (else one step size, every column below C active)
-template <int PREC, int WMODE, bool PERCOL, int LPR, int NT>
+// BATCH: the form of a batch's launch.  Its momentum stays in global memory (this launch's scratch, in L2), which
+// leaves room for a second CTA on the SM or for wider slabs, and its warps take the next slice from a counter, longest
+// first: scale-free graphs have hubs whose slices cost ten times the others'.  48 BA graphs of 200 - 1 200 rows, 256
+// starts, FP32, two rounds: k_slab 40.3 ms; slabs of 2 vectors, momentum in shared memory, slices by turns 28.4; here
+// 20.1 with 4 vectors (2: 22.3; slices by turns 21.5).  One graph's phase keeps turns (torus 0.61 ms, 0.70 by counter).
+template <int PREC, int WMODE, bool PERCOL, int LPR, bool BATCH, int NT>
 __global__ void __launch_bounds__(NT) k_rows(const __grid_constant__ RowsParams P) {
   extern __shared__ __align__(128) unsigned char smem[];
+  __shared__ int s_next[2];                              // BATCH: next slice of an even / odd step
   constexpr int VN = PREC == DECO_PREC_BF16 ? 8 : 4;     // columns of a vector
   constexpr size_t ESZ = PREC == DECO_PREC_BF16 ? 2 : 4;
   constexpr int SR = 32 / LPR;                           // rows of a slice
@@ -154,7 +160,9 @@ __global__ void __launch_bounds__(NT) k_rows(const __grid_constant__ RowsParams 
   const uint32_t img16 = (uint32_t)G.nslices + (uint32_t)G.list16 + (uint32_t)G.wts16;
   unsigned char* const img = smem + 2 * (size_t)rep_bytes;
   float* const dn = reinterpret_cast<float*>(img + 16 * (size_t)img16);
-  float* const vsm = reinterpret_cast<float*>(img + 16 * (size_t)img16 + (lap ? up16((size_t)n * 4) : 0));
+  // momentum by position: in shared memory, or (BATCH) this slab's part of G.v, n x (LPR x VN) floats from G.v + col0 n
+  float* const vsm = BATCH ? G.v + (size_t)col0 * n
+                             : reinterpret_cast<float*>(img + 16 * (size_t)img16 + (lap ? up16((size_t)n * 4) : 0));
   for (uint32_t i = tid; i < img16; i += nt) reinterpret_cast<uint4*>(img)[i] = __ldg(G.image + i);
   const int c0 = col0 + sub * VN;                        // this lane's first column
   const bool in = c0 < ld;                               // ld % 8 == 0: a vector lies inside a row or past it
@@ -170,11 +178,12 @@ __global__ void __launch_bounds__(NT) k_rows(const __grid_constant__ RowsParams 
 #pragma unroll
       for (int h = 0; h < VN; h += 4) {
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (P.load_v && in) v = *reinterpret_cast<const float4*>(G.v + (size_t)r * ld + c0 + h);
+        if (!BATCH && P.load_v && in) v = *reinterpret_cast<const float4*>(G.v + (size_t)r * ld + c0 + h);
         *reinterpret_cast<float4*>(vsm + (size_t)i * VN + h) = v;
       }
     }
   }
+  if (BATCH && tid < 2) s_next[tid] = nw;
   if (tid < 2 * LPR)
     *reinterpret_cast<uint4*>(smem + (tid / LPR) * (size_t)rep_bytes + (size_t)n * W + (tid % LPR) * 16) =
         make_uint4(0u, 0u, 0u, 0u);
@@ -196,17 +205,28 @@ __global__ void __launch_bounds__(NT) k_rows(const __grid_constant__ RowsParams 
 
   const uint32_t base = lds_addr(smem), table = base + 2 * rep_bytes, lists = table + 16u * G.nslices,
                  wts = lists + 16u * G.list16;
-  const int nsteps = P.steps_dev ? min(P.steps, __ldg(P.steps_dev)) : P.steps;
+  int nsteps = P.steps_dev ? min(P.steps, __ldg(P.steps_dev)) : P.steps;
+  if (PERCOL) {
+    // past its longest budget nothing of the slab changes; every warp's lanes hold all of its columns
+    int longest = 0;
+#pragma unroll
+    for (int h = 0; h < VN; ++h) longest = max(longest, tmax[PERCOL ? h : 0]);
+    nsteps = min(nsteps, __reduce_max_sync(0xFFFFFFFFu, longest));
+  }
   uint32_t cur = 0;
   bool bad = false;
   for (int t = 0; t < nsteps; ++t) {
     const uint32_t rep = base + cur * rep_bytes + sub * 16u;
     unsigned char* const next = smem + (size_t)(cur ^ 1u) * rep_bytes;
-    // slices by turns, forth and back, so that every warp gets long and short ones
-    for (int i = 0, s = warp; s < G.nslices; ++i, s = i * nw + ((i & 1) ? nw - 1 - warp : warp)) {
+    if (BATCH && tid == 0) s_next[(t + 1) & 1] = nw;     // last read in step t - 1
+    // slices by turns, forth and back, so that every warp gets long and short ones (BATCH: from the counter)
+    for (int i = 0, s = warp, ahead = 0; s < G.nslices;
+         ++i, s = BATCH ? __shfl_sync(0xFFFFFFFFu, ahead, 0) : i * nw + ((i & 1) ? nw - 1 - warp : warp)) {
       const int p = s * SR + ri;
       const bool row = p < n;
+      const size_t vs = ((size_t)p * LPR + sub) * VN;
       float v[VN] = {};
+      if (BATCH && mom && row) load_f32(v, vsm + vs);   // ahead of the gathers, which hide its latency
       const uint4 si = lds128(table + 16u * s);
       float acc[VN];
 #pragma unroll
@@ -214,6 +234,7 @@ __global__ void __launch_bounds__(NT) k_rows(const __grid_constant__ RowsParams 
       const uint32_t l0 = lists + 16u * (si.x + ri), w0 = wts + 16u * (si.w + 2 * ri);
       gather_rows<PREC, +1, GEN>(acc, rep, l0, w0, 16u * SR, (int)si.y);
       if (WMODE == W_SIGN) gather_rows<PREC, -1, false>(acc, rep, l0 + 16u * SR * ((si.y + 7) / 8), 0, 16u * SR, (int)si.z);
+      if (BATCH && lane == 0) ahead = atomicAdd(&s_next[t & 1], 1);
       if (!row) continue;
       // fused epilogue: gradient, momentum, step, projection
       const uint4 old = lds128(rep + (uint32_t)p * W);
@@ -225,8 +246,7 @@ __global__ void __launch_bounds__(NT) k_rows(const __grid_constant__ RowsParams 
 #pragma unroll
         for (int h = 0; h < 4; ++h) { y[(2 * h) % VN] = bf16lo(u[h]); y[(2 * h + 1) % VN] = bf16hi(u[h]); }
       }
-      float* const vs = vsm + ((size_t)p * LPR + sub) * VN;
-      if (mom) load_f32(v, vs);
+      if (!BATCH && mom) load_f32(v, vsm + vs);
       const float dr = lap ? dn[p] : 0.0f;
       float out[VN];
 #pragma unroll
@@ -247,7 +267,7 @@ __global__ void __launch_bounds__(NT) k_rows(const __grid_constant__ RowsParams 
         q = make_uint4(pack_bf16x2(out[0], out[1]), pack_bf16x2(out[2], out[3]), pack_bf16x2(out[4 % VN], out[5 % VN]),
                        pack_bf16x2(out[6 % VN], out[7 % VN]));
       *reinterpret_cast<uint4*>(next + (size_t)p * W + sub * 16) = q;
-      if (mom) store_f32(vs, v);
+      if (mom) store_f32(vsm + vs, v);
     }
     __syncthreads();
     cur ^= 1u;
@@ -259,7 +279,7 @@ __global__ void __launch_bounds__(NT) k_rows(const __grid_constant__ RowsParams 
     for (int i = tid; i < n * LPR; i += nt) {
       const int r = __ldg(G.order + i / LPR);
       *reinterpret_cast<uint4*>(yg + (size_t)r * ld * ESZ) = fin[i];
-      if (mom && P.store_v) {
+      if (!BATCH && mom && P.store_v) {
 #pragma unroll
         for (int h = 0; h < VN; h += 4)
           *reinterpret_cast<float4*>(G.v + (size_t)r * ld + c0 + h) = *reinterpret_cast<const float4*>(vsm + (size_t)i * VN + h);
@@ -269,30 +289,30 @@ __global__ void __launch_bounds__(NT) k_rows(const __grid_constant__ RowsParams 
   if (bad && P.flag) atomicOr(P.flag, 1);
 }
 
-template <int PREC, int WMODE, bool PERCOL, int LPR>
+template <int PREC, int WMODE, bool PERCOL, int LPR, bool BATCH>
 cudaError_t launch_l(const RowsParams& p, int n_items, cudaStream_t st) {
-  // 1024 threads leave 64 registers: enough but for 8 columns with their own step sizes and budgets
-  constexpr int NT = PREC == DECO_PREC_BF16 && PERCOL ? 512 : 1024;
-  auto fn = k_rows<PREC, WMODE, PERCOL, LPR, NT>;
+  constexpr int NT = rows_max_threads(PREC, PERCOL);
+  auto fn = k_rows<PREC, WMODE, PERCOL, LPR, BATCH, NT>;
   const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
   if (e != cudaSuccess) return e;
   fn<<<(unsigned)n_items, std::min(p.threads, NT), p.smem, st>>>(p);
   return cudaGetLastError();
 }
 
-template <int PREC, int WMODE, bool PERCOL>
+template <int PREC, int WMODE, bool PERCOL, bool BATCH>
 cudaError_t launch_c(const RowsParams& p, int n_items, cudaStream_t st) {
   switch (p.lpr) {
-    case 1: return launch_l<PREC, WMODE, PERCOL, 1>(p, n_items, st);
-    case 2: return launch_l<PREC, WMODE, PERCOL, 2>(p, n_items, st);
-    case 4: return launch_l<PREC, WMODE, PERCOL, 4>(p, n_items, st);
-    default: return launch_l<PREC, WMODE, PERCOL, 8>(p, n_items, st);
+    case 1: return launch_l<PREC, WMODE, PERCOL, 1, BATCH>(p, n_items, st);
+    case 2: return launch_l<PREC, WMODE, PERCOL, 2, BATCH>(p, n_items, st);
+    case 4: return launch_l<PREC, WMODE, PERCOL, 4, BATCH>(p, n_items, st);
+    default: return launch_l<PREC, WMODE, PERCOL, 8, BATCH>(p, n_items, st);
   }
 }
 
 template <int PREC, int WMODE>
 cudaError_t launch_w(const RowsParams& p, bool percol, int n_items, cudaStream_t st) {
-  return percol ? launch_c<PREC, WMODE, true>(p, n_items, st) : launch_c<PREC, WMODE, false>(p, n_items, st);
+  if (p.graphs) return launch_c<PREC, WMODE, true, true>(p, n_items, st);
+  return percol ? launch_c<PREC, WMODE, true, false>(p, n_items, st) : launch_c<PREC, WMODE, false, false>(p, n_items, st);
 }
 
 template <int PREC>
@@ -351,7 +371,7 @@ void slice_table(const int32_t* row_ptr, int wmode, int32_t row0, const std::vec
 
 }  // namespace
 
-size_t rows_smem_bytes(const RowsImage& im, int prec, bool lap, bool mom) {
+size_t rows_smem_bytes(const RowsImage& im, int prec, bool lap, bool mom) {   // mom: in shared memory
   const size_t rep = (size_t)(im.n + 1) * 16 * im.lpr;
   return 2 * rep + 16 * ((size_t)im.nslices + im.list16 + im.wts16) + (lap ? up16((size_t)im.n * 4) : 0) +
          (mom ? (size_t)im.n * im.lpr * (prec == DECO_PREC_BF16 ? 32 : 16) : 0);
@@ -372,8 +392,8 @@ void rows_measure(const int32_t* row_ptr, const float* w, int wmode, int32_t row
   }
 }
 
-int rows_image_rows(const int32_t* row_ptr, const int32_t* col, const float* w, int wmode, int32_t row0, int32_t n,
-                    int lpr, RowsImage* out) {
+void rows_build(const int32_t* row_ptr, const int32_t* col, const float* w, int wmode, int32_t row0, int32_t n,
+                int lpr, RowsImage* out, std::vector<uint32_t>* words_out) {
   RowsImage im;
   im.lpr = lpr;
   im.n = n;
@@ -399,7 +419,8 @@ int rows_image_rows(const int32_t* row_ptr, const int32_t* col, const float* w, 
     }
   }
   const size_t words = 4 * ((size_t)im.nslices + im.list16 + im.wts16) + (size_t)n;
-  std::vector<uint32_t> host(words);
+  std::vector<uint32_t>& host = *words_out;
+  host.assign(words, 0u);
   uint32_t* at = host.data();
   auto put = [&](const void* src, size_t bytes) {
     if (bytes) memcpy(at, src, bytes);
@@ -409,24 +430,23 @@ int rows_image_rows(const int32_t* row_ptr, const int32_t* col, const float* w, 
   put(lists.data(), 16 * (size_t)im.list16);
   put(wts.data(), 16 * (size_t)im.wts16);
   put(order.data(), 4 * (size_t)n);
-  cudaError_t e = cudaMalloc((void**)&im.data, words * 4);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(row image)");
-  e = cudaMemcpy(im.data, host.data(), words * 4, cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) {
-    cudaFree(im.data);
-    return cuda_fail(e, "cudaMemcpy(row image)");
-  }
   *out = im;
-  return DECO_OK;
 }
 
 int rows_image(deco_graph* g, int lpr, const RowsImage** out) {
   for (auto& im : g->rows)
     if (im.lpr == lpr) { *out = &im; return DECO_OK; }
   RowsImage im;
-  int rc = rows_image_rows(g->h_row_ptr.data(), g->h_col.data(), g->h_w.empty() ? nullptr : g->h_w.data(), g->wmode, 0,
-                           g->n, lpr, &im);
-  if (rc) return rc;
+  std::vector<uint32_t> host;
+  rows_build(g->h_row_ptr.data(), g->h_col.data(), g->h_w.empty() ? nullptr : g->h_w.data(), g->wmode, 0, g->n, lpr,
+             &im, &host);
+  cudaError_t e = cudaMalloc((void**)&im.data, host.size() * 4);
+  if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(row image)");
+  e = cudaMemcpy(im.data, host.data(), host.size() * 4, cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) {
+    cudaFree(im.data);
+    return cuda_fail(e, "cudaMemcpy(row image)");
+  }
   g->rows.push_back(im);
   *out = &g->rows.back();
   return DECO_OK;

@@ -15,7 +15,7 @@ struct RowsGraph {
   const int32_t* order;
   const float* dnet;
   void* y;                    // n x ld iterate in global memory (in/out)
-  float* v;                   // n x ld momentum or null
+  float* v;                   // n x ld momentum or null (a batched launch: its scratch, zeroed by the kernel)
   const float* alpha_cols;    // per column or null
   const int32_t* steps_cols;  // per column or null
 };
@@ -41,13 +41,15 @@ size_t rows_smem_bytes(const RowsImage& im, int prec, bool lap, bool mom);
 // sizes and counts of the images of rows [row0, row0 + n) for every lpr, nothing uploaded
 void rows_measure(const int32_t* row_ptr, const float* w, int wmode, int32_t row0, int32_t n,
                   std::vector<RowsImage>* out);
-// one image, on the device (im->data, owned by the caller)
-int rows_image_rows(const int32_t* row_ptr, const int32_t* col, const float* w, int wmode, int32_t row0, int32_t n,
-                    int lpr, RowsImage* im);
+// one image: its sizes and its words (table, lists, weights, order), nothing uploaded
+void rows_build(const int32_t* row_ptr, const int32_t* col, const float* w, int wmode, int32_t row0, int32_t n,
+                int lpr, RowsImage* im, std::vector<uint32_t>* words);
 int rows_image(deco_graph* g, int lpr, const RowsImage** out);   // built once and kept with the graph
 // cycles of one step of one CTA that has its SM to itself, and the shared-memory cycles among them
 double rows_cycles(const RowsImage& im, double* pipe);
 int rows_threads(int32_t n, int lpr);
+// threads of an SM: 1024 leave 64 registers, enough but for 8 columns with their own step sizes and budgets
+constexpr int rows_max_threads(int prec, bool percol) { return prec == DECO_PREC_BF16 && percol ? 512 : 1024; }
 RowsGraph rows_graph(const RowsImage& im);
 int launch_rows(const RowsParams& p, int n_items, int prec, int wmode, cudaStream_t st);
 

@@ -352,7 +352,10 @@ __global__ void __launch_bounds__(NT, 1) k_slab(SlabParams P) {
 
   // a device-side bound (the longest budget of a population round) keeps the
   // launch as short as the round, inside a captured graph as well
-  const int nsteps = P.steps_dev ? min(P.steps, __ldg(P.steps_dev)) : P.steps;
+  int nsteps = P.steps_dev ? min(P.steps, __ldg(P.steps_dev)) : P.steps;
+  // past its longest budget nothing of the slab changes; a warp's lanes hold all of its columns, so every warp of
+  // every CTA of the cluster finds the same bound
+  nsteps = min(nsteps, __reduce_max_sync(0xFFFFFFFFu, max(max(tmax[0], tmax[1]), max(tmax[2], tmax[3]))));
   for (int t = 0; t < nsteps; ++t) {
     if constexpr (PAIR) {
       // two rows per warp, one per half-warp (the second half idles on the

@@ -85,3 +85,30 @@ def test_row_vector_form_flags_nonfinite_and_keeps_limits():
     with pytest.raises(deco.DecoError):
         deco.deco_run_phase(big, 64, 64, torch.zeros(2300, 64, device=DEV), None, 1, deco.step_args(),
                             kernel=deco.DECO_KERNEL_ONCHIP)
+
+
+# Batches: members of unequal sizes in the on-chip form that the planner takes (rows or, for the dense members,
+# 128-byte slabs) and the per-step kernels over the union give the same cuts, scores and population.  Candidates
+# own between one and several slabs' columns, so CTAs stop at budgets of their own.
+@pytest.mark.parametrize("precision", [deco.DECO_PREC_FP32, deco.DECO_PREC_BF16])
+@pytest.mark.parametrize("kind", ["ba", "sign", "weights", "dense"])
+@pytest.mark.parametrize("objective,mu,B,P", [(0, 0.9, 64, 4), (1, 0.9, 30, 15), (1, 0.0, 200, 2)])
+def test_batched_row_vector_form_equals_the_other_forms(precision, kind, objective, mu, B, P):
+    rng = np.random.default_rng(5)
+    graphs = [gg.ba_graph(int(n), 4, 10 + i) for i, n in enumerate(list(rng.integers(20, 900, 20)) + [33])] + [gg.from_edges(1, [], []), gg.er_graph(40, 0.2, 3)]
+    if kind == "sign":
+        graphs = [_weighted(g, [-1.0, 1.0], i) if g.n > 1 else g for i, g in enumerate(graphs)]
+    elif kind == "weights":
+        graphs = [_weighted(g, [-3.0, 2.0, 7.0], i) if g.n > 1 else g for i, g in enumerate(graphs)]
+    elif kind == "dense":
+        graphs = [gg.er_graph(int(n), 0.3, int(n)) for n in rng.integers(20, 300, 12)]
+    batch = deco.deco_create_batch([deco.graph_from(g) for g in graphs])
+    pop = deco.population(candidates=P, rounds=3, t_lo=0, t_hi=25, e_lo=-2.5, e_hi=-1.5, momentum=mu, lifts=(1, 2))
+    outs = []
+    for kernel in (deco.DECO_KERNEL_GLOBAL, deco.DECO_KERNEL_AUTO):
+        p = deco.params(objective=objective, init=deco.DECO_INIT_IDI, precision=precision, kernel=kernel)
+        for _ in range(2):   # the images are kept with the batch
+            _, best, ex = deco.deco_solve_batch(batch, B, p, pop, 9, want_assignment=True, want_round_cuts=True)
+            outs.append((best.tolist(), ex["assignment"].tobytes(), ex["round_cuts"].tobytes(),
+                         ex["round_scores"].tobytes(), ex["final_T"].tobytes()))
+    assert all(o == outs[0] for o in outs)
