@@ -7,10 +7,30 @@
 //
 // Layout: a group of G lanes owns one (row, column chunk); each lane owns one
 // 16-byte vector of the row (4 FP32 or 8 BF16 columns).  Every gathered
-// neighbour row segment is therefore read as G x 16 contiguous bytes; the
-// gather itself (spmm.cuh) keeps eight independent gathers in flight per
-// lane.  Used for graphs whose iterate does not fit on chip and as the
-// reference launch shape for the persistent kernels.
+// neighbour row segment is therefore read as G x 16 contiguous bytes.  The
+// column chunks are the grid's second dimension: all rows of one before the
+// next, so that a gathered chunk keeps L2 to itself.  Used for graphs whose
+// iterate does not fit on chip and as the reference launch shape for the
+// persistent kernels.
+//
+// Bound by the latency of a row's chain (row bounds, indices, gathers) over
+// the warps that the registers allow, and by instruction issue (78 % with
+// 16-bit blocks before the mixed-precision adds).  So: few registers and many
+// warps; four gathers at once and the last one to three together, not one by
+// one; the own row and momentum loaded ahead of the gathers and the momentum
+// past L2 (evict-first); the sums of +-1 and unit graphs in 16 bits by
+// mixed-precision adds.  us per step, before and after:
+//   n        degree  C    precision  weights   momentum
+//   200 003  12      100  FP32       general   0.9       195 -> 178
+//   200 003  12      128  BF16       unit      0          97 ->  75
+//   200 003  12      128  BF16       unit      0.9       127 -> 105
+//   200 003  12       60  FP32       unit      0          80 ->  69
+//   10^6      8      128  BF16       unit      0         531 -> 365
+//   10^6     10       64  FP32       unit      0.9       535 -> 464
+//   10^6      8       20  FP32       unit      0         248 -> 189
+// Eight gathers in flight without momentum: 79 and 380 us on the second and
+// fifth; a loop over rows with the next row's indices prefetched: 136 and 649
+// (24 warps an SM).
 #include <algorithm>
 
 #include "deco_internal.cuh"
@@ -20,7 +40,8 @@ namespace deco {
 namespace {
 
 struct KArgs {
-  int32_t n, C, ld, G, nchunks;
+  int32_t n, C, ld, G, lg;   // G = 2^lg lanes per row
+  int32_t ch0;               // first column chunk of the launch
   const int32_t* row_ptr;
   const int32_t* col_idx;
   const uint32_t* col_sw;
@@ -38,68 +59,144 @@ struct KArgs {
   int32_t* flag;
 };
 
-template <int PREC, int WMODE, bool MOM, bool LAP>
-__global__ void __launch_bounds__(256) k_step_global(KArgs a) {
-  using V = VecT<PREC>;
-  constexpr int VN = V::N;
-  const int lane = threadIdx.x & 31;
-  const int gl = lane % a.G;                      // lane within the group
-  const int64_t group = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / a.G;
-  const int64_t total = (int64_t)a.n * a.nchunks;
-  if (group >= total) return;
-  const int32_t r = (int32_t)(group / a.nchunks);
-  const int32_t ch = (int32_t)(group % a.nchunks);
-  const int32_t vi = ch * a.G + gl;               // vector index within the row
-  const int32_t c0 = vi * VN;                     // first column of this lane
-  if (c0 >= a.C) return;                          // lane beyond the last column
+// Gathers in flight per lane, and blocks per SM (registers): more of both at once does not fit.  Momentum in FP32 is
+// the exception where more gathers win over more warps (464 against 491 us on the sixth graph above).
+template <int PREC, bool MOM>
+struct Shape {
+  static constexpr int U = MOM && PREC == DECO_PREC_FP32 ? 8 : 4;
+  static constexpr int BLOCKS = !MOM ? 6 : PREC == DECO_PREC_FP32 ? 4 : 5;
+};
 
-  float acc[VN];
+__device__ __forceinline__ void unpack(const uint4 q, float (&v)[4]) {
+  v[0] = __uint_as_float(q.x); v[1] = __uint_as_float(q.y); v[2] = __uint_as_float(q.z); v[3] = __uint_as_float(q.w);
+}
+__device__ __forceinline__ void unpack(const uint4 q, float (&v)[8]) {
+  v[0] = bf16lo(q.x); v[1] = bf16hi(q.x); v[2] = bf16lo(q.y); v[3] = bf16hi(q.y);
+  v[4] = bf16lo(q.z); v[5] = bf16hi(q.z); v[6] = bf16lo(q.w); v[7] = bf16hi(q.w);
+}
+
+// acc += the vector q of entry x (column index, or index | sign bit), weight w (W_GENERAL)
+template <int PREC, int WMODE, int VN>
+__device__ __forceinline__ void add_entry(float (&acc)[VN], uint4 q, uint32_t x, float w) {
+  if constexpr (PREC == DECO_PREC_BF16 && WMODE != W_GENERAL) {
+    // +-1: the sign bits of both halves, then the mixed-precision add (bf16 widened exactly, one rounding)
+    const uint32_t flip = WMODE == W_SIGN && (x & 0x80000000u) ? 0x80008000u : 0u;
+    const uint32_t u[4] = {q.x ^ flip, q.y ^ flip, q.z ^ flip, q.w ^ flip};
 #pragma unroll
-  for (int k = 0; k < VN; ++k) acc[k] = 0.0f;
-  const int32_t e0 = __ldg(a.row_ptr + r), e1 = __ldg(a.row_ptr + r + 1);
-  const CsrView A{a.col_idx, a.col_sw, a.w};
-  csr_gather_row<PREC, WMODE>(A, a.yin, a.ld, c0, e0, e1, acc);
+    for (int h = 0; h < 4; ++h)
+      asm("{\n .reg .b16 lo, hi;\n mov.b32 {lo, hi}, %2;\n add.rn.f32.bf16 %0, lo, %0;\n add.rn.f32.bf16 %1, hi, %1;\n}"
+          : "+f"(acc[2 * h]), "+f"(acc[2 * h + 1])
+          : "r"(u[h]));
+  } else {
+    float v[VN];
+    unpack(q, v);
+    if (WMODE == W_SIGN) w = (x & 0x80000000u) ? -1.0f : 1.0f;
+#pragma unroll
+    for (int k = 0; k < VN; ++k) acc[k] = WMODE == W_UNIT ? acc[k] + v[k] : fmaf(w, v[k], acc[k]);
+  }
+}
 
-  // ---- epilogue: gradient, momentum, step, projection
+template <int PREC, int WMODE, bool MOM, bool LAP>
+__global__ void __launch_bounds__(256, Shape<PREC, MOM>::BLOCKS) k_step_global(const __grid_constant__ KArgs a) {
+  using V = VecT<PREC>;
+  constexpr int VN = V::N, U = Shape<PREC, MOM>::U;
+  const int gl = threadIdx.x & (a.G - 1);         // lane within the group
+  const int64_t row = ((int64_t)blockIdx.x << (8 - a.lg)) + (threadIdx.x >> a.lg);
+  const int32_t c0 = ((a.ch0 + (int32_t)blockIdx.y) * a.G + gl) * VN;   // first column of this lane
+  if (row >= a.n || c0 >= a.C) return;
+  const int32_t r = (int32_t)row;
+
+  const int32_t e1 = __ldg(a.row_ptr + r + 1);
+  int32_t e = __ldg(a.row_ptr + r);
+  // own row and momentum ahead of the gathers, which hide their latency
   const size_t base = (size_t)r * a.ld + c0;
-  float y[VN], out[VN];
-  V::load(a.yin, base, y);
-  const float dr = LAP ? __ldg(a.dnet + r) : 0.0f;
+  const uint4 own = __ldg(reinterpret_cast<const uint4*>(static_cast<const char*>(a.yin) + base * (16 / VN)));
   float vv[VN];
   if (MOM) {
 #pragma unroll
     for (int k = 0; k < VN; k += 4) {
-      float4 q = *reinterpret_cast<const float4*>(a.v + base + k);
+      const float4 q = __ldcs(reinterpret_cast<const float4*>(a.v + base + k));
       vv[k] = q.x; vv[k + 1] = q.y; vv[k + 2] = q.z; vv[k + 3] = q.w;
     }
   }
-  bool bad = false;
+  const float dr = LAP ? __ldg(a.dnet + r) : 0.0f;
+  const char* const yb = static_cast<const char*>(a.yin) + (size_t)c0 * (16 / VN);
+  const uint32_t row_bytes = (uint32_t)a.ld * (16 / VN);
+  const uint32_t* const col = WMODE == W_SIGN ? a.col_sw : reinterpret_cast<const uint32_t*>(a.col_idx);
+  auto gather = [&](uint32_t x) {
+    return __ldg(reinterpret_cast<const uint4*>(yb + (size_t)(WMODE == W_SIGN ? x & 0x7FFFFFFFu : x) * row_bytes));
+  };
+
+  float acc[VN];
 #pragma unroll
-  for (int k = 0; k < VN; ++k) {
-    const int32_t c = c0 + k;
-    float grad = LAP ? fmaf(dr, y[k], -acc[k]) : -acc[k];
-    float step = grad;
-    if (MOM) {
-      step = fmaf(a.mu, vv[k], grad);
+  for (int k = 0; k < VN; ++k) acc[k] = 0.0f;
+  uint4 raw[U];
+  uint32_t x[U];
+  float w[U] = {};
+  for (; e + U <= e1; e += U) {
+#pragma unroll
+    for (int q = 0; q < U; ++q) {
+      x[q] = __ldg(col + e + q);
+      if (WMODE == W_GENERAL) w[q] = __ldg(a.w + e + q);
+      raw[q] = gather(x[q]);
     }
-    float alpha = a.alpha_cols ? a.afac * __ldg(a.alpha_cols + (c < a.C ? c : 0)) : a.alpha_eff;
-    bool active = (c < a.C) && (!a.steps_cols || a.t < __ldg(a.steps_cols + c));
-    float yn = fmaf(alpha, step, y[k]);
-    if (active && !isfinite(yn)) bad = true;
-    yn = fminf(fmaxf(yn, -1.0f), 1.0f);
-    out[k] = active ? yn : y[k];
-    if (MOM && active) vv[k] = step;
+#pragma unroll
+    for (int q = 0; q < U; ++q) add_entry<PREC, WMODE>(acc, raw[q], x[q], w[q]);
   }
-  if (c0 + VN <= a.C) {
+  // the last entries, together
+#pragma unroll
+  for (int q = 0; q < U - 1; ++q) {
+    if (e + q < e1) {
+      x[q] = __ldg(col + e + q);
+      if (WMODE == W_GENERAL) w[q] = __ldg(a.w + e + q);
+      raw[q] = gather(x[q]);
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < U - 1; ++q)
+    if (e + q < e1) add_entry<PREC, WMODE>(acc, raw[q], x[q], w[q]);
+
+  // ---- epilogue: gradient, momentum, step, projection
+  float y[VN], out[VN];
+  unpack(own, y);
+  bool bad = false;
+  const bool whole = c0 + VN <= a.C;
+  if (whole && !a.alpha_cols && !a.steps_cols) {
+#pragma unroll
+    for (int k = 0; k < VN; ++k) {
+      const float grad = LAP ? fmaf(dr, y[k], -acc[k]) : -acc[k];
+      if (MOM) vv[k] = fmaf(a.mu, vv[k], grad);
+      const float yn = fmaf(a.alpha_eff, MOM ? vv[k] : grad, y[k]);
+      bad = bad || !isfinite(yn);
+      out[k] = fminf(fmaxf(yn, -1.0f), 1.0f);
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < VN; ++k) {
+      const int32_t c = c0 + k;
+      const float grad = LAP ? fmaf(dr, y[k], -acc[k]) : -acc[k];
+      const float step = MOM ? fmaf(a.mu, vv[k], grad) : grad;
+      const float alpha = a.alpha_cols ? a.afac * __ldg(a.alpha_cols + (c < a.C ? c : 0)) : a.alpha_eff;
+      const bool active = (c < a.C) && (!a.steps_cols || a.t < __ldg(a.steps_cols + c));
+      float yn = fmaf(alpha, step, y[k]);
+      if (active && !isfinite(yn)) bad = true;
+      yn = fminf(fmaxf(yn, -1.0f), 1.0f);
+      out[k] = active ? yn : y[k];
+      if (MOM && active) vv[k] = step;
+    }
+  }
+  if (whole) {
     V::store(a.yout, base, out);
     if (MOM) {
 #pragma unroll
       for (int k = 0; k < VN; k += 4)
-        *reinterpret_cast<float4*>(a.v + base + k) = make_float4(vv[k], vv[k + 1], vv[k + 2], vv[k + 3]);
+        __stcs(reinterpret_cast<float4*>(a.v + base + k), make_float4(vv[k], vv[k + 1], vv[k + 2], vv[k + 3]));
     }
   } else {
     // ragged last vector: only columns < C are written
-    for (int k = 0; k < VN && c0 + k < a.C; ++k) {
+#pragma unroll
+    for (int k = 0; k < VN; ++k) {
+      if (c0 + k >= a.C) continue;
       if (PREC == DECO_PREC_FP32) static_cast<float*>(a.yout)[base + k] = out[k];
       else static_cast<__nv_bfloat16*>(a.yout)[base + k] = __float2bfloat16_rn(out[k]);
       if (MOM) a.v[base + k] = vv[k];
@@ -108,29 +205,22 @@ __global__ void __launch_bounds__(256) k_step_global(KArgs a) {
   if (bad && a.flag) atomicExch(a.flag, 1);
 }
 
-template <int PREC, int WMODE, bool MOM, bool LAP>
-void launch_t(const KArgs& a, int64_t threads, cudaStream_t st) {
-  const int block = 256;
-  const int64_t grid = (threads + block - 1) / block;
-  k_step_global<PREC, WMODE, MOM, LAP><<<(unsigned)grid, block, 0, st>>>(a);
-}
-
 template <int PREC, int WMODE>
-void launch_w(const KArgs& a, bool mom, bool lap, int64_t threads, cudaStream_t st) {
+void launch_w(const KArgs& a, bool mom, bool lap, dim3 grid, cudaStream_t st) {
   if (mom) {
-    if (lap) launch_t<PREC, WMODE, true, true>(a, threads, st);
-    else launch_t<PREC, WMODE, true, false>(a, threads, st);
+    if (lap) k_step_global<PREC, WMODE, true, true><<<grid, 256, 0, st>>>(a);
+    else k_step_global<PREC, WMODE, true, false><<<grid, 256, 0, st>>>(a);
   } else {
-    if (lap) launch_t<PREC, WMODE, false, true>(a, threads, st);
-    else launch_t<PREC, WMODE, false, false>(a, threads, st);
+    if (lap) k_step_global<PREC, WMODE, false, true><<<grid, 256, 0, st>>>(a);
+    else k_step_global<PREC, WMODE, false, false><<<grid, 256, 0, st>>>(a);
   }
 }
 
 template <int PREC>
-void launch_p(const KArgs& a, int wmode, bool mom, bool lap, int64_t threads, cudaStream_t st) {
-  if (wmode == W_UNIT) launch_w<PREC, W_UNIT>(a, mom, lap, threads, st);
-  else if (wmode == W_SIGN) launch_w<PREC, W_SIGN>(a, mom, lap, threads, st);
-  else launch_w<PREC, W_GENERAL>(a, mom, lap, threads, st);
+void launch_p(const KArgs& a, int wmode, bool mom, bool lap, dim3 grid, cudaStream_t st) {
+  if (wmode == W_UNIT) launch_w<PREC, W_UNIT>(a, mom, lap, grid, st);
+  else if (wmode == W_SIGN) launch_w<PREC, W_SIGN>(a, mom, lap, grid, st);
+  else launch_w<PREC, W_GENERAL>(a, mom, lap, grid, st);
 }
 
 }  // namespace
@@ -140,12 +230,11 @@ int launch_step_global(const StepLaunch& s, cudaStream_t st) {
   const int VN = s.precision == DECO_PREC_BF16 ? 8 : 4;
   const int nvec = (s.C + VN - 1) / VN;
   int G = 1;
-  while (G < nvec && G < 32) G <<= 1;
+  for (; G < nvec && G < 32; G <<= 1) ++a.lg;
   a.n = s.n;
   a.C = s.C;
   a.ld = s.ld;
   a.G = G;
-  a.nchunks = (nvec + G - 1) / G;
   a.row_ptr = s.row_ptr;
   a.col_idx = s.col_idx;
   a.col_sw = s.col_sw;
@@ -162,13 +251,17 @@ int launch_step_global(const StepLaunch& s, cudaStream_t st) {
   a.steps_cols = s.steps_cols;
   a.t = s.t;
   a.flag = s.flag;
-  const int64_t threads = (int64_t)s.n * a.nchunks * G;
-  if (threads == 0) return DECO_OK;
+  if (s.n == 0 || s.C == 0) return DECO_OK;
   const bool mom = s.mu != 0.0f;
   const bool lap = s.objective == DECO_OBJ_LAPLACIAN;
-  if (s.precision == DECO_PREC_BF16) launch_p<DECO_PREC_BF16>(a, s.wmode, mom, lap, threads, st);
-  else launch_p<DECO_PREC_FP32>(a, s.wmode, mom, lap, threads, st);
-  DECO_CUDA_TRY(cudaGetLastError());
+  const int32_t nchunks = (nvec + G - 1) / G;
+  const unsigned rows = (unsigned)(((int64_t)s.n * G + 255) / 256);
+  for (a.ch0 = 0; a.ch0 < nchunks; a.ch0 += 65535) {
+    const dim3 grid(rows, (unsigned)std::min(nchunks - a.ch0, 65535));
+    if (s.precision == DECO_PREC_BF16) launch_p<DECO_PREC_BF16>(a, s.wmode, mom, lap, grid, st);
+    else launch_p<DECO_PREC_FP32>(a, s.wmode, mom, lap, grid, st);
+    DECO_CUDA_TRY(cudaGetLastError());
+  }
   return DECO_OK;
 }
 
