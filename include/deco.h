@@ -622,13 +622,16 @@ int deco_probe_wait_timeout(int32_t which, float* waited_ms, void* stream);
  * against concurrent calls.  No paper counterpart.  Errors: DECO_ERR_ARG. */
 int deco_debug_fail_scratch_alloc(int32_t k);
 
-/* Diagnostic for tests of allocation behaviour: the current device's current
- * stream-ordered memory pool, from which every scratch buffer of the library
- * is taken (cudaMallocAsync).  used_now (host, or NULL) receives the bytes of
+/* Diagnostic for tests of allocation behaviour: the stream-ordered memory pool
+ * from which every scratch buffer of the library is taken on the current
+ * device.  It is the library's own pool, which keeps up to 256 MiB between
+ * calls and gives them back when the last graph is destroyed; where the caller
+ * has made another pool the device's current one (cudaDeviceSetMemPool), it is
+ * that pool.  used_now (host, or NULL) receives the bytes of
  * the pool in use now, used_high (host, or NULL) the most bytes in use at once
  * since the high-water mark was last reset; reset != 0 then restarts the
- * high-water mark from the current use.  Process-wide (the pool is shared with
- * every other user of it in the process).  No paper counterpart.
+ * high-water mark from the current use.  Process-wide (the pool is shared by
+ * all calls in the process).  No paper counterpart.
  * Errors: CUDA. */
 int deco_debug_pool_usage(int64_t* used_now, int64_t* used_high, int32_t reset);
 

@@ -383,8 +383,8 @@ def deco_debug_fail_scratch_alloc(k: int):
 
 
 def deco_debug_pool_usage(reset: bool = False):
-    """(bytes in use, high-water mark) of the current device's stream-ordered
-    memory pool, which every scratch buffer of the library comes from; with
+    """(bytes in use, high-water mark) of the stream-ordered memory pool that
+    the library's scratch buffers come from on the current device; with
     reset the high-water mark then restarts from the current use."""
     now, high = ctypes.c_int64(), ctypes.c_int64()
     _check(lib.deco_debug_pool_usage(ctypes.byref(now), ctypes.byref(high), 1 if reset else 0))

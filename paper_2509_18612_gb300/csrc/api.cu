@@ -51,10 +51,8 @@ extern "C" int deco_debug_fail_scratch_alloc(int32_t k) {
 
 extern "C" int deco_debug_pool_usage(int64_t* used_now, int64_t* used_high, int32_t reset) {
   clear_error();
-  int dev = 0;
-  DECO_CUDA_TRY(cudaGetDevice(&dev));
   cudaMemPool_t pool = nullptr;
-  DECO_CUDA_TRY(cudaDeviceGetMemPool(&pool, dev));
+  DECO_CUDA_TRY(scratch_pool(&pool));
   cuuint64_t now = 0, high = 0;
   DECO_CUDA_TRY(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &now));
   DECO_CUDA_TRY(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemHigh, &high));

@@ -60,8 +60,8 @@ struct Scratch {
     }
     void* p = nullptr;
     if (bytes == 0) bytes = 16;
-    cudaError_t e = cudaMallocAsync(&p, bytes, st);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync(scratch)");
+    cudaError_t e = scratch_malloc(&p, bytes, st);
+    if (e != cudaSuccess) return cuda_fail(e, "scratch allocation");
     ptrs.push_back(p);
     *out = static_cast<T*>(p);
     return DECO_OK;

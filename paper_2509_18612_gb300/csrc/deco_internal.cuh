@@ -49,6 +49,14 @@ void set_error(const char* fmt, ...);
 void clear_error();
 int cuda_fail(cudaError_t e, const char* what);   // records message, returns DECO_ERR_CUDA / OOM
 
+// Stream-ordered scratch memory (freed by cudaFreeAsync), scratch.cu: its pool, an allocation, and the return of
+// what the pool keeps
+cudaError_t scratch_pool(cudaMemPool_t* pool);
+cudaError_t scratch_malloc(void** p, size_t bytes, cudaStream_t st);
+void scratch_reserve();   // makes the pool: with the first graph, so that no call makes it while a stream captures
+void scratch_trim();
+int current_context_id(unsigned long long* id);   // unique id of the current context (noalloc.cu)
+
 #define DECO_CUDA_TRY(expr)                                   \
   do {                                                        \
     cudaError_t _e = (expr);                                  \
@@ -133,6 +141,7 @@ struct deco_graph {
   int wmode = deco::W_UNIT;     // storage used by the kernels
   int32_t max_abs_w = 1;        // largest |w|
   int device = 0;
+  bool counted = false;         // a handle that has been given to a caller
   // host-side facts (degree statistics for IDI / DUI)
   int64_t deg_s1 = 0, deg_s2 = 0;
   int32_t max_deg = 0;

@@ -2,6 +2,7 @@
 // Def. 1 / Eq. 1 (undirected graph, each crossing edge counted once) and the
 // Sec. 2 notation (A symmetric adjacency, D degree matrix, L = D - A).
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -43,6 +44,8 @@ double idi_threshold(const deco_graph* g, float beta) {
   return mean + (double)beta * std::sqrt(var);
 }
 
+static std::atomic<int64_t> g_graphs{0};   // handles that callers hold
+
 static void free_graph(deco_graph* g) {
   if (!g) return;
   for (auto& im : g->images) cudaFree(im.data);
@@ -56,7 +59,9 @@ static void free_graph(deco_graph* g) {
   cudaFree(g->wint);
   cudaFree(g->dnet);
   cudaFree(g->deg);
+  const bool counted = g->counted;
   delete g;
+  if (counted && --g_graphs == 0) scratch_trim();
 }
 
 }  // namespace deco
@@ -332,6 +337,9 @@ int deco::create_graph_impl(int32_t n, int64_t nnz, const int32_t* row_ptr, cons
     free_graph(g);
     return rc;
   }
+  g->counted = true;
+  ++g_graphs;
+  scratch_reserve();
   *out = g;
   return DECO_OK;
 }

@@ -17,6 +17,51 @@ using namespace deco;
 
 namespace {
 
+// cuCtxGetCurrent and cuCtxGetId through the runtime's driver entry-point
+// query, so that the library needs no link-time dependency on the driver API.
+using CtxGetCurrentFn = int (*)(void**);
+using CtxGetIdFn = int (*)(void*, unsigned long long*);
+template <typename F>
+int driver_fn(const char* name, F* fn) {
+  if (*fn) return DECO_OK;
+  void* f = nullptr;
+  cudaDriverEntryPointQueryResult q{};
+  cudaError_t e = cudaGetDriverEntryPointByVersion(name, &f, 12000, cudaEnableDefault, &q);
+  if (e != cudaSuccess) return cuda_fail(e, "cudaGetDriverEntryPointByVersion");
+  if (q != cudaDriverEntryPointSuccess || !f) {
+    set_error("%s is not available from the driver", name);
+    return DECO_ERR_CUDA;
+  }
+  *fn = reinterpret_cast<F>(f);
+  return DECO_OK;
+}
+
+}  // namespace
+
+namespace deco {
+// unique id of the current context (DECO_ERR_CUDA when none is current)
+int current_context_id(unsigned long long* id) {
+  static std::mutex mutex;
+  std::lock_guard<std::mutex> lock(mutex);
+  static CtxGetCurrentFn get_current = nullptr;
+  static CtxGetIdFn get_id = nullptr;
+  int rc = driver_fn("cuCtxGetCurrent", &get_current);
+  if (rc || (rc = driver_fn("cuCtxGetId", &get_id))) return rc;
+  void* ctx = nullptr;
+  if (get_current(&ctx) != 0 || !ctx) {
+    set_error("no current CUDA context");
+    return DECO_ERR_CUDA;
+  }
+  if (get_id(ctx, id) != 0) {
+    set_error("cuCtxGetId failed");
+    return DECO_ERR_CUDA;
+  }
+  return DECO_OK;
+}
+}  // namespace deco
+
+namespace {
+
 // Fixed scratch: the second block of the ping-pong between steps.  It is a
 // file-scope device array, so every GPU that loads the library keeps these
 // 16 MiB until the process exits.
@@ -38,43 +83,6 @@ struct ScratchSlot {
 };
 ScratchSlot g_scratch_slot[kMaxDevices];
 std::mutex g_scratch_mutex;
-
-// cuCtxGetCurrent and cuCtxGetId through the runtime's driver entry-point
-// query, so that the library needs no link-time dependency on the driver API.
-using CtxGetCurrentFn = int (*)(void**);
-using CtxGetIdFn = int (*)(void*, unsigned long long*);
-template <typename F>
-int driver_fn(const char* name, F* fn) {
-  if (*fn) return DECO_OK;
-  void* f = nullptr;
-  cudaDriverEntryPointQueryResult q{};
-  cudaError_t e = cudaGetDriverEntryPointByVersion(name, &f, 12000, cudaEnableDefault, &q);
-  if (e != cudaSuccess) return cuda_fail(e, "cudaGetDriverEntryPointByVersion");
-  if (q != cudaDriverEntryPointSuccess || !f) {
-    set_error("%s is not available from the driver", name);
-    return DECO_ERR_CUDA;
-  }
-  *fn = reinterpret_cast<F>(f);
-  return DECO_OK;
-}
-
-// unique id of the current context (DECO_ERR_CUDA when none is current)
-int current_context_id(unsigned long long* id) {
-  static CtxGetCurrentFn get_current = nullptr;
-  static CtxGetIdFn get_id = nullptr;
-  int rc = driver_fn("cuCtxGetCurrent", &get_current);
-  if (rc || (rc = driver_fn("cuCtxGetId", &get_id))) return rc;
-  void* ctx = nullptr;
-  if (get_current(&ctx) != 0 || !ctx) {
-    set_error("no current CUDA context");
-    return DECO_ERR_CUDA;
-  }
-  if (get_id(ctx, id) != 0) {
-    set_error("cuCtxGetId failed");
-    return DECO_ERR_CUDA;
-  }
-  return DECO_OK;
-}
 
 int scratch_address(void** out) {
   int dev = 0;

@@ -322,19 +322,19 @@ int PhaseRunner::prepare(const deco_graph* g_, int32_t C_, int32_t ld_, int prec
     }
     const size_t elems = (size_t)plan.cpad * plan.kpad;
     for (int i = 0; i < 2; ++i) {
-      cudaError_t e = cudaMallocAsync((void**)&yt[i], elems * 2, st);
-      if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync(transposed block)");
+      cudaError_t e = scratch_malloc((void**)&yt[i], elems * 2, st);
+      if (e != cudaSuccess) return cuda_fail(e, "scratch allocation (transposed block)");
       // node padding of YT must stay zero (finite) for the products with A's zero columns
       if ((e = cudaMemsetAsync(yt[i], 0, elems * 2, st)) != cudaSuccess) return cuda_fail(e, "memset");
     }
-    cudaError_t e = cudaMallocAsync((void**)&vt, elems * sizeof(float), st);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync(transposed momentum)");
+    cudaError_t e = scratch_malloc((void**)&vt, elems * sizeof(float), st);
+    if (e != cudaSuccess) return cuda_fail(e, "scratch allocation (transposed momentum)");
     if ((e = cudaMemsetAsync(vt, 0, elems * sizeof(float), st)) != cudaSuccess) return cuda_fail(e, "memset");
     maps = new (std::nothrow) DenseMaps;
     if (!maps) { set_error("out of host memory"); return DECO_ERR_OOM; }
     if (plan.dpersist) {
-      if ((e = cudaMallocAsync((void**)&gbar, sizeof(unsigned int), st)) != cudaSuccess)
-        return cuda_fail(e, "cudaMallocAsync(grid barrier)");
+      if ((e = scratch_malloc((void**)&gbar, sizeof(unsigned int), st)) != cudaSuccess)
+        return cuda_fail(e, "scratch allocation (grid barrier)");
     }
     return dense_make_maps(g->dense, plan.kpad, yt, plan.cpad, plan.dpersist ? plan.dphase.w : 0, maps);
   }
@@ -359,8 +359,8 @@ int PhaseRunner::prepare(const deco_graph* g_, int32_t C_, int32_t ld_, int prec
   }
   if ((plan.k > 1 && plan.xmode == 2) || plan.lean) {
     const size_t bytes = 2 * (size_t)plan.items * g->n * 128;
-    cudaError_t e = cudaMallocAsync((void**)&xbuf, bytes, st);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync(exchange buffer)");
+    cudaError_t e = scratch_malloc((void**)&xbuf, bytes, st);
+    if (e != cudaSuccess) return cuda_fail(e, "scratch allocation (exchange buffer)");
   }
   return DECO_OK;
 }
@@ -509,8 +509,8 @@ int PhaseRunner::run(void* y[2], int& cur, float* v, int32_t steps, int objectiv
     const size_t esz = prec == DECO_PREC_BF16 ? 2 : 4;
     const bool momv = mu != 0.0f && v != nullptr;
     if (!ypart) {
-      cudaError_t e = cudaMallocAsync((void**)&ypart, (size_t)g->n * w * S * esz, st);
-      if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync(slab partner)");
+      cudaError_t e = scratch_malloc((void**)&ypart, (size_t)g->n * w * S * esz, st);
+      if (e != cudaSuccess) return cuda_fail(e, "scratch allocation (slab partner)");
     }
     // y[cur] is only read (into slab-major A) and, at the end, its columns
     // < C are rewritten; its padding columns are never touched
@@ -520,8 +520,8 @@ int PhaseRunner::run(void* y[2], int& cur, float* v, int32_t steps, int objectiv
     if (rc) return rc;
     if (momv) {
       if (!vslab) {
-        cudaError_t e = cudaMallocAsync((void**)&vslab, (size_t)g->n * w * S * sizeof(float), st);
-        if (e != cudaSuccess) return cuda_fail(e, "cudaMallocAsync(slab momentum)");
+        cudaError_t e = scratch_malloc((void**)&vslab, (size_t)g->n * w * S * sizeof(float), st);
+        if (e != cudaSuccess) return cuda_fail(e, "scratch allocation (slab momentum)");
       }
       if ((rc = launch_slab_layout(g->n, ld, C, w, S, 4, v, vslab, true, st))) return rc;
     }

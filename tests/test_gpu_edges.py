@@ -256,3 +256,23 @@ def test_rounding_by_vectors_equals_rounding_by_columns(lift, pad, precision):
     bits = ((words[:, :, None] >> np.arange(32, dtype=np.uint32)) & 1).reshape(n, 64)
     np.testing.assert_array_equal(bits[:, :B], Z.astype(np.uint32))
     assert not bits[:, B:].any()
+
+
+def test_scratch_pool_takes_back_what_calls_used_on_two_streams():
+    G = deco.graph_from(gg.er_graph_avg_degree(3000, 6.0, 1))
+    C = 64
+    y0 = torch.rand(3000, C, device="cuda")
+    blocks = [y0.clone(), y0.clone(), y0.clone()]
+    args = deco.step_args(0, 0, 0.01, 0.0)
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    torch.cuda.synchronize()
+    before, _ = deco.deco_debug_pool_usage(reset=True)
+    for _ in range(3):
+        for y, st in zip(blocks, streams):   # both calls' scratch in flight at once
+            deco.deco_run_phase(G, C, C, y, None, 9, args, deco.DECO_KERNEL_GLOBAL, stream=st.cuda_stream)
+    torch.cuda.synchronize()
+    now, high = deco.deco_debug_pool_usage()
+    assert now == before and high >= before + 3000 * C * 4
+    for _ in range(3):
+        deco.deco_run_phase(G, C, C, blocks[2], None, 9, args, deco.DECO_KERNEL_GLOBAL)
+    assert torch.equal(blocks[0], blocks[2]) and torch.equal(blocks[1], blocks[2])
