@@ -320,7 +320,7 @@ int batch_rows_shape(const deco_batch* b, int32_t C, int prec, bool lap, BatchSl
     double sum = 0.0, last = 0.0;
     for (const auto& sizes : b->rows_sizes) {
       double pipe = 0.0;
-      const double alone = rows_cycles(sizes[l], &pipe);
+      const double alone = rows_cycles(sizes[l], false, &pipe);
       sum += std::max(pipe, alone / per_sm) * (double)items / sms;
       last = std::max(last, alone);
     }

@@ -72,20 +72,22 @@ double slab_cycles(int64_t own_nnz, int32_t own, int32_t n, int k, int waves, in
   return waves * (gather * (double)own_nnz + 3.0 * n + (k == 8 ? 2500.0 : 3600.0) + (bf ? 1100.0 : 0.0));
 }
 // k_rows: several CTAs may share an SM; they then share its shared-memory pipe
-static double rows_step_cycles(const RowsImage& im, int prec, int items, int max_smem) {
+static double rows_step_cycles(const RowsImage& im, int prec, int wmode, int items, int max_smem) {
   double pipe = 0.0;
-  const double alone = rows_cycles(im, &pipe);
-  const size_t smem = rows_smem_bytes(im, prec, true, true);
+  const bool registers = rows_reg_fits(im, wmode);
+  const double alone = rows_cycles(im, registers, &pipe);
+  const size_t smem = registers ? rows_reg_smem_bytes(im) : rows_smem_bytes(im, prec, true, true);
   const int threads = rows_threads(im.n, im.lpr);
-  const int per_sm = std::max(1, std::min((int)((max_smem + 2048) / (smem + 1024)), 1024 / threads));
+  const int per_sm = std::max(1, std::min((int)((max_smem + 2048) / (smem + 1024)), (registers ? 768 : 1024) / threads));
   const int sms = device_sm_count();
   const int waves = (items + sms * per_sm - 1) / (sms * per_sm);
   const int share = std::min(per_sm, (items + sms - 1) / sms);
   return waves * std::max(alone, share * pipe + 350.0);
 }
-// one launch of the per-step kernel: the launch, and its gathers at ~4.5 TB/s
+// one launch of the per-step kernel: the launch (4.6 - 6.3 us a step for graphs of 1 400 - 5 000 rows and 8 columns),
+// and its gathers at ~4.5 TB/s
 static double step_cycles(const deco_graph* g, int32_t C, int prec) {
-  return 5500.0 + (double)g->nnz * C * (prec == DECO_PREC_BF16 ? 2.0 : 4.0) / 4.5e12 * 2.07e9;
+  return 9000.0 + (double)g->nnz * C * (prec == DECO_PREC_BF16 ? 2.0 : 4.0) / 4.5e12 * 2.07e9;
 }
 
 bool valid_selector(int kernel) {
@@ -286,9 +288,9 @@ int plan_phase(const deco_graph* g, int32_t C, int32_t ld, int prec, int force, 
     if (sizes.empty())
       rows_measure(g->h_row_ptr.data(), g->h_w.empty() ? nullptr : g->h_w.data(), g->wmode, 0, g->n, &sizes);
     for (const RowsImage& im : sizes) {
-      if (rows_smem_bytes(im, prec, true, true) > (size_t)max_smem) continue;
+      if (rows_smem_bytes(im, prec, true, true) > (size_t)max_smem) continue;   // k_rows may run it as well
       const int w = im.lpr * (prec == DECO_PREC_BF16 ? 8 : 4);
-      const double t = rows_step_cycles(im, prec, (C + w - 1) / w, max_smem);
+      const double t = rows_step_cycles(im, prec, g->wmode, (C + w - 1) / w, max_smem);
       if (t < least) {
         least = t;
         plan->kernel = KERNEL_ROWS;
@@ -429,7 +431,9 @@ int PhaseRunner::run(void* y[2], int& cur, float* v, int32_t steps, int objectiv
     p.load_v = load_v ? 1 : 0;
     p.store_v = store_v ? 1 : 0;
     p.flag = flag;
-    const int rc = launch_rows(p, plan.items, prec, g->wmode, st);
+    const bool in_registers = !alpha_cols && !steps_cols && rows_reg_fits(*plan.rows, g->wmode);
+    const int rc = in_registers ? launch_rows_reg(p, *plan.rows, plan.items, prec, g->wmode, st)
+                                : launch_rows(p, plan.items, prec, g->wmode, st);
     if (rc) return rc;
     if (kernels) *kernels += 1;
     return DECO_OK;

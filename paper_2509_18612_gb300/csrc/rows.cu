@@ -68,12 +68,19 @@ __device__ __forceinline__ void add_vec(float* acc, uint4 q, float w) {
 #pragma unroll
     for (int h = 0; h < 4; ++h) acc[h] = GEN ? fmaf(w, y[h], acc[h]) : SIGN > 0 ? acc[h] + y[h] : acc[h] - y[h];
   } else {
-    const uint32_t u[4] = {q.x, q.y, q.z, q.w};
+    const uint32_t flip = !GEN && SIGN < 0 ? 0x80008000u : 0u;
+    const uint32_t u[4] = {q.x ^ flip, q.y ^ flip, q.z ^ flip, q.w ^ flip};
 #pragma unroll
     for (int h = 0; h < 4; ++h) {
-      const float lo = bf16lo(u[h]), hi = bf16hi(u[h]);
-      acc[2 * h] = GEN ? fmaf(w, lo, acc[2 * h]) : SIGN > 0 ? acc[2 * h] + lo : acc[2 * h] - lo;
-      acc[2 * h + 1] = GEN ? fmaf(w, hi, acc[2 * h + 1]) : SIGN > 0 ? acc[2 * h + 1] + hi : acc[2 * h + 1] - hi;
+      if (GEN) {
+        acc[2 * h] = fmaf(w, bf16lo(u[h]), acc[2 * h]);
+        acc[2 * h + 1] = fmaf(w, bf16hi(u[h]), acc[2 * h + 1]);
+      } else {
+        // the mixed-precision add: the 16-bit value widened exactly, one rounding
+        asm("{\n .reg .b16 lo, hi;\n mov.b32 {lo, hi}, %2;\n add.rn.f32.bf16 %0, lo, %0;\n add.rn.f32.bf16 %1, hi, %1;\n}"
+            : "+f"(acc[2 * h]), "+f"(acc[2 * h + 1])
+            : "r"(u[h]));
+      }
     }
   }
 }
@@ -465,11 +472,16 @@ RowsGraph rows_graph(const RowsImage& im) {
 
 // Fitted to the measured steps of ER(800, 0.06), degree 48 (FP32: 14 500 / 22 600 / 33 000 cycles for LPR 1 / 2 / 4)
 // and of graphs of degree 4 ... 20; the shared-memory part is within 10 % of them.
-double rows_cycles(const RowsImage& im, double* pipe) {
+// In registers only the entries' vectors and the new row are left (graphs of 60 - 1 000 rows, degree 5 - 16: within 12 %).
+double rows_cycles(const RowsImage& im, bool registers, double* pipe) {
   const double conflict = im.lpr == 8 ? 1.0 : im.lpr == 4 ? 1.5 : im.lpr == 2 ? 2.1 : 2.8;
   // wavefronts: the entries' vectors, the lists (16 bytes per 8 entries), the row's own loads and stores
   const double wave = (double)im.padded * im.lpr / 8.0 * conflict +
                       (double)(im.list16 + im.wts16) / 8.0 + 4.0 * im.n * im.lpr / 8.0;
+  if (registers) {
+    *pipe = (double)im.padded * im.lpr / 8.0 * conflict + im.n * im.lpr / 8.0;
+    return *pipe + 400.0;
+  }
   // the longest slice is one warp's chain: about 9 cycles an entry
   const double chain = 9.0 * im.longest + 60.0;
   *pipe = wave;

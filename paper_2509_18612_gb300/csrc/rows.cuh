@@ -45,12 +45,18 @@ void rows_measure(const int32_t* row_ptr, const float* w, int wmode, int32_t row
 void rows_build(const int32_t* row_ptr, const int32_t* col, const float* w, int wmode, int32_t row0, int32_t n,
                 int lpr, RowsImage* im, std::vector<uint32_t>* words);
 int rows_image(deco_graph* g, int lpr, const RowsImage** out);   // built once and kept with the graph
-// cycles of one step of one CTA that has its SM to itself, and the shared-memory cycles among them
-double rows_cycles(const RowsImage& im, double* pipe);
+// cycles of one step of one CTA that has its SM to itself, and the shared-memory cycles among them; registers: of the
+// form with a row's data in registers
+double rows_cycles(const RowsImage& im, bool registers, double* pipe);
 int rows_threads(int32_t n, int lpr);
 // threads of an SM: 1024 leave 64 registers, enough but for 8 columns with their own step sizes and budgets
 constexpr int rows_max_threads(int prec, bool percol) { return prec == DECO_PREC_BF16 && percol ? 512 : 1024; }
 RowsGraph rows_graph(const RowsImage& im);
 int launch_rows(const RowsParams& p, int n_items, int prec, int wmode, cudaStream_t st);
+// the form with a row's data in registers (rows_reg.cu): one graph, a slice per warp, at most 32 entries a row, no
+// general weights, the same step size and budget for every column
+bool rows_reg_fits(const RowsImage& im, int wmode);
+size_t rows_reg_smem_bytes(const RowsImage& im);
+int launch_rows_reg(const RowsParams& p, const RowsImage& im, int n_items, int prec, int wmode, cudaStream_t st);
 
 }  // namespace deco
