@@ -229,6 +229,7 @@ struct StepLaunch {
   const int32_t* steps_cols;
   int32_t t;
   int32_t* flag;
+  bool overlap = false; // may start while the kernel before it on the stream, the step that wrote yin, still runs
 };
 int launch_step_global(const StepLaunch& s, cudaStream_t st);
 // The pipelined form of the same step (bit-identical iterates): the shape

@@ -84,10 +84,10 @@ static double rows_step_cycles(const RowsImage& im, int prec, int wmode, int ite
   const int share = std::min(per_sm, (items + sms - 1) / sms);
   return waves * std::max(alone, share * pipe + 350.0);
 }
-// one launch of the per-step kernel: the launch (4.6 - 6.3 us a step for graphs of 1 400 - 5 000 rows and 8 columns),
-// and its gathers at ~4.5 TB/s
+// one launch of the per-step kernel: the launch (4.2 us a step for 5 000 rows and 8 columns), and its gathers at
+// ~4.5 TB/s
 static double step_cycles(const deco_graph* g, int32_t C, int prec) {
-  return 9000.0 + (double)g->nnz * C * (prec == DECO_PREC_BF16 ? 2.0 : 4.0) / 4.5e12 * 2.07e9;
+  return 8000.0 + (double)g->nnz * C * (prec == DECO_PREC_BF16 ? 2.0 : 4.0) / 4.5e12 * 2.07e9;
 }
 
 bool valid_selector(int kernel) {
@@ -504,6 +504,9 @@ int PhaseRunner::run(void* y[2], int& cur, float* v, int32_t steps, int objectiv
   sl.dnet = g->dnet;
   sl.v = v; sl.alpha = alpha; sl.mu = mu;
   sl.alpha_cols = alpha_cols; sl.steps_cols = steps_cols; sl.flag = flag;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  if (cudaError_t e = cudaStreamIsCapturing(st, &capture)) return cuda_fail(e, "cudaStreamIsCapturing");
+  const bool overlap = capture == cudaStreamCaptureStatusNone;
   if (plan.col_slabs > 1 && steps > 0) {
     // Column-slab schedule: copy the block into S dense n x w slabs, run all
     // steps of one slab before the next (a narrow dense slab and the CSR stay
@@ -544,6 +547,7 @@ int PhaseRunner::run(void* y[2], int& cur, float* v, int32_t steps, int objectiv
         sl.yin = blk[c];
         sl.yout = blk[c ^ 1];
         sl.t = t;
+        sl.overlap = overlap && t > 0;
         if ((rc = step_launch(sl, st))) return rc;
         c ^= 1;
       }
@@ -558,6 +562,7 @@ int PhaseRunner::run(void* y[2], int& cur, float* v, int32_t steps, int objectiv
     sl.yin = y[cur];
     sl.yout = y[cur ^ 1];
     sl.t = t;
+    sl.overlap = overlap && t > 0;
     int rc = step_launch(sl, st);
     if (rc) return rc;
     cur ^= 1;

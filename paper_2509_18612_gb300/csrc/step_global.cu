@@ -21,16 +21,16 @@
 // past L2 (evict-first); the sums of +-1 and unit graphs in 16 bits by
 // mixed-precision adds.  us per step, before and after:
 //   n        degree  C    precision  weights   momentum
-//   200 003  12      100  FP32       general   0.9       195 -> 178
-//   200 003  12      128  BF16       unit      0          97 ->  75
-//   200 003  12      128  BF16       unit      0.9       127 -> 105
-//   200 003  12       60  FP32       unit      0          80 ->  69
-//   10^6      8      128  BF16       unit      0         531 -> 365
-//   10^6     10       64  FP32       unit      0.9       535 -> 464
-//   10^6      8       20  FP32       unit      0         248 -> 189
-// Eight gathers in flight without momentum: 79 and 380 us on the second and
-// fifth; a loop over rows with the next row's indices prefetched: 136 and 649
-// (24 warps an SM).
+//   200 003  12      100  FP32       general   0.9       195 -> 169
+//   200 003  12      128  BF16       unit      0          97 ->  64
+//   200 003  12      128  BF16       unit      0.9       127 ->  97
+//   200 003  12       60  FP32       unit      0          80 ->  54
+//   10^6      8      128  BF16       unit      0         531 -> 352
+//   10^6     10       64  FP32       unit      0.9       535 -> 451
+//   10^6      8       20  FP32       unit      0         248 -> 176
+// Eight gathers in flight without momentum cost 5 % on the second and fifth; a
+// loop over rows with the next row's indices prefetched took 136 and 649 us
+// (24 warps an SM); indices held a chunk ahead spill.
 #include <algorithm>
 
 #include "deco_internal.cuh"
@@ -59,12 +59,12 @@ struct KArgs {
   int32_t* flag;
 };
 
-// Gathers in flight per lane, and blocks per SM (registers): more of both at once does not fit.  Momentum in FP32 is
-// the exception where more gathers win over more warps (464 against 491 us on the sixth graph above).
-template <int PREC, bool MOM>
+// Gathers in flight per lane, and blocks per SM (registers): more of both at once does not fit.  With momentum more
+// gathers win over more warps (by 6 % on the sixth graph above; 206 319 nodes, 9 columns, 16-bit 31 against 26 us).
+template <bool MOM>
 struct Shape {
-  static constexpr int U = MOM && PREC == DECO_PREC_FP32 ? 8 : 4;
-  static constexpr int BLOCKS = !MOM ? 6 : PREC == DECO_PREC_FP32 ? 4 : 5;
+  static constexpr int U = MOM ? 8 : 4;
+  static constexpr int BLOCKS = MOM ? 4 : 6;
 };
 
 __device__ __forceinline__ void unpack(const uint4 q, float (&v)[4]) {
@@ -96,21 +96,39 @@ __device__ __forceinline__ void add_entry(float (&acc)[VN], uint4 q, uint32_t x,
   }
 }
 
-template <int PREC, int WMODE, bool MOM, bool LAP>
-__global__ void __launch_bounds__(256, Shape<PREC, MOM>::BLOCKS) k_step_global(const __grid_constant__ KArgs a) {
+// OVERLAP: launched to start while the step before it still runs (programmatic dependent launch).  It then reads the
+// graph ahead of waiting for that step, and the block by plain loads, since others still write it when this kernel
+// starts.  Saves the launch gap of the smaller steps; on large ones the wait ahead of the own row's loads costs 1 - 5 %.
+// us per step without and with: 8 000 nodes, degree 20, 128 columns, FP32 11.2 / 8.8; 5 000, degree 3, 8 columns 5.1 /
+// 4.2; 200 003, degree 12, 60 columns 62 / 54, 100 columns with momentum and general weights 169 / 174.
+template <int PREC, int WMODE, bool MOM, bool LAP, bool OVERLAP>
+__global__ void __launch_bounds__(256, Shape<MOM>::BLOCKS) k_step_global(const __grid_constant__ KArgs a) {
   using V = VecT<PREC>;
-  constexpr int VN = V::N, U = Shape<PREC, MOM>::U;
+  constexpr int VN = V::N, U = Shape<MOM>::U;
+  if (OVERLAP) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the next step's blocks may be placed
   const int gl = threadIdx.x & (a.G - 1);         // lane within the group
   const int64_t row = ((int64_t)blockIdx.x << (8 - a.lg)) + (threadIdx.x >> a.lg);
   const int32_t c0 = ((a.ch0 + (int32_t)blockIdx.y) * a.G + gl) * VN;   // first column of this lane
   if (row >= a.n || c0 >= a.C) return;
   const int32_t r = (int32_t)row;
 
+  const uint32_t* const col = WMODE == W_SIGN ? a.col_sw : reinterpret_cast<const uint32_t*>(a.col_idx);
   const int32_t e1 = __ldg(a.row_ptr + r + 1);
   int32_t e = __ldg(a.row_ptr + r);
+  if (OVERLAP) {
+    if (e < e1) {
+      asm volatile("prefetch.global.L1 [%0];" ::"l"(col + e));
+      if (WMODE == W_GENERAL) asm volatile("prefetch.global.L1 [%0];" ::"l"(a.w + e));
+    }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+  }
+  auto vector = [](const char* at) {
+    const uint4* const q = reinterpret_cast<const uint4*>(at);
+    return OVERLAP ? *q : __ldg(q);
+  };
   // own row and momentum ahead of the gathers, which hide their latency
   const size_t base = (size_t)r * a.ld + c0;
-  const uint4 own = __ldg(reinterpret_cast<const uint4*>(static_cast<const char*>(a.yin) + base * (16 / VN)));
+  const uint4 own = vector(static_cast<const char*>(a.yin) + base * (16 / VN));
   float vv[VN];
   if (MOM) {
 #pragma unroll
@@ -122,10 +140,7 @@ __global__ void __launch_bounds__(256, Shape<PREC, MOM>::BLOCKS) k_step_global(c
   const float dr = LAP ? __ldg(a.dnet + r) : 0.0f;
   const char* const yb = static_cast<const char*>(a.yin) + (size_t)c0 * (16 / VN);
   const uint32_t row_bytes = (uint32_t)a.ld * (16 / VN);
-  const uint32_t* const col = WMODE == W_SIGN ? a.col_sw : reinterpret_cast<const uint32_t*>(a.col_idx);
-  auto gather = [&](uint32_t x) {
-    return __ldg(reinterpret_cast<const uint4*>(yb + (size_t)(WMODE == W_SIGN ? x & 0x7FFFFFFFu : x) * row_bytes));
-  };
+  auto gather = [&](uint32_t x) { return vector(yb + (size_t)(WMODE == W_SIGN ? x & 0x7FFFFFFFu : x) * row_bytes); };
 
   float acc[VN];
 #pragma unroll
@@ -161,13 +176,13 @@ __global__ void __launch_bounds__(256, Shape<PREC, MOM>::BLOCKS) k_step_global(c
   unpack(own, y);
   bool bad = false;
   const bool whole = c0 + VN <= a.C;
-  if (whole && !a.alpha_cols && !a.steps_cols) {
+  if (!a.alpha_cols && !a.steps_cols) {   // the same for the warp; columns past C are not stored
 #pragma unroll
     for (int k = 0; k < VN; ++k) {
       const float grad = LAP ? fmaf(dr, y[k], -acc[k]) : -acc[k];
       if (MOM) vv[k] = fmaf(a.mu, vv[k], grad);
       const float yn = fmaf(a.alpha_eff, MOM ? vv[k] : grad, y[k]);
-      bad = bad || !isfinite(yn);
+      bad = bad || (!isfinite(yn) && (whole || c0 + k < a.C));
       out[k] = fminf(fmaxf(yn, -1.0f), 1.0f);
     }
   } else {
@@ -205,22 +220,41 @@ __global__ void __launch_bounds__(256, Shape<PREC, MOM>::BLOCKS) k_step_global(c
   if (bad && a.flag) atomicExch(a.flag, 1);
 }
 
+void launch_k(void (*fn)(const KArgs), const KArgs& a, bool overlap, dim3 grid, cudaStream_t st) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(256, 1, 1);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = overlap ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, fn, a);   // the caller reads the error
+}
+
+template <int PREC, int WMODE, bool MOM, bool LAP>
+void launch_o(const KArgs& a, bool overlap, dim3 grid, cudaStream_t st) {
+  if (overlap) launch_k(k_step_global<PREC, WMODE, MOM, LAP, true>, a, true, grid, st);
+  else launch_k(k_step_global<PREC, WMODE, MOM, LAP, false>, a, false, grid, st);
+}
+
 template <int PREC, int WMODE>
-void launch_w(const KArgs& a, bool mom, bool lap, dim3 grid, cudaStream_t st) {
+void launch_w(const KArgs& a, bool mom, bool lap, bool overlap, dim3 grid, cudaStream_t st) {
   if (mom) {
-    if (lap) k_step_global<PREC, WMODE, true, true><<<grid, 256, 0, st>>>(a);
-    else k_step_global<PREC, WMODE, true, false><<<grid, 256, 0, st>>>(a);
+    if (lap) launch_o<PREC, WMODE, true, true>(a, overlap, grid, st);
+    else launch_o<PREC, WMODE, true, false>(a, overlap, grid, st);
   } else {
-    if (lap) k_step_global<PREC, WMODE, false, true><<<grid, 256, 0, st>>>(a);
-    else k_step_global<PREC, WMODE, false, false><<<grid, 256, 0, st>>>(a);
+    if (lap) launch_o<PREC, WMODE, false, true>(a, overlap, grid, st);
+    else launch_o<PREC, WMODE, false, false>(a, overlap, grid, st);
   }
 }
 
 template <int PREC>
-void launch_p(const KArgs& a, int wmode, bool mom, bool lap, dim3 grid, cudaStream_t st) {
-  if (wmode == W_UNIT) launch_w<PREC, W_UNIT>(a, mom, lap, grid, st);
-  else if (wmode == W_SIGN) launch_w<PREC, W_SIGN>(a, mom, lap, grid, st);
-  else launch_w<PREC, W_GENERAL>(a, mom, lap, grid, st);
+void launch_p(const KArgs& a, int wmode, bool mom, bool lap, bool overlap, dim3 grid, cudaStream_t st) {
+  if (wmode == W_UNIT) launch_w<PREC, W_UNIT>(a, mom, lap, overlap, grid, st);
+  else if (wmode == W_SIGN) launch_w<PREC, W_SIGN>(a, mom, lap, overlap, grid, st);
+  else launch_w<PREC, W_GENERAL>(a, mom, lap, overlap, grid, st);
 }
 
 }  // namespace
@@ -255,11 +289,14 @@ int launch_step_global(const StepLaunch& s, cudaStream_t st) {
   const bool mom = s.mu != 0.0f;
   const bool lap = s.objective == DECO_OBJ_LAPLACIAN;
   const int32_t nchunks = (nvec + G - 1) / G;
+  // steps of up to 64 MB of block and momentum (10 - 70 us): the gap between two launches is worth the wait
+  const bool overlap = s.overlap && nchunks <= 65535 &&
+                       (int64_t)s.n * s.C * ((s.precision == DECO_PREC_BF16 ? 2 : 4) + (mom ? 8 : 0)) <= (64 << 20);
   const unsigned rows = (unsigned)(((int64_t)s.n * G + 255) / 256);
   for (a.ch0 = 0; a.ch0 < nchunks; a.ch0 += 65535) {
     const dim3 grid(rows, (unsigned)std::min(nchunks - a.ch0, 65535));
-    if (s.precision == DECO_PREC_BF16) launch_p<DECO_PREC_BF16>(a, s.wmode, mom, lap, grid, st);
-    else launch_p<DECO_PREC_FP32>(a, s.wmode, mom, lap, grid, st);
+    if (s.precision == DECO_PREC_BF16) launch_p<DECO_PREC_BF16>(a, s.wmode, mom, lap, overlap, grid, st);
+    else launch_p<DECO_PREC_FP32>(a, s.wmode, mom, lap, overlap, grid, st);
     DECO_CUDA_TRY(cudaGetLastError());
   }
   return DECO_OK;

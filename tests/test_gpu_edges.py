@@ -276,3 +276,39 @@ def test_scratch_pool_takes_back_what_calls_used_on_two_streams():
     for _ in range(3):
         deco.deco_run_phase(G, C, C, blocks[2], None, 9, args, deco.DECO_KERNEL_GLOBAL)
     assert torch.equal(blocks[0], blocks[2]) and torch.equal(blocks[1], blocks[2])
+
+
+# Steps small enough to start while the step before still runs, against single steps with the stream drained between
+# them; a second program on another stream at the same time.
+@pytest.mark.parametrize("n,degree,C,weights", [(1, 0.0, 8, None), (5000, 3.0, 8, None), (9001, 11.0, 37, "sign"),
+                                                (20011, 6.0, 130, "weights")])
+@pytest.mark.parametrize("precision", [deco.DECO_PREC_FP32, deco.DECO_PREC_BF16])
+@pytest.mark.parametrize("mu", [0.0, 0.9])
+def test_overlapping_steps_equal_single_steps(n, degree, C, weights, precision, mu):
+    g = gg.er_graph_avg_degree(n, degree, 3) if n > 1 else gg.from_edges(1, [], [])
+    if weights:
+        u, v, _ = g.edges()
+        choices = [-1.0, 1.0] if weights == "sign" else [-3.0, 2.0, 7.0]
+        g = gg.from_edges(g.n, u, v, np.random.default_rng(1).choice(np.array(choices), size=u.size))
+    G = deco.graph_from(g)
+    ld = (C + 63) // 64 * 64
+    dtype = torch.bfloat16 if precision else torch.float32
+    y0 = ((torch.rand(n, ld, device=DEV) * 2 - 1) * 0.3).to(dtype)
+    args = deco.step_args(0, precision, 0.004, mu)
+    T = 41
+    a, b = y0.clone(), y0.clone()
+    v = torch.zeros(n, ld, device=DEV)
+    for _ in range(T):
+        deco.deco_step(G, C, ld, a, b, v if mu else None, args)
+        torch.cuda.synchronize()
+        a, b = b, a
+    other = torch.cuda.Stream()
+    y, w = y0.clone(), torch.zeros(n, ld, device=DEV)
+    y2, w2 = y0.clone(), torch.zeros(n, ld, device=DEV)
+    torch.cuda.synchronize()
+    deco.deco_run_phase(G, C, ld, y, w if mu else None, T, args, deco.DECO_KERNEL_GLOBAL)
+    deco.deco_run_phase(G, C, ld, y2, w2 if mu else None, T, args, deco.DECO_KERNEL_GLOBAL, stream=other.cuda_stream)
+    torch.cuda.synchronize()
+    assert torch.equal(y[:, :C], a[:, :C]) and torch.equal(y2[:, :C], a[:, :C])
+    if mu:
+        assert torch.equal(w[:, :C], v[:, :C]) and torch.equal(w2[:, :C], v[:, :C])
