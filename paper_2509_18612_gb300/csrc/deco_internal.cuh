@@ -145,6 +145,7 @@ struct deco_graph {
   // host-side facts (degree statistics for IDI / DUI)
   int64_t deg_s1 = 0, deg_s2 = 0;
   int32_t max_deg = 0;
+  int32_t max_row_abs = 0;      // largest sum of |w| over a row
   std::vector<int32_t> h_row_ptr;   // host copy (row splits of the on-chip kernel)
   std::vector<int32_t> h_col;       // host copy of the device edge order
   std::vector<float> h_w;           // host copy of the device-order weights (or empty)

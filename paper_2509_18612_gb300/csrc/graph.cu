@@ -234,7 +234,7 @@ int deco::create_graph_impl(int32_t n, int64_t nnz, const int32_t* row_ptr, cons
   {
     // degrees, their sums and maximum, net weighted degrees; per thread, then
     // combined in thread order (integer sums: the same totals in any order)
-    struct Part { int64_t s1 = 0, s2 = 0; int32_t maxd = 0, bad = -1; double sabs = 0.0; };
+    struct Part { int64_t s1 = 0, s2 = 0; int32_t maxd = 0, bad = -1, max_sabs = 0; double sabs = 0.0; };
     std::vector<Part> part(std::max<unsigned>(1, std::thread::hardware_concurrency()));
     const int nt = host_parallel(n, nnz, [&](int t, int64_t r0, int64_t r1) {
       Part& P = part[t];
@@ -249,6 +249,7 @@ int deco::create_graph_impl(int32_t n, int64_t nnz, const int32_t* row_ptr, cons
           sabs += weights ? std::fabs(weights[e]) : 1.0;
         }
         if (sabs > 16777216.0 && P.bad < 0) { P.bad = v; P.sabs = sabs; }
+        P.max_sabs = std::max(P.max_sabs, (int32_t)std::min(sabs, 16777216.0));
         dnet[v] = (float)s;   // integral and |s| <= 2^24: exact in FP32
       }
     });
@@ -262,6 +263,7 @@ int deco::create_graph_impl(int32_t n, int64_t nnz, const int32_t* row_ptr, cons
       g->deg_s1 += part[t].s1;
       g->deg_s2 += part[t].s2;
       g->max_deg = std::max(g->max_deg, part[t].maxd);
+      g->max_row_abs = std::max(g->max_row_abs, part[t].max_sabs);
     }
   }
 

@@ -2,8 +2,7 @@
 // output h = tanh(o) in (-1,1)^n becomes the mean of the Gaussian starts of
 // the solver (Sec. 4.2's "Gaussian around a mean vector", with a learned mean
 // instead of IDI).  Inference, loss, backward pass and Adam run in these
-// kernels; the neighbour aggregation uses the same CSR gather as the
-// projected-gradient step (spmm.cuh).
+// kernels; the neighbour aggregation is the CSR gather of spmm.cuh.
 //
 //   X  = node features [d/Delta, d/mean(d), 1/sqrt(d+1), 5 x U(-1,1)]   (n x 8)
 //   H0 = relu(X W0 + b0)

@@ -19,6 +19,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "api_util.cuh"
 #include "deco_internal.cuh"
@@ -286,11 +287,13 @@ __global__ void k_ls_flip(int32_t n, int32_t W, int32_t B, const int32_t* row_pt
   }
 }
 
-// ---- unit and +-1 weights: gains as bit planes.  A word's 32 columns are
+// ---- gains as bit planes.  A word's 32 columns are
 // worked on together: the neighbours on the side that a flip would lose are
 // counted by ripple-carry adders over bit planes (plane p holds bit p of every
 // column's count), positive gains are kept as NP planes, and two nodes' gains
-// compare in two operations a plane.  A thread owns a (row, word).
+// compare in two operations a plane.  A thread owns a (row, word).  Integral
+// weights (GEN) count an entry once for every set bit of |w|, from that bit's
+// plane up; the sum of |w| takes the degree's place.
 template <int NP>
 __device__ __forceinline__ void planes_load(const uint32_t* p, uint32_t* g) {
 #pragma unroll
@@ -315,6 +318,22 @@ __device__ __forceinline__ void ls_count(uint32_t* c, uint32_t x) {
     const uint32_t t = c[p] & x;
     c[p] ^= x;
     x = t;
+  }
+}
+
+// counts: add a to the columns of x
+template <int NP>
+__device__ __forceinline__ void ls_count_weight(uint32_t* c, uint32_t x, uint32_t a) {
+#pragma unroll
+  for (int b = 0; b < NP; ++b) {
+    if (!(a >> b)) break;
+    uint32_t y = (a >> b) & 1u ? x : 0u;
+#pragma unroll
+    for (int p = b; p < NP; ++p) {
+      const uint32_t t = c[p] & y;
+      c[p] ^= y;
+      y = t;
+    }
   }
 }
 
@@ -345,28 +364,39 @@ __device__ __forceinline__ uint32_t ls_beats(const uint32_t* gu, const uint32_t*
   return beats;
 }
 
-// col: index, or index | sign bit of a +-1 graph.  zk: the word column, row u at zk[u W].
-template <int NP>
+// col: index, or index | sign bit of a +-1 graph; wint: weights (GEN).  zk: the word column, row u at zk[u W].
+template <int NP, bool GEN>
 __device__ __forceinline__ void ls_gain_row(int32_t v, int32_t W, const int32_t* __restrict__ row_ptr,
-                                            const uint32_t* __restrict__ col, const uint32_t* zk, uint32_t cols,
-                                            uint32_t* gains) {
+                                            const uint32_t* __restrict__ col, const int32_t* __restrict__ wint,
+                                            const uint32_t* zk, uint32_t cols, uint32_t* gains) {
   const int32_t e0 = __ldg(row_ptr + v), e1 = __ldg(row_ptr + v + 1);
   const uint32_t zv = zk[(size_t)v * W];
   uint32_t c[NP], g[NP];
+  int32_t sum = GEN ? 0 : e1 - e0;
 #pragma unroll
   for (int p = 0; p < NP; ++p) c[p] = 0u;
   for (int32_t e = e0; e < e1; e += 8) {
     uint32_t u[8], x[8];
+    int32_t w[8];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) u[q] = __ldg(col + min(e + q, e1 - 1));
+    for (int q = 0; q < 8; ++q) {
+      u[q] = __ldg(col + min(e + q, e1 - 1));
+      if (GEN) w[q] = e + q < e1 ? __ldg(wint + e + q) : 0;
+    }
 #pragma unroll
     for (int q = 0; q < 8; ++q) x[q] = zk[(size_t)(u[q] & 0x7FFFFFFFu) * W];
     // columns where the entry is lost to a flip: the other side of a +1, the same side of a -1
 #pragma unroll
-    for (int q = 0; q < 8; ++q)
-      ls_count<NP>(c, e + q < e1 ? x[q] ^ zv ^ ((u[q] & 0x80000000u) ? 0xFFFFFFFFu : 0u) : 0u);
+    for (int q = 0; q < 8; ++q) {
+      if (GEN) {
+        sum += abs(w[q]);
+        ls_count_weight<NP>(c, x[q] ^ zv ^ (w[q] < 0 ? 0xFFFFFFFFu : 0u), (uint32_t)abs(w[q]));
+      } else {
+        ls_count<NP>(c, e + q < e1 ? x[q] ^ zv ^ ((u[q] & 0x80000000u) ? 0xFFFFFFFFu : 0u) : 0u);
+      }
+    }
   }
-  ls_gain<NP>(c, e1 - e0, cols, g);
+  ls_gain<NP>(c, sum, cols, g);
   planes_store<NP>(gains + (size_t)v * NP, g);
 }
 
@@ -403,7 +433,7 @@ __device__ __forceinline__ uint32_t word_columns(int32_t B, int32_t k) {
 // All rounds of one word in one cluster of LS_CLUSTER CTAs (columns are
 // independent of one another), so the word stops at its own optimum.  CTA i
 // owns a range of rows, holds their entries in shared memory (16-bit index |
-// sign) and a copy of the word's column of z and of its positive-gain masks,
+// sign, |w| in the upper half of a word with integral weights) and a copy of the word's column of z and of its positive-gain masks,
 // which the owners of the rows update in all CTAs through distributed shared
 // memory; a cluster barrier ends each half round.  Only gains of neighbours
 // that have a positive gain in a column still open are read (L2).  Bound by
@@ -415,30 +445,31 @@ constexpr int LS_CLUSTER = 8;
 struct LsSmem {
   size_t z, pos, rp, ent, total;   // byte offsets
 };
-__host__ __device__ inline LsSmem ls_smem(int32_t n, int32_t entries) {
+__host__ __device__ inline LsSmem ls_smem(int32_t n, int32_t entries, bool gen) {
   LsSmem L;
   const int32_t own = (n + LS_CLUSTER - 1) / LS_CLUSTER;
   L.z = 0;
   L.pos = L.z + (size_t)n * 4;
   L.rp = L.pos + (size_t)n * 4;
   L.ent = L.rp + (size_t)(own + 1) * 4;
-  L.total = L.ent + ((size_t)entries * 2 + 15) / 16 * 16;
+  L.total = L.ent + ((size_t)entries * (gen ? 4 : 2) + 15) / 16 * 16;
   return L;
 }
 
-template <int NP>
+template <int NP, bool GEN>
 __global__ void __cluster_dims__(LS_CLUSTER, 1, 1) __launch_bounds__(1024)
     k_ls_cluster(int32_t n, int32_t W, int32_t B, const int32_t* __restrict__ row_ptr,
-                 const uint32_t* __restrict__ col, uint32_t* zb, uint32_t* gains, int32_t max_rounds,
+                 const uint32_t* __restrict__ col, const int32_t* __restrict__ wint, uint32_t* zb, uint32_t* gains, int32_t max_rounds,
                  int32_t* changed, int32_t max_entries) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int32_t s_any[2][LS_CLUSTER];
   cg::cluster_group cluster = cg::this_cluster();
-  const LsSmem L = ls_smem(n, max_entries);
+  const LsSmem L = ls_smem(n, max_entries, GEN);
   uint32_t* const z = reinterpret_cast<uint32_t*>(smem + L.z);
   uint32_t* const pos = reinterpret_cast<uint32_t*>(smem + L.pos);
   int32_t* const rp = reinterpret_cast<int32_t*>(smem + L.rp);
-  uint16_t* const ent = reinterpret_cast<uint16_t*>(smem + L.ent);
+  using Entry = std::conditional_t<GEN, uint32_t, uint16_t>;
+  Entry* const ent = reinterpret_cast<Entry*>(smem + L.ent);
   const int rank = (int)cluster.block_rank(), tid = threadIdx.x, nt = blockDim.x;
   const int32_t k = blockIdx.x / LS_CLUSTER, own = (n + LS_CLUSTER - 1) / LS_CLUSTER;
   const int32_t ra = min(n, rank * own), rows = min(n, ra + own) - ra;
@@ -449,7 +480,12 @@ __global__ void __cluster_dims__(LS_CLUSTER, 1, 1) __launch_bounds__(1024)
   const int32_t entries = __ldg(row_ptr + ra + rows) - ebase;
   for (int32_t i = tid; i < entries; i += nt) {
     const uint32_t c = __ldg(col + ebase + i);
-    ent[i] = (uint16_t)((c & 0x7FFFu) | (c >> 31 << 15));
+    if (GEN) {
+      const int32_t w = __ldg(wint + ebase + i);
+      ent[i] = (Entry)((c & 0x7FFFu) | (w < 0 ? 0x8000u : 0u) | (uint32_t)abs(w) << 16);
+    } else {
+      ent[i] = (Entry)((c & 0x7FFFu) | (c >> 31 << 15));
+    }
   }
   for (int32_t v = tid; v < n; v += nt) z[v] = zb[(size_t)v * W + k];
   // the same word of every CTA of the cluster
@@ -463,14 +499,21 @@ __global__ void __cluster_dims__(LS_CLUSTER, 1, 1) __launch_bounds__(1024)
       const int32_t e0 = rp[i], d = rp[i + 1] - e0;
       const uint32_t zv = z[ra + i];
       uint32_t c[NP], g[NP];
+      int32_t sum = GEN ? 0 : d;
 #pragma unroll
       for (int p = 0; p < NP; ++p) c[p] = 0u;
 #pragma unroll 4
       for (int32_t e = 0; e < d; ++e) {
         const uint32_t u = ent[e0 + e];
-        ls_count<NP>(c, z[u & 0x7FFFu] ^ zv ^ ((u & 0x8000u) ? 0xFFFFFFFFu : 0u));
+        const uint32_t lost = z[u & 0x7FFFu] ^ zv ^ ((u & 0x8000u) ? 0xFFFFFFFFu : 0u);
+        if (GEN) {
+          sum += (int32_t)(u >> 16);
+          ls_count_weight<NP>(c, lost, u >> 16);
+        } else {
+          ls_count<NP>(c, lost);
+        }
       }
-      const uint32_t any = ls_gain<NP>(c, d, cols, g);
+      const uint32_t any = ls_gain<NP>(c, sum, cols, g);
       put(pos + ra + i, any);
       if (any) planes_store<NP>(gk + (size_t)(ra + i) * NP, g);
     }
@@ -517,15 +560,16 @@ __global__ void __cluster_dims__(LS_CLUSTER, 1, 1) __launch_bounds__(1024)
 }
 
 // one half round of all words per launch (graphs with more rows than a cluster covers well)
-template <int NP>
+template <int NP, bool GEN>
 __global__ void __launch_bounds__(128) k_ls_gain_planes(int32_t n, int32_t W, int32_t B,
                                                         const int32_t* __restrict__ row_ptr,
-                                                        const uint32_t* __restrict__ col, const uint32_t* zb,
+                                                        const uint32_t* __restrict__ col,
+                                                        const int32_t* __restrict__ wint, const uint32_t* zb,
                                                         uint32_t* gains, const int32_t* run) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= (int64_t)n * W || !*run) return;
   const int32_t v = (int32_t)(i % n), k = (int32_t)(i / n);
-  ls_gain_row<NP>(v, W, row_ptr, col, zb + k, word_columns(B, k), gains + (size_t)k * n * NP);
+  ls_gain_row<NP, GEN>(v, W, row_ptr, col, wint, zb + k, word_columns(B, k), gains + (size_t)k * n * NP);
 }
 template <int NP>
 __global__ void __launch_bounds__(128) k_ls_flip_planes(int32_t n, int32_t W, const int32_t* __restrict__ row_ptr,
@@ -541,13 +585,13 @@ unsigned blocks_for(int64_t threads, int per) { return (unsigned)((threads + per
 
 }  // namespace
 
-// Bit planes of a positive gain (at most the row's degree), 0: the weights or
-// the degrees do not allow them and the gains are kept as integers.
+// Bit planes of a positive gain (at most the row's sum of |w|), 0: the sums do
+// not allow them and the gains are kept as integers.
 static int ls_planes(const deco_graph* g) {
-  if (g->wmode == W_GENERAL) return 0;
-  if (g->max_deg < 16) return 4;
-  if (g->max_deg < 256) return 8;
-  return g->max_deg < 65536 ? 16 : 0;
+  const int32_t most = g->wmode == W_GENERAL ? g->max_row_abs : g->max_deg;
+  if (most < 16) return 4;
+  if (most < 256) return 8;
+  return most < 65536 ? 16 : 0;
 }
 
 size_t local_search_words(const deco_graph* g, int32_t B) {
@@ -555,7 +599,7 @@ size_t local_search_words(const deco_graph* g, int32_t B) {
   return (size_t)g->n * ((B + 31) / 32) * (np ? np : 32);
 }
 
-template <int NP>
+template <int NP, bool GEN>
 static int run_planes(const deco_graph* g, int32_t B, uint32_t* zbits, int32_t max_rounds, uint32_t* gains,
                       int32_t* changed, int64_t* kernels, cudaStream_t st) {
   const int32_t W = (B + 31) / 32, n = g->n;
@@ -566,11 +610,11 @@ static int run_planes(const deco_graph* g, int32_t B, uint32_t* zbits, int32_t m
   const int32_t own = (n + LS_CLUSTER - 1) / LS_CLUSTER;
   for (int q = 0; q < LS_CLUSTER; ++q)
     entries = std::max(entries, g->h_row_ptr[std::min(n, (q + 1) * own)] - g->h_row_ptr[std::min(n, q * own)]);
-  const size_t smem = ls_smem(n, entries).total;
+  const size_t smem = ls_smem(n, entries, GEN).total;
   if (n <= 32768 && smem + 1024 <= (size_t)slab_max_smem()) {
     const int nt = own <= 256 ? 256 : own <= 512 ? 512 : 1024;
-    DECO_CUDA_TRY(cudaFuncSetAttribute(k_ls_cluster<NP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_ls_cluster<NP><<<(unsigned)W * LS_CLUSTER, nt, smem, st>>>(n, W, B, g->row_ptr, col, zbits, gains, max_rounds,
+    DECO_CUDA_TRY(cudaFuncSetAttribute(k_ls_cluster<NP, GEN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    k_ls_cluster<NP, GEN><<<(unsigned)W * LS_CLUSTER, nt, smem, st>>>(n, W, B, g->row_ptr, col, g->wint, zbits, gains, max_rounds,
                                                                  changed, entries);
     DECO_CUDA_TRY(cudaGetLastError());
     if (kernels) *kernels += 1;
@@ -578,13 +622,21 @@ static int run_planes(const deco_graph* g, int32_t B, uint32_t* zbits, int32_t m
   }
   const int64_t threads = (int64_t)n * W;
   for (int32_t r = 0; r < max_rounds; ++r) {
-    k_ls_gain_planes<NP><<<blocks_for(threads, 128), 128, 0, st>>>(n, W, B, g->row_ptr, col, zbits, gains, changed + r);
+    k_ls_gain_planes<NP, GEN><<<blocks_for(threads, 128), 128, 0, st>>>(n, W, B, g->row_ptr, col, g->wint, zbits, gains,
+                                                                        changed + r);
     k_ls_flip_planes<NP><<<blocks_for(threads, 128), 128, 0, st>>>(n, W, g->row_ptr, col, gains, zbits, changed + r,
                                                                    changed + r + 1);
   }
   DECO_CUDA_TRY(cudaGetLastError());
   if (kernels) *kernels += 2 * (int64_t)max_rounds;
   return DECO_OK;
+}
+
+template <int NP>
+static int run_weights(const deco_graph* g, int32_t B, uint32_t* zbits, int32_t max_rounds, uint32_t* gains,
+                       int32_t* changed, int64_t* kernels, cudaStream_t st) {
+  return g->wmode == W_GENERAL ? run_planes<NP, true>(g, B, zbits, max_rounds, gains, changed, kernels, st)
+                               : run_planes<NP, false>(g, B, zbits, max_rounds, gains, changed, kernels, st);
 }
 
 // The rounds of the local search on bit-packed columns (stream-ordered).
@@ -597,9 +649,9 @@ int launch_local_search(const deco_graph* g, int32_t B, uint32_t* zbits, int32_t
   DECO_CUDA_TRY(cudaMemsetAsync(changed, 0, sizeof(int32_t) * (size_t)(max_rounds + 1), st));
   DECO_CUDA_TRY(cudaMemsetAsync(changed, 1, sizeof(int32_t), st));   // round 0 runs (any nonzero word)
   switch (ls_planes(g)) {
-    case 4: return run_planes<4>(g, B, zbits, max_rounds, gains, changed, kernels, st);
-    case 8: return run_planes<8>(g, B, zbits, max_rounds, gains, changed, kernels, st);
-    case 16: return run_planes<16>(g, B, zbits, max_rounds, gains, changed, kernels, st);
+    case 4: return run_weights<4>(g, B, zbits, max_rounds, gains, changed, kernels, st);
+    case 8: return run_weights<8>(g, B, zbits, max_rounds, gains, changed, kernels, st);
+    case 16: return run_weights<16>(g, B, zbits, max_rounds, gains, changed, kernels, st);
     default: break;
   }
   const int64_t threads = (int64_t)g->n * W;

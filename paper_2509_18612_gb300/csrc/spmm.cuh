@@ -1,6 +1,6 @@
-// CSR gather (one row of A Y for one lane's 16-byte vector of columns),
-// shared by the projected-gradient step kernel and the message-passing
-// aggregation of the learned proposal.
+// 16-byte vectors of the iterate (the per-step kernels), and the CSR gather
+// (one row of A Y for one lane's vector of columns) of the learned proposal's
+// message passing.
 #pragma once
 
 #include "deco_internal.cuh"

@@ -197,12 +197,17 @@ SEARCH_GRAPHS = {
     "several rows per thread": lambda: gg.er_graph_avg_degree(20000, 6.0, 4),
     "a launch per half round": lambda: gg.er_graph_avg_degree(33000, 5.0, 5),
     "launches, signed": lambda: _sign(gg.er_graph_avg_degree(33000, 5.0, 6)),
+    "weights (4 planes)": lambda: signed_graph(12, 0.5, 3, (1.0, -2.0)),
+    "weights (8 planes)": lambda: signed_graph(700, 0.02, 4, (-7.0, 3.0, 5.0, 1.0)),
+    "weights (16 planes)": lambda: signed_graph(300, 0.1, 5, (-300.0, 150.0, 77.0)),
+    "weights (integers)": lambda: signed_graph(200, 0.1, 6, (-30000.0, 15000.0, 9999.0)),
+    "launches, weights": lambda: _sign(gg.er_graph_avg_degree(33000, 5.0, 7), [-3.0, 2.0, 6.0]),
 }
 
 
-def _sign(g):
+def _sign(g, choices=(-1.0, 1.0)):
     u, v, _ = g.edges()
-    return gg.from_edges(g.n, u, v, np.random.default_rng(g.n).choice([-1.0, 1.0], size=u.size))
+    return gg.from_edges(g.n, u, v, np.random.default_rng(g.n).choice(choices, size=u.size))
 
 
 @pytest.mark.parametrize("name", list(SEARCH_GRAPHS))
