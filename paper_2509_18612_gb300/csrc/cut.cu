@@ -5,13 +5,15 @@
 //          16-byte vectors and writes 8 bits; blocks whose rows are not
 //          16-byte aligned, and lifts above 4, take one warp per (row, 32
 //          starting points) and a ballot.
-//  cut:    warps take equal ranges of the stored entries, a lane per entry:
-//          the words z_v xor z_u of 32 entries form a 32 x 32 bit matrix that
-//          the warp transposes, so that lane b counts starting point b with
-//          one popc (weights: one per bit of |w| and sign).  Entries with
-//          u > v count (each unordered edge once), in integers; the block
-//          reduces and issues one 64-bit atomic per starting point.  Integer
-//          sums are exact in any order.
+//  cut:    warps take equal ranges of the stored entries, a lane per entry.
+//          Without weights a lane counts its entries' words z_v xor z_u in bit
+//          planes (carry-save adders); now and then the warp transposes the
+//          planes, 32 x 32 bits each, and lane b adds starting point b's bits
+//          with one popc a plane.  With weights the words of 32 entries are
+//          transposed themselves, and lane b takes one popc per bit of |w| and
+//          sign.  Entries with u > v count (each unordered edge once), in
+//          integers; the block reduces and issues one 64-bit atomic per
+//          starting point.  Integer sums are exact in any order.
 //  argmax: one block; lowest index among the maximal cuts.
 #include <algorithm>
 
@@ -57,16 +59,19 @@ __global__ void k_pack(int32_t n, int32_t B, int32_t lift, int32_t ld, int32_t W
 // Byte q of row v: starting points 8q ... 8q + 7, i.e. columns 8 q LIFT ... of
 // the row, 16-byte aligned (ld % 8 == 0).  A vector may reach past column C
 // but not past ld; points >= B give 0.  Bound by HBM: 10^6 rows of 128 BF16
-// columns in 64 us (4.2 TB/s); a warp per word, 2 bytes a lane, took 456.
+// columns in 56 us (4.8 TB/s; 64 with 64-bit divisions); a warp per word, 2
+// bytes a lane, took 456.
 template <int PREC, int LIFT>
 __global__ void __launch_bounds__(256) k_pack_vec(int32_t n, int32_t B, int32_t ld, int32_t W, const void* y,
                                                   uint8_t* zbytes) {
   constexpr int VN = PREC == DECO_PREC_BF16 ? 8 : 4;    // values of a vector
   constexpr int NV = 8 * LIFT / VN;                     // vectors of 8 points
   const int64_t total = (int64_t)n * W * 4, step = (int64_t)gridDim.x * blockDim.x;
-  const int32_t W4 = W * 4;
+  const uint32_t W4 = (uint32_t)W * 4u;
+  const bool small = total < (int64_t)1 << 31;          // 32-bit divisions: a 64-bit one costs more than the rounding
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += step) {
-    const int32_t v = (int32_t)(i / W4), q = (int32_t)(i % W4);
+    const int32_t v = small ? (int32_t)((uint32_t)i / W4) : (int32_t)(i / W4);
+    const int32_t q = (int32_t)(i - (int64_t)v * W4);
     uint32_t bits = 0;
     const int32_t c0 = 8 * q * LIFT;
     const uint4* src = reinterpret_cast<const uint4*>(static_cast<const char*>(y) +
@@ -98,8 +103,9 @@ __global__ void __launch_bounds__(256) k_pack_vec(int32_t n, int32_t B, int32_t 
         for (int l = 0; l < LIFT; ++l) s += val[k * LIFT + l];
         bit = s >= 0.0f;                                 // Eq. 11: non-strict
       }
-      if (bit && 8 * q + k < B) bits |= 1u << k;
+      if (bit) bits |= 1u << k;
     }
+    if (8 * q + 8 > B) bits &= 8 * q < B ? (1u << (B - 8 * q)) - 1u : 0u;   // points below B
     zbytes[i] = (uint8_t)bits;
   }
 }
@@ -128,19 +134,21 @@ __device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
 }
 
 constexpr int CUT_BLOCK = 256;
-constexpr int CUT_U = 2;   // batches of 32 entries in flight per warp
+constexpr int cut_batches(bool wt) { return wt ? 2 : 4; }   // batches of 32 entries in flight per warp
+constexpr int CUT_PLANES = 5;                               // a lane's counts below 32
 
 // Cuts of the starting points of V words (word group blockIdx.y) over the
 // rows of graph blockIdx.z (goff: first rows; null: all n rows), added to
-// cuts[graph B + b].  Bound by the latency of the gathered words and the
-// transposes' issue slots: 10^6 nodes, degree 10, 128 starting points in
-// 108 us; a warp per row that walked its neighbours one by one took 1 059.
+// cuts[graph B + b].  Bound by the latency of the gathered words and by issue
+// slots: 10^6 nodes, degree 10, 128 starting points in 69 us; every entry's
+// words transposed 109, a warp per row that walked its neighbours 1 059.
 template <int V, bool WT>
-__global__ void __launch_bounds__(CUT_BLOCK) k_cut(int32_t n, int32_t B, int32_t W, const int32_t* __restrict__ row_ptr,
+__global__ void __launch_bounds__(CUT_BLOCK, 4) k_cut(int32_t n, int32_t B, int32_t W, const int32_t* __restrict__ row_ptr,
                                                    const int32_t* __restrict__ col_idx, const int32_t* __restrict__ wint,
                                                    int wbits, const uint32_t* __restrict__ zbits,
                                                    const int32_t* __restrict__ goff, int64_t* cuts) {
   __shared__ long long part[CUT_BLOCK / 32][32 * V];
+  constexpr int CUT_U = cut_batches(WT);
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int32_t k0 = blockIdx.y * V, g = blockIdx.z;
   const int32_t ra = goff ? __ldg(goff + g) : 0, rb = goff ? __ldg(goff + g + 1) : n;
@@ -152,6 +160,18 @@ __global__ void __launch_bounds__(CUT_BLOCK) k_cut(int32_t n, int32_t B, int32_t
   long long acc[V];
 #pragma unroll
   for (int j = 0; j < V; ++j) acc[j] = 0;
+  uint32_t plane[V][CUT_PLANES] = {};
+  int held = 0;            // entries a lane may have counted since the planes were last emptied
+  auto empty_planes = [&]() {
+#pragma unroll
+    for (int j = 0; j < V; ++j)
+#pragma unroll
+      for (int p = 0; p < CUT_PLANES; ++p) {
+        acc[j] += (long long)__popc(transpose32(plane[j][p], lane)) << p;
+        plane[j][p] = 0u;
+      }
+    held = 0;
+  };
   if (e < E1) {
     // the row that holds entry e: row_ptr[r] <= e < row_ptr[r + 1]
     int32_t lo = ra, hi = rb;
@@ -213,14 +233,31 @@ __global__ void __launch_bounds__(CUT_BLOCK) k_cut(int32_t n, int32_t B, int32_t
             }
           }
         }
+        if constexpr (!WT) {
 #pragma unroll
-        for (int q = 0; q < CUT_U; ++q) {
+          for (int j = 0; j < V; ++j) {
+            uint32_t* const c = plane[j];
+            const uint32_t d0 = d[0][j], d1 = d[1][j], d2 = d[2 % CUT_U][j], d3 = d[3 % CUT_U][j];
+            const uint32_t t0 = (c[0] & d0) | (c[0] & d1) | (d0 & d1);
+            c[0] ^= d0 ^ d1;
+            const uint32_t t1 = (c[0] & d2) | (c[0] & d3) | (d2 & d3);
+            c[0] ^= d2 ^ d3;
+            uint32_t carry = (c[1] & t0) | (c[1] & t1) | (t0 & t1);
+            c[1] ^= t0 ^ t1;
 #pragma unroll
-          for (int j = 0; j < V; ++j) d[q][j] = transpose32(d[q][j], lane);
-          if (!WT) {
+            for (int p = 2; p < CUT_PLANES; ++p) {
+              const uint32_t t = c[p] & carry;
+              c[p] ^= carry;
+              carry = t;
+            }
+          }
+          held += CUT_U;
+          if (held + CUT_U >= 1 << CUT_PLANES) empty_planes();
+        } else {
 #pragma unroll
-            for (int j = 0; j < V; ++j) acc[j] += __popc(d[q][j]);
-          } else {
+          for (int q = 0; q < CUT_U; ++q) {
+#pragma unroll
+            for (int j = 0; j < V; ++j) d[q][j] = transpose32(d[q][j], lane);
             for (int h = 0; h < wbits; ++h) {
               const uint32_t pos = __ballot_sync(0xFFFFFFFFu, w[q] > 0 && ((w[q] >> h) & 1));
               const uint32_t neg = __ballot_sync(0xFFFFFFFFu, w[q] < 0 && ((-w[q] >> h) & 1));
@@ -233,6 +270,7 @@ __global__ void __launch_bounds__(CUT_BLOCK) k_cut(int32_t n, int32_t B, int32_t
       }
       e = lim;
     }
+    if (!WT && held) empty_planes();
   }
 #pragma unroll
   for (int j = 0; j < V; ++j) part[wib][32 * j + lane] = acc[j];

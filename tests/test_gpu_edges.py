@@ -312,3 +312,23 @@ def test_overlapping_steps_equal_single_steps(n, degree, C, weights, precision, 
     assert torch.equal(y[:, :C], a[:, :C]) and torch.equal(y2[:, :C], a[:, :C])
     if mu:
         assert torch.equal(w[:, :C], v[:, :C]) and torch.equal(w2[:, :C], v[:, :C])
+
+
+# Cuts by bit planes: entry ranges that empty a lane's planes often, once or never; hub rows and ragged words.
+@pytest.mark.parametrize("name", ["dense", "hub", "sparse"])
+@pytest.mark.parametrize("B", [1, 33, 64, 97, 128, 200])
+def test_cuts_by_bit_planes_match_oracle(name, B):
+    if name == "dense":
+        g = gg.er_graph(900, 0.9, 2)
+    elif name == "hub":
+        u = np.arange(1, 4001)
+        g = gg.from_edges(4001, np.zeros(4000, np.int64), u)
+    else:
+        g = gg.er_graph_avg_degree(70001, 9.0, 4)
+    Z = (np.random.default_rng(B).random((g.n, B)) < 0.5).astype(np.uint8)
+    Z[:, 0] = 0
+    if B > 1:
+        Z[:, 1] = (np.arange(g.n) > 0)   # every entry of the hub is cut
+    cuts = torch.zeros(B, dtype=torch.int64, device=DEV)
+    deco.deco_eval_cuts(deco.graph_from(g), B, torch.from_numpy(Z.reshape(-1)).to(DEV), cuts)
+    np.testing.assert_array_equal(cuts.cpu().numpy(), O.cut_values(g, Z))
