@@ -74,7 +74,7 @@ extern "C" int deco_step(const deco_graph* g, int32_t C, int32_t ld, const void*
   if (y_in == y_out) { set_error("y_out must not alias y_in"); return DECO_ERR_ARG; }
   if (a->momentum != 0.0f && !v) { set_error("momentum needs the v buffer"); return DECO_ERR_ARG; }
   StepLaunch s{};
-  s.n = g->n; s.C = C; s.ld = ld;
+  s.n = g->n; s.nnz = g->nnz; s.C = C; s.ld = ld;
   s.precision = a->precision; s.objective = a->objective; s.wmode = g->wmode;
   s.row_ptr = g->row_ptr; s.col_idx = g->col_idx; s.col_sw = g->col_sw; s.w = g->w; s.dnet = g->dnet;
   s.yin = y_in; s.yout = y_out; s.v = v;

@@ -215,6 +215,7 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 
 struct StepLaunch {
   int32_t n, C, ld;
+  int64_t nnz;
   int precision, objective, wmode;
   const int32_t* row_ptr;
   const int32_t* col_idx;

@@ -143,7 +143,7 @@ extern "C" int deco_run_phase_noalloc(const deco_graph* g, int32_t C, int32_t ld
 
   cudaStream_t st = as_stream(stream);
   StepLaunch sl{};
-  sl.n = g->n; sl.C = C; sl.ld = ld;
+  sl.n = g->n; sl.nnz = g->nnz; sl.C = C; sl.ld = ld;
   sl.precision = a->precision; sl.objective = a->objective; sl.wmode = g->wmode;
   sl.row_ptr = g->row_ptr; sl.col_idx = g->col_idx; sl.col_sw = g->col_sw; sl.w = g->w; sl.dnet = g->dnet;
   sl.v = v; sl.alpha = a->alpha; sl.mu = a->momentum;

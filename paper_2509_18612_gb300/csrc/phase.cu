@@ -498,7 +498,7 @@ int PhaseRunner::run(void* y[2], int& cur, float* v, int32_t steps, int objectiv
     return launch_step_global(s, stream);
   };
   StepLaunch sl{};
-  sl.n = g->n; sl.C = C; sl.ld = ld;
+  sl.n = g->n; sl.nnz = g->nnz; sl.C = C; sl.ld = ld;
   sl.precision = prec; sl.objective = objective; sl.wmode = g->wmode;
   sl.row_ptr = g->row_ptr; sl.col_idx = g->col_idx; sl.col_sw = g->col_sw; sl.w = g->w;
   sl.dnet = g->dnet;

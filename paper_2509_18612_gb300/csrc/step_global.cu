@@ -37,6 +37,9 @@
 #include "spmm.cuh"
 
 namespace deco {
+
+int device_sm_count();
+
 namespace {
 
 struct KArgs {
@@ -60,11 +63,13 @@ struct KArgs {
 };
 
 // Gathers in flight per lane, and blocks per SM (registers): more of both at once does not fit.  With momentum more
-// gathers win over more warps (by 6 % on the sixth graph above; 206 319 nodes, 9 columns, 16-bit 31 against 26 us).
-template <bool MOM>
+// gathers win over more warps (by 6 % on the sixth graph above; 206 319 nodes, 9 columns, 16-bit 31 against 26 us), and
+// without it on long rows and small grids (4 / 8 gathers: 4 096 nodes of degree 300 45 / 29 us, 8 000 of degree 20
+// 9.2 / 8.1; 200 000 of degree 24, 16-bit 88 / 96).
+template <bool EIGHT>
 struct Shape {
-  static constexpr int U = MOM ? 8 : 4;
-  static constexpr int BLOCKS = MOM ? 4 : 6;
+  static constexpr int U = EIGHT ? 8 : 4;
+  static constexpr int BLOCKS = EIGHT ? 4 : 6;
 };
 
 __device__ __forceinline__ void unpack(const uint4 q, float (&v)[4]) {
@@ -101,10 +106,10 @@ __device__ __forceinline__ void add_entry(float (&acc)[VN], uint4 q, uint32_t x,
 // starts.  Saves the launch gap of the smaller steps; on large ones the wait ahead of the own row's loads costs 1 - 5 %.
 // us per step without and with: 8 000 nodes, degree 20, 128 columns, FP32 11.2 / 8.8; 5 000, degree 3, 8 columns 5.1 /
 // 4.2; 200 003, degree 12, 60 columns 62 / 54, 100 columns with momentum and general weights 169 / 174.
-template <int PREC, int WMODE, bool MOM, bool LAP, bool OVERLAP>
-__global__ void __launch_bounds__(256, Shape<MOM>::BLOCKS) k_step_global(const __grid_constant__ KArgs a) {
+template <int PREC, int WMODE, bool MOM, bool LAP, bool EIGHT, bool OVERLAP>
+__global__ void __launch_bounds__(256, Shape<EIGHT>::BLOCKS) k_step_global(const __grid_constant__ KArgs a) {
   using V = VecT<PREC>;
-  constexpr int VN = V::N, U = Shape<MOM>::U;
+  constexpr int VN = V::N, U = Shape<EIGHT>::U;
   if (OVERLAP) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the next step's blocks may be placed
   const int gl = threadIdx.x & (a.G - 1);         // lane within the group
   const int64_t row = ((int64_t)blockIdx.x << (8 - a.lg)) + (threadIdx.x >> a.lg);
@@ -176,13 +181,13 @@ __global__ void __launch_bounds__(256, Shape<MOM>::BLOCKS) k_step_global(const _
   unpack(own, y);
   bool bad = false;
   const bool whole = c0 + VN <= a.C;
-  if (!a.alpha_cols && !a.steps_cols) {   // the same for the warp; columns past C are not stored
+  if (whole && !a.alpha_cols && !a.steps_cols) {
 #pragma unroll
     for (int k = 0; k < VN; ++k) {
       const float grad = LAP ? fmaf(dr, y[k], -acc[k]) : -acc[k];
       if (MOM) vv[k] = fmaf(a.mu, vv[k], grad);
       const float yn = fmaf(a.alpha_eff, MOM ? vv[k] : grad, y[k]);
-      bad = bad || (!isfinite(yn) && (whole || c0 + k < a.C));
+      bad = bad || !isfinite(yn);
       out[k] = fminf(fmaxf(yn, -1.0f), 1.0f);
     }
   } else {
@@ -233,28 +238,29 @@ void launch_k(void (*fn)(const KArgs), const KArgs& a, bool overlap, dim3 grid, 
   cudaLaunchKernelEx(&cfg, fn, a);   // the caller reads the error
 }
 
-template <int PREC, int WMODE, bool MOM, bool LAP>
-void launch_o(const KArgs& a, bool overlap, dim3 grid, cudaStream_t st) {
-  if (overlap) launch_k(k_step_global<PREC, WMODE, MOM, LAP, true>, a, true, grid, st);
-  else launch_k(k_step_global<PREC, WMODE, MOM, LAP, false>, a, false, grid, st);
-}
-
-template <int PREC, int WMODE>
-void launch_w(const KArgs& a, bool mom, bool lap, bool overlap, dim3 grid, cudaStream_t st) {
-  if (mom) {
-    if (lap) launch_o<PREC, WMODE, true, true>(a, overlap, grid, st);
-    else launch_o<PREC, WMODE, true, false>(a, overlap, grid, st);
+template <int PREC, int WMODE, bool MOM, bool EIGHT>
+void launch_o(const KArgs& a, bool lap, bool overlap, dim3 grid, cudaStream_t st) {
+  if (lap) {
+    if (overlap) launch_k(k_step_global<PREC, WMODE, MOM, true, EIGHT, true>, a, true, grid, st);
+    else launch_k(k_step_global<PREC, WMODE, MOM, true, EIGHT, false>, a, false, grid, st);
   } else {
-    if (lap) launch_o<PREC, WMODE, false, true>(a, overlap, grid, st);
-    else launch_o<PREC, WMODE, false, false>(a, overlap, grid, st);
+    if (overlap) launch_k(k_step_global<PREC, WMODE, MOM, false, EIGHT, true>, a, true, grid, st);
+    else launch_k(k_step_global<PREC, WMODE, MOM, false, EIGHT, false>, a, false, grid, st);
   }
 }
 
+template <int PREC, int WMODE>
+void launch_w(const KArgs& a, bool mom, bool lap, bool eight, bool overlap, dim3 grid, cudaStream_t st) {
+  if (mom) launch_o<PREC, WMODE, true, true>(a, lap, overlap, grid, st);
+  else if (eight) launch_o<PREC, WMODE, false, true>(a, lap, overlap, grid, st);
+  else launch_o<PREC, WMODE, false, false>(a, lap, overlap, grid, st);
+}
+
 template <int PREC>
-void launch_p(const KArgs& a, int wmode, bool mom, bool lap, bool overlap, dim3 grid, cudaStream_t st) {
-  if (wmode == W_UNIT) launch_w<PREC, W_UNIT>(a, mom, lap, overlap, grid, st);
-  else if (wmode == W_SIGN) launch_w<PREC, W_SIGN>(a, mom, lap, overlap, grid, st);
-  else launch_w<PREC, W_GENERAL>(a, mom, lap, overlap, grid, st);
+void launch_p(const KArgs& a, int wmode, bool mom, bool lap, bool eight, bool overlap, dim3 grid, cudaStream_t st) {
+  if (wmode == W_UNIT) launch_w<PREC, W_UNIT>(a, mom, lap, eight, overlap, grid, st);
+  else if (wmode == W_SIGN) launch_w<PREC, W_SIGN>(a, mom, lap, eight, overlap, grid, st);
+  else launch_w<PREC, W_GENERAL>(a, mom, lap, eight, overlap, grid, st);
 }
 
 }  // namespace
@@ -288,15 +294,19 @@ int launch_step_global(const StepLaunch& s, cudaStream_t st) {
   if (s.n == 0 || s.C == 0) return DECO_OK;
   const bool mom = s.mu != 0.0f;
   const bool lap = s.objective == DECO_OBJ_LAPLACIAN;
+  // long rows, and grids that leave warps' slots empty anyway: eight gathers in flight
+  const bool eight = s.nnz >= (int64_t)64 * s.n || (int64_t)s.n * s.C <= (int64_t)device_sm_count() * 2048 * VN;
   const int32_t nchunks = (nvec + G - 1) / G;
-  // steps of up to 64 MB of block and momentum (10 - 70 us): the gap between two launches is worth the wait
-  const bool overlap = s.overlap && nchunks <= 65535 &&
+  // steps of up to 64 MB of block and momentum (10 - 70 us): the gap between two launches is worth the wait.  Not rows of
+  // 1 024 entries and more, whose gathers the compiler overlaps better as read-only loads (4 096 nodes of degree 2 047,
+  // 128 columns, 16-bit: 205 us overlapping, 110 not; degree 300, FP32 29.5 and 31.8)
+  const bool overlap = s.overlap && nchunks <= 65535 && s.nnz < (int64_t)1024 * s.n &&
                        (int64_t)s.n * s.C * ((s.precision == DECO_PREC_BF16 ? 2 : 4) + (mom ? 8 : 0)) <= (64 << 20);
   const unsigned rows = (unsigned)(((int64_t)s.n * G + 255) / 256);
   for (a.ch0 = 0; a.ch0 < nchunks; a.ch0 += 65535) {
     const dim3 grid(rows, (unsigned)std::min(nchunks - a.ch0, 65535));
-    if (s.precision == DECO_PREC_BF16) launch_p<DECO_PREC_BF16>(a, s.wmode, mom, lap, overlap, grid, st);
-    else launch_p<DECO_PREC_FP32>(a, s.wmode, mom, lap, overlap, grid, st);
+    if (s.precision == DECO_PREC_BF16) launch_p<DECO_PREC_BF16>(a, s.wmode, mom, lap, eight, overlap, grid, st);
+    else launch_p<DECO_PREC_FP32>(a, s.wmode, mom, lap, eight, overlap, grid, st);
     DECO_CUDA_TRY(cudaGetLastError());
   }
   return DECO_OK;
