@@ -717,7 +717,7 @@ def batched_roofline(res):
     gathered = 4.0 * res.edge_updates
     ach = gathered / (res.device_ms / 1e3) / 1e9
     return {"bound": "alu", "achieved": ach, "peak": peak_onchip, "unit": "GB/s", "frac": ach / peak_onchip,
-            "traffic": None, "kernel": "k_slab (batched: one item per graph and column slab)",
+            "traffic": None, "kernel": "k_rows (batched: one item per graph and column slab)",
             "algorithmic_bytes": gathered, "time_s": res.device_ms / 1e3,
             "peak_kind": "measured: deco_probe_smem_rate (shared-memory load path, all SMs)",
             "derived_peak": derived, "frac_of_derived": ach / derived,
