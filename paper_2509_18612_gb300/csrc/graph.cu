@@ -44,7 +44,8 @@ double idi_threshold(const deco_graph* g, float beta) {
   return mean + (double)beta * std::sqrt(var);
 }
 
-static std::atomic<int64_t> g_graphs{0};   // handles that callers hold
+static std::atomic<int64_t> g_graphs[64];   // handles that callers hold, per device
+static std::atomic<int64_t>& graphs_on(int device) { return g_graphs[device & 63]; }
 
 static void free_graph(deco_graph* g) {
   if (!g) return;
@@ -60,8 +61,15 @@ static void free_graph(deco_graph* g) {
   cudaFree(g->dnet);
   cudaFree(g->deg);
   const bool counted = g->counted;
+  const int device = g->device;
   delete g;
-  if (counted && --g_graphs == 0) scratch_trim();
+  if (counted && --graphs_on(device) == 0) {
+    int current = device;
+    cudaGetDevice(&current);
+    if (current != device) cudaSetDevice(device);
+    scratch_trim();
+    if (current != device) cudaSetDevice(current);
+  }
 }
 
 }  // namespace deco
@@ -340,7 +348,7 @@ int deco::create_graph_impl(int32_t n, int64_t nnz, const int32_t* row_ptr, cons
     return rc;
   }
   g->counted = true;
-  ++g_graphs;
+  ++graphs_on(g->device);
   scratch_reserve();
   *out = g;
   return DECO_OK;

@@ -5,7 +5,7 @@
 // after which the first allocation of the next call maps it again: 110 us,
 // more than many calls take in all (a phase of one step on a 5 000-node
 // graph 150 -> 26 us).  What the pool keeps is bounded, is handed back
-// when the last graph is destroyed and when an allocation fails, and a pool
+// when a device's last graph is destroyed and when an allocation fails, and a pool
 // that the caller has made the device's current one is used instead of it.
 #include <mutex>
 
