@@ -559,6 +559,7 @@ extern "C" void deco_destroy_batch(deco_batch* b) {
   cudaFree(b->gsize);
   cudaFree(b->gmean);
   deco_destroy_graph(b->U);
+  for (auto& br : b->rows) cudaFree(br.data);
   delete b;
 }
 
