@@ -57,6 +57,16 @@ void scratch_reserve();   // makes the pool: with the first graph, so that no ca
 void scratch_trim();
 int current_context_id(unsigned long long* id);   // unique id of the current context (noalloc.cu)
 
+// Shared memory a block may have on the current device, static and dynamic (slab.cu)
+int block_smem_limit();
+// Lets fn be launched with dynamic shared memory: as much as a block may have beside `fixed` bytes (at least fn's static
+// shared memory).  The setting belongs to the function and not to the launch, so it is the same for every launch: one
+// launch's own size would refuse another host thread's larger launch between that thread's setting and its launch.
+template <class F>
+cudaError_t allow_smem(F fn, size_t fixed = 1024) {
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, block_smem_limit() - (int)fixed);
+}
+
 #define DECO_CUDA_TRY(expr)                                   \
   do {                                                        \
     cudaError_t _e = (expr);                                  \

@@ -34,7 +34,6 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
-#include <atomic>
 #include <mutex>
 
 #include "dense_tc.cuh"
@@ -874,9 +873,6 @@ int transpose(int32_t rows, int32_t cols, const T* in, int32_t ldin, T* out, int
   return DECO_OK;
 }
 
-// largest dynamic shared memory enabled per kernel instance [MOM][LAP][log2 KS]
-std::atomic<int> g_smem_set[2][2][4];
-
 using KernelFn = void (*)(DenseArgs);
 
 template <bool MOM, bool LAP>
@@ -1048,8 +1044,6 @@ PhaseFn pick_phase(int ks) {
   }
 }
 
-std::atomic<int> g_phase_smem[2][2][4];
-
 }  // namespace
 
 int launch_dense_phase(const DenseStep& p, const DenseMaps& maps, __nv_bfloat16* const yt[2],
@@ -1058,13 +1052,7 @@ int launch_dense_phase(const DenseStep& p, const DenseMaps& maps, __nv_bfloat16*
   const bool mom = p.mu != 0.0f, lap = p.objective == DECO_OBJ_LAPLACIAN;
   PhaseFn fn = mom ? (lap ? pick_phase<true, true>(sh.ks) : pick_phase<true, false>(sh.ks))
                    : (lap ? pick_phase<false, true>(sh.ks) : pick_phase<false, false>(sh.ks));
-  const int lk = sh.ks == 1 ? 0 : (sh.ks == 2 ? 1 : (sh.ks == 4 ? 2 : 3));
-  std::atomic<int>& set = g_phase_smem[mom][lap][lk];
-  if (set.load() < (int)sh.smem) {
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh.smem);
-    if (e != cudaSuccess) return cuda_fail(e, "dense phase shared memory");
-    set.store((int)sh.smem);
-  }
+  DECO_CUDA_TRY(allow_smem(fn, 512));
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(p.kpad / BM * sh.ks), (unsigned)((p.cpad + sh.w - 1) / sh.w), 1);
   cfg.blockDim = dim3(PT, 1, 1);
@@ -1131,13 +1119,7 @@ int launch_dense_step(const DenseStep& p, const DenseMaps& maps, int which, cuda
   const bool mom = p.mu != 0.0f, lap = p.objective == DECO_OBJ_LAPLACIAN;
   KernelFn fn = mom ? (lap ? pick_ks<true, true>(p.ks) : pick_ks<true, false>(p.ks))
                     : (lap ? pick_ks<false, true>(p.ks) : pick_ks<false, false>(p.ks));
-  const int lk = p.ks == 1 ? 0 : (p.ks == 2 ? 1 : (p.ks == 4 ? 2 : 3));
-  std::atomic<int>& set = g_smem_set[mom][lap][lk];
-  if (set.load() < (int)smem) {
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return cuda_fail(e, "dense step shared memory");
-    set.store((int)smem);
-  }
+  DECO_CUDA_TRY(allow_smem(fn, 512));
   DenseArgs args;
   args.tmA = maps.a;
   args.tmY = maps.y[which];

@@ -565,19 +565,11 @@ struct Acts {
   int32_t chunk = 0, chunks = 0;
 };
 
-template <class F>
-int max_smem(F fn, size_t bytes) {
-  if (bytes <= 48 * 1024) return DECO_OK;
-  DECO_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-  return DECO_OK;
-}
-
 // picks the kernel of the graph's weight storage and launches it over the node tiles
 #define DECO_LAUNCH_TILES(kernel, g, H, smem, st, args)                                                      \
   do {                                                                                                       \
     auto fn_ = (g)->wmode == W_UNIT ? kernel<W_UNIT> : (g)->wmode == W_SIGN ? kernel<W_SIGN> : kernel<W_GENERAL>; \
-    int rc_ = max_smem(fn_, smem);                                                                           \
-    if (rc_) return rc_;                                                                                     \
+    DECO_CUDA_TRY(allow_smem(fn_));                                                                          \
     fn_<<<nb((g)->n, LTILE), 4 * (H), smem, st>>>(args);                                                     \
     DECO_CUDA_TRY(cudaGetLastError());                                                                       \
   } while (0)
@@ -723,8 +715,7 @@ int backward(deco_mpnn* m, const deco_graph* g, const FeatureInfo& fi, const uin
   w.obo = lo.bo;
   w.part = a.part;
   const size_t wsm = sizeof(float) * std::max<size_t>((size_t)WG_TILE * (std::min(2 * H, rows) + 12 + H), WG_THREADS);
-  int rc = max_smem(k_wgrad_part, wsm);
-  if (rc) return rc;
+  DECO_CUDA_TRY(allow_smem(k_wgrad_part));
   k_wgrad_part<<<dim3((unsigned)a.chunks, (unsigned)((L + 2) * w.passes)), WG_THREADS, wsm, st>>>(w);
   DECO_CUDA_TRY(cudaGetLastError());
   SumArgs sa{};

@@ -300,7 +300,7 @@ template <int PREC, int WMODE, bool PERCOL, int LPR, bool BATCH>
 cudaError_t launch_l(const RowsParams& p, int n_items, cudaStream_t st) {
   constexpr int NT = rows_max_threads(PREC, PERCOL);
   auto fn = k_rows<PREC, WMODE, PERCOL, LPR, BATCH, NT>;
-  const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+  const cudaError_t e = allow_smem(fn);
   if (e != cudaSuccess) return e;
   fn<<<(unsigned)n_items, std::min(p.threads, NT), p.smem, st>>>(p);
   return cudaGetLastError();

@@ -177,7 +177,7 @@ template <int PREC, int WMODE, int E>
 cudaError_t launch_e(const RowsParams& p, int n_items, int threads, size_t smem, cudaStream_t st) {
   // up to 16 warps: eight gathers in flight; up to 32 leave 64 registers a thread
   auto fn = threads <= 512 ? k_rows_reg<PREC, WMODE, E, 8, 512> : k_rows_reg<PREC, WMODE, E, 4, 1024>;
-  const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = allow_smem(fn);
   if (e != cudaSuccess) return e;
   fn<<<(unsigned)n_items, threads, smem, st>>>(p);
   return cudaGetLastError();

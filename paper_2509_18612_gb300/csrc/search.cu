@@ -613,7 +613,7 @@ static int run_planes(const deco_graph* g, int32_t B, uint32_t* zbits, int32_t m
   const size_t smem = ls_smem(n, entries, GEN).total;
   if (n <= 32768 && smem + 1024 <= (size_t)slab_max_smem()) {
     const int nt = own <= 256 ? 256 : own <= 512 ? 512 : 1024;
-    DECO_CUDA_TRY(cudaFuncSetAttribute(k_ls_cluster<NP, GEN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    DECO_CUDA_TRY(allow_smem(k_ls_cluster<NP, GEN>));
     k_ls_cluster<NP, GEN><<<(unsigned)W * LS_CLUSTER, nt, smem, st>>>(n, W, B, g->row_ptr, col, g->wint, zbits, gains, max_rounds,
                                                                  changed, entries);
     DECO_CUDA_TRY(cudaGetLastError());
@@ -697,10 +697,11 @@ extern "C" int deco_greedy(const deco_graph* g, int32_t B, uint64_t seed, uint8_
   DECO_CUDA_TRY(cudaGetLastError());
   const size_t smem = ((size_t)n + 15) / 16 * 16;
   // the sides, beside the two windows of loaded rows
-  const bool fits = smem + sizeof(GreedyWindow<true>) * 2 <= (size_t)slab_max_smem();
+  constexpr size_t windows = 2 * sizeof(GreedyWindow<true>) + 1024;
+  const bool fits = smem + windows <= (size_t)block_smem_limit();
   auto fn = g->wint ? (fits ? k_greedy<true, true> : k_greedy<true, false>)
                     : (fits ? k_greedy<false, true> : k_greedy<false, false>);
-  if (fits) DECO_CUDA_TRY(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  if (fits) DECO_CUDA_TRY(allow_smem(fn, windows));
   else DECO_CUDA_TRY(cudaMemsetAsync(z, 2, (size_t)n * B, st));
   fn<<<(unsigned)B, 64, fits ? smem : 0, st>>>(n, B, g->row_ptr, g->col_idx, g->wint, order, z);
   DECO_CUDA_TRY(cudaGetLastError());

@@ -503,7 +503,7 @@ __global__ void __launch_bounds__(NT, 1) k_slab(SlabParams P) {
 template <int PREC, int WMODE, int NT, bool LEAN>
 cudaError_t launch_t(const SlabParams& p, int n_items, size_t smem, cudaStream_t st) {
   auto fn = p.pairs ? k_slab<PREC, WMODE, NT, LEAN, true> : k_slab<PREC, WMODE, NT, LEAN, false>;
-  cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem(fn);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(n_items * p.k), 1, 1);
@@ -554,15 +554,17 @@ size_t slab_smem_bytes(int max_n, int max_own, int max_img_words, int prec, bool
   return slab_layout(max_n, max_own, max_img_words, prec, lean).total;
 }
 
-int slab_max_smem() {
+int block_smem_limit() {
   int dev = 0, v = 0;
   cudaGetDevice(&dev);
   if (cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
     cudaGetLastError();
     v = 227 * 1024;
   }
-  return v - 1024;   // room for the kernel's static shared memory (mbarrier)
+  return v;
 }
+
+int slab_max_smem() { return block_smem_limit() - 1024; }   // room for the kernel's static shared memory (mbarrier)
 
 int slab_resident_clusters(int k) {
   static std::atomic<int> held[SLAB_MAX_CLUSTER + 1];   // every thread finds the same value
@@ -582,7 +584,7 @@ int slab_resident_clusters(int k) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+    if (allow_smem(fn) != cudaSuccess ||
         cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess || n < 1) {
       cudaGetLastError();
       n = std::max(1, 152 / k);

@@ -35,3 +35,73 @@ def test_batches_leave_no_device_memory_behind(precision):
 
     before = program(3)
     assert before - program(40) <= 8 << 20
+
+
+def _greedy(n):
+    G = deco.graph_from(gg.er_graph_avg_degree(n, 5.0, 1))
+    z, cuts = torch.zeros(n, dtype=torch.uint8, device=DEV), torch.zeros(1, dtype=torch.int64, device=DEV)
+    return lambda st: deco.deco_greedy(G, 1, 1, z, cuts, stream=st)
+
+
+def _search(n):
+    G = deco.graph_from(gg.torus_graph(n // 4, 4, 1))
+    z, cuts = torch.zeros(n * 8, dtype=torch.uint8, device=DEV), torch.zeros(8, dtype=torch.int64, device=DEV)
+    return lambda st: deco.deco_local_search(G, 8, z, 1, cuts, stream=st)
+
+
+def _phase(n, kernel, per_column):
+    G = deco.graph_from(gg.er_graph_avg_degree(n, 5.0, 1))
+    y = torch.zeros(n, 64, device=DEV)
+    alpha = torch.full((64,), 0.01, device=DEV)
+    args = deco.step_args(alpha_cols=alpha if per_column else None)
+    return lambda st, _alpha=alpha: deco.deco_run_phase(G, 64, 64, y, None, 1, args, kernel, stream=st)
+
+
+def _infer(hidden):
+    G = deco.graph_from(gg.er_graph_avg_degree(500, 5.0, 1))
+    m, h = deco.Mpnn(hidden, 1, 1), torch.zeros(500, device=DEV)
+    return lambda st: m.infer(G, h, 1, stream=st)
+
+
+def _train(hidden):
+    G = deco.graph_from(gg.er_graph_avg_degree(500, 5.0, 1))
+    m, z = deco.Mpnn(hidden, 1, 1), torch.zeros(500, dtype=torch.uint8, device=DEV)
+    return lambda st: m.train(G, z, 1, stream=st)
+
+
+SLAB = deco.DECO_KERNEL_ONCHIP | (8 << 8) | deco.DECO_KERNEL_ROW_PAIRS
+
+
+# Two host threads on graphs of different sizes, each with a stream of its own: launches of the same kernels with much
+# and with little shared memory in turn, none of which may refuse the other's.
+@pytest.mark.parametrize("name,big,small", [
+    ("greedy", lambda: _greedy(150000), lambda: _greedy(64)),
+    ("search", lambda: _search(20000), lambda: _search(64)),
+    ("rows", lambda: _phase(1500, deco.DECO_KERNEL_AUTO, True), lambda: _phase(40, deco.DECO_KERNEL_AUTO, True)),
+    ("registers", lambda: _phase(500, deco.DECO_KERNEL_AUTO, False), lambda: _phase(300, deco.DECO_KERNEL_AUTO, False)),
+    ("slab", lambda: _phase(1200, SLAB, False), lambda: _phase(60, SLAB, False)),
+    ("infer", lambda: _infer(128), lambda: _infer(64)),
+    ("train", lambda: _train(128), lambda: _train(64)),
+])
+def test_host_threads_do_not_refuse_each_others_launches(name, big, small):
+    calls, errors = [big(), small()], []
+    end = time.time() + 1.5
+
+    def loop(call):
+        stream = torch.cuda.Stream()
+        try:
+            while time.time() < end and not errors:
+                for _ in range(8):
+                    call(stream.cuda_stream)
+                stream.synchronize()
+        except deco.DecoError as e:
+            errors.append(str(e))
+
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=loop, args=(c,)) for c in calls]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors, errors
