@@ -37,6 +37,8 @@
 namespace cg = cooperative_groups;
 
 namespace deco {
+
+int device_sm_count();
 namespace {
 
 
@@ -567,31 +569,32 @@ int block_smem_limit() {
 int slab_max_smem() { return block_smem_limit() - 1024; }   // room for the kernel's static shared memory (mbarrier)
 
 int slab_resident_clusters(int k) {
-  static std::atomic<int> held[SLAB_MAX_CLUSTER + 1];   // every thread finds the same value
+  constexpr int DEVICES = 64;
+  static std::atomic<int> held[DEVICES][SLAB_MAX_CLUSTER + 1];   // every thread finds the same value
+  int dev = 0;
   if (k < 1 || k > SLAB_MAX_CLUSTER) return 1;
-  if (held[k] == 0) {
-    auto fn = k_slab<DECO_PREC_FP32, W_UNIT, 1024, false, true>;
-    const size_t smem = (size_t)slab_max_smem();
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(k * 64), 1, 1);
-    cfg.blockDim = dim3(1024, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)k;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (allow_smem(fn) != cudaSuccess ||
-        cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess || n < 1) {
-      cudaGetLastError();
-      n = std::max(1, 152 / k);
-    }
-    held[k] = n;
+  if (cudaGetDevice(&dev) != cudaSuccess) cudaGetLastError();
+  const bool known = dev >= 0 && dev < DEVICES;
+  if (known && held[dev][k] != 0) return held[dev][k];
+  auto fn = k_slab<DECO_PREC_FP32, W_UNIT, 1024, false, true>;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(k * 64), 1, 1);
+  cfg.blockDim = dim3(1024, 1, 1);
+  cfg.dynamicSmemBytes = (size_t)slab_max_smem();
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)k;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (allow_smem(fn) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, fn, &cfg) != cudaSuccess || n < 1) {
+    cudaGetLastError();
+    return std::max(1, device_sm_count() / k);   // not kept: the next call asks again
   }
-  return held[k];
+  if (known) held[dev][k] = n;
+  return n;
 }
 
 // Row split of one graph into k parts by cost(r) = row_ptr[r] + 2 r.
