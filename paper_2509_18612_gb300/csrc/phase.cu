@@ -302,15 +302,46 @@ int plan_phase(const deco_graph* g, int32_t C, int32_t ld, int prec, int force, 
   return DECO_OK;
 }
 
+// The plan of a phase on a capturing stream, which allows no cudaMalloc, where
+// the image of the planned on-chip form is not there yet.  AUTO: the per-step
+// kernel.  ONCHIP, whose form is the planner's choice: the row-vector form of
+// another slab width whose image is there, else k_slab.
+static int plan_captured(const deco_graph* g, int32_t C, int32_t ld, int prec, int force, PhasePlan* plan) {
+  const bool chosen = force == DECO_KERNEL_ONCHIP;
+  if (!chosen && (force & 0x3) == DECO_KERNEL_ONCHIP) return DECO_OK;   // a fixed shape: refused when it is built
+  {
+    std::lock_guard<std::mutex> lock(g_image_mutex);
+    const RowsImage* other = nullptr;
+    for (const RowsImage& im : g->rows) {
+      if (plan->kernel == KERNEL_ROWS && im.lpr == plan->rows_lpr) return DECO_OK;
+      if (rows_smem_bytes(im, prec, true, true) <= (size_t)slab_max_smem()) other = &im;
+    }
+    for (const SlabImage& im : g->images)
+      if (plan->kernel == KERNEL_ONCHIP && im.k == plan->k) return DECO_OK;
+    if (chosen && other) {
+      const int w = other->lpr * (prec == DECO_PREC_BF16 ? 8 : 4);
+      plan->kernel = KERNEL_ROWS;
+      plan->rows_lpr = other->lpr;
+      plan->items = (C + w - 1) / w;
+      return DECO_OK;
+    }
+  }
+  return plan_phase(g, C, ld, prec, chosen ? DECO_KERNEL_ONCHIP | DECO_KERNEL_THREADS_1024 : DECO_KERNEL_GLOBAL, plan);
+}
+
 int PhaseRunner::prepare(const deco_graph* g_, int32_t C_, int32_t ld_, int prec_, int force,
                          cudaStream_t st) {
-  (void)st;
   g = g_;
   C = C_;
   ld = ld_;
   prec = prec_;
   int rc = plan_phase(g, C, ld, prec, force, &plan);
   if (rc) return rc;
+  if (plan.kernel == KERNEL_ROWS || plan.kernel == KERNEL_ONCHIP) {
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
+    if (capture != cudaStreamCaptureStatusNone && (rc = plan_captured(g, C, ld, prec, force, &plan))) return rc;
+  }
   if (plan.kernel == KERNEL_DENSE) {
     {
       std::lock_guard<std::mutex> lock(g_image_mutex);

@@ -105,3 +105,33 @@ def test_host_threads_do_not_refuse_each_others_launches(name, big, small):
         t.join()
     torch.cuda.synchronize()
     assert not errors, errors
+
+
+# A phase whose first call on a graph, or first call of its width, is captured: the images of the on-chip forms, which
+# need an allocation, are not there.  (ONCHIP: warmed with another width, whose image serves.)
+@pytest.mark.parametrize("n,degree,warm,C,kernel", [
+    (3000, 6.0, 0, 64, deco.DECO_KERNEL_AUTO), (800, 5.0, 0, 64, deco.DECO_KERNEL_AUTO),
+    (800, 48.0, 64, 1024, deco.DECO_KERNEL_AUTO), (800, 5.0, 64, 1024, deco.DECO_KERNEL_AUTO),
+    (800, 5.0, 64, 1024, deco.DECO_KERNEL_ONCHIP), (800, 5.0, 64, 64, deco.DECO_KERNEL_ONCHIP)])
+@pytest.mark.parametrize("precision", [deco.DECO_PREC_FP32, deco.DECO_PREC_BF16])
+def test_phases_captured_before_their_images_are_built(n, degree, warm, C, kernel, precision):
+    G = deco.graph_from(gg.er_graph_avg_degree(n, degree, 1))
+    dtype = torch.bfloat16 if precision else torch.float32
+    args = deco.step_args(0, precision, 0.01, 0.9)
+    y0 = (torch.rand(n, C, device=DEV) - 0.5).to(dtype)
+    y, v = y0.clone(), torch.zeros(n, C, device=DEV)
+    ref, vref = y0.clone(), v.clone()
+    deco.deco_run_phase(G, C, C, ref, vref, 5, args, deco.DECO_KERNEL_GLOBAL)
+    if warm:
+        deco.deco_run_phase(G, warm, warm, torch.zeros(n, warm, device=DEV, dtype=dtype),
+                            torch.zeros(n, warm, device=DEV), 2, args, kernel)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        deco.deco_run_phase(G, C, C, y, v, 5, args, kernel, stream=torch.cuda.current_stream().cuda_stream)
+    for _ in range(2):
+        y.copy_(y0)
+        v.zero_()
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(y, ref) and torch.equal(v, vref)
