@@ -216,7 +216,9 @@ int deco_eval_cut(const deco_graph* g, const uint8_t* z, int64_t* cut_out);
 
 /* Batched integer cut values (Eq. 1) of B binary columns.
  *  z     device, n x B bytes row-major (z[v*B + b]), 0/1.
- *  cuts  device, B int64 (overwritten).  Stream-ordered, asynchronous. */
+ *  cuts  device, B int64 (overwritten).  Stream-ordered, asynchronous.
+ * Many vectors are packed into scratch memory first (n x ceil(B/32) words);
+ * where there is none, and on a capturing stream, they are read as they are. */
 int deco_eval_cuts(const deco_graph* g, int32_t B, const uint8_t* z, int64_t* cuts, void* stream);
 
 /* Arguments of one fused PGA step.  Reading of the momentum form (the paper

@@ -13,7 +13,8 @@
 //          transposed themselves, and lane b takes one popc per bit of |w| and
 //          sign.  Entries with u > v count (each unordered edge once), in
 //          integers; the block reduces and issues one 64-bit atomic per
-//          starting point.  Integer sums are exact in any order.
+//          starting point.  Integer sums are exact in any order.  Vectors
+//          given as bytes are packed first, or read where they are (k_cut_bytes).
 //  argmax: one block; lowest index among the maximal cuts.
 #include <algorithm>
 
@@ -284,6 +285,44 @@ __global__ void __launch_bounds__(CUT_BLOCK, 4) k_cut(int32_t n, int32_t B, int3
   }
 }
 
+// Cuts of byte columns read where they are: a warp per row, 2^lb lanes over the
+// columns of group k0 + blockIdx.y (of 32) times 32 / 2^lb over the row's entries.
+// No scratch memory: for few vectors or small graphs, where packing them first
+// (an allocation, a launch) costs more than it saves, and where none is to be had.
+template <bool WT>
+__global__ void __launch_bounds__(CUT_BLOCK) k_cut_bytes(int32_t n, int32_t B, int lb, int32_t k0, const int32_t* __restrict__ row_ptr,
+                                                         const int32_t* __restrict__ col_idx,
+                                                         const int32_t* __restrict__ wint, const uint8_t* __restrict__ z,
+                                                         int64_t* cuts) {
+  __shared__ long long part[CUT_BLOCK / 32][32];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  const int32_t b = 32 * (k0 + (int32_t)blockIdx.y) + (lane & ((1 << lb) - 1));
+  const int slots = 32 >> lb;
+  const int64_t warps = (int64_t)gridDim.x * (CUT_BLOCK / 32);
+  long long acc = 0;
+  if (b < B) {
+    for (int64_t v = (int64_t)blockIdx.x * (CUT_BLOCK / 32) + wib; v < n; v += warps) {
+      const int32_t e1 = __ldg(row_ptr + v + 1);
+      const bool zv = __ldg(z + (size_t)v * B + b) != 0;
+      int32_t sum = 0;   // |sum| <= the row's sum of |w| <= 2^24
+#pragma unroll 4
+      for (int32_t e = __ldg(row_ptr + v) + (lane >> lb); e < e1; e += slots) {
+        const int32_t u = __ldg(col_idx + e);
+        if (u > v && (__ldg(z + (size_t)u * B + b) != 0) != zv) sum += WT ? __ldg(wint + e) : 1;
+      }
+      acc += sum;
+    }
+  }
+  for (int s = 16; s >= 1 << lb; s >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, s);
+  part[wib][lane] = acc;
+  __syncthreads();
+  if (threadIdx.x < (1 << lb) && b < B) {
+    long long s = 0;
+    for (int i = 0; i < CUT_BLOCK / 32; ++i) s += part[i][threadIdx.x];
+    if (s != 0) atomicAdd(reinterpret_cast<unsigned long long*>(cuts + b), (unsigned long long)s);
+  }
+}
+
 __global__ void k_argmax(int32_t B, const int64_t* cuts, int32_t* best) {
   __shared__ long long sv[1024];
   __shared__ int32_t si[1024];
@@ -421,10 +460,39 @@ int launch_bytes_to_bits(int32_t n, int32_t B, const uint8_t* z, uint32_t* bits,
   return DECO_OK;
 }
 
+static int launch_cut_bytes(const deco_graph* g, int32_t B, const uint8_t* z, int64_t* cuts, cudaStream_t st) {
+  const int32_t W = (B + 31) / 32;
+  int lb = 0;
+  while ((1 << lb) < std::min(B, 32)) ++lb;
+  DECO_CUDA_TRY(cudaMemsetAsync(cuts, 0, sizeof(int64_t) * (size_t)B, st));
+  const int64_t rows = ((int64_t)g->n + CUT_BLOCK / 32 - 1) / (CUT_BLOCK / 32), sms = device_sm_count();
+  for (int32_t k0 = 0; k0 < W; k0 += 65535) {   // grid limit
+    const dim3 grid((unsigned)std::min(rows, std::max(sms, sms * 8 / W)), (unsigned)std::min(W - k0, 65535));
+    if (g->wint) k_cut_bytes<true><<<grid, CUT_BLOCK, 0, st>>>(g->n, B, lb, k0, g->row_ptr, g->col_idx, g->wint, z, cuts);
+    else k_cut_bytes<false><<<grid, CUT_BLOCK, 0, st>>>(g->n, B, lb, k0, g->row_ptr, g->col_idx, nullptr, z, cuts);
+    DECO_CUDA_TRY(cudaGetLastError());
+  }
+  return DECO_OK;
+}
+
+// Packed where that is faster, the scratch for it is there and the stream is
+// not capturing (the caller's graph then holds no memory of ours).  us a call,
+// packed and as they are: n = 100, degree 10, B = 1 31 / 19, B = 256 31 / 21;
+// n = 5 000, degree 10, B = 16 31 / 21, B = 256 40 / 34; n = 3 000, degree 300,
+// B = 4 37 / 30, B = 16 37 / 46; n = 20 000, degree 60, B = 4 39 / 27, B = 33
+// 45 / 87; n = 10^6, degree 8, B = 1 122 / 97, B = 8 121 / 139.
 int cut_bytes(const deco_graph* g, int32_t B, const uint8_t* z, int64_t* cuts, cudaStream_t st) {
+  if (g->nnz * B <= (B <= 16 ? 6000000 : 1000000)) return launch_cut_bytes(g, B, z, cuts, st);
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  DECO_CUDA_TRY(cudaStreamIsCapturing(st, &capture));
+  if (capture != cudaStreamCaptureStatusNone) return launch_cut_bytes(g, B, z, cuts, st);
   Scratch s(st);
   uint32_t* bits = nullptr;
   int rc = s.alloc(&bits, sizeof(uint32_t) * (size_t)g->n * ((B + 31) / 32));
+  if (rc == DECO_ERR_OOM) {
+    clear_error();
+    return launch_cut_bytes(g, B, z, cuts, st);
+  }
   if (rc || (rc = launch_bytes_to_bits(g->n, B, z, bits, st))) return rc;
   return launch_cut_bits(g, B, bits, cuts, st);
 }

@@ -266,7 +266,7 @@ int launch_cut_graphs(const deco_graph* g, int32_t B, const uint32_t* zbits, con
                       int64_t* cuts, cudaStream_t st);
 // n x B bytes (nonzero = 1) to n x ceil(B/32) words
 int launch_bytes_to_bits(int32_t n, int32_t B, const uint8_t* z, uint32_t* bits, cudaStream_t st);
-// cuts of byte columns, through a packed scratch copy
+// cuts of byte columns, through a packed scratch copy or (few vectors, no scratch, capture) as they are
 int cut_bytes(const deco_graph* g, int32_t B, const uint8_t* z, int64_t* cuts, cudaStream_t st);
 int launch_argmax(int32_t B, const int64_t* cuts, int32_t* best, cudaStream_t st);
 // 1-flip local search on bit-packed columns (n x ceil(B/32) words), in place;

@@ -332,3 +332,32 @@ def test_cuts_by_bit_planes_match_oracle(name, B):
     cuts = torch.zeros(B, dtype=torch.int64, device=DEV)
     deco.deco_eval_cuts(deco.graph_from(g), B, torch.from_numpy(Z.reshape(-1)).to(DEV), cuts)
     np.testing.assert_array_equal(cuts.cpu().numpy(), O.cut_values(g, Z))
+
+
+# Cuts of byte vectors read where they are (few vectors, small graphs) and packed first; without scratch memory, and
+# captured, they are read where they are whatever their number.
+@pytest.mark.parametrize("name", list(CUT_GRAPHS) + ["edgeless", "many entries"])
+@pytest.mark.parametrize("B", [1, 2, 3, 16, 17, 31, 32, 33, 75])
+@pytest.mark.parametrize("how", ["plain", "no scratch", "captured"])
+def test_cuts_of_byte_vectors_match_oracle(name, B, how):
+    rng = np.random.default_rng(B)
+    g = (gg.from_edges(40, [], []) if name == "edgeless" else gg.er_graph(2500, 0.08, 3) if name == "many entries"
+         else CUT_GRAPHS[name](rng))
+    G = deco.graph_from(g)
+    Z = (rng.random((g.n, B)) < 0.5).astype(np.uint8)
+    z = torch.from_numpy((Z * rng.integers(1, 256, Z.shape)).astype(np.uint8).reshape(-1)).to(DEV)   # nonzero is 1
+    cuts = torch.full((B,), -1, dtype=torch.int64, device=DEV)
+    if how == "captured":
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            deco.deco_eval_cuts(G, B, z, cuts, stream=torch.cuda.current_stream().cuda_stream)
+        graph.replay()
+    else:
+        deco.deco_debug_fail_scratch_alloc(1 if how == "no scratch" else 0)
+        try:
+            deco.deco_eval_cuts(G, B, z, cuts)
+        finally:
+            deco.deco_debug_fail_scratch_alloc(0)
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(cuts.cpu().numpy(), O.cut_values(g, Z))
