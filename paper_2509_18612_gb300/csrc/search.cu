@@ -96,45 +96,49 @@ __global__ void __launch_bounds__(256) k_orders(Feistel F, int32_t B, int32_t* o
 // One run per block places its vertices in order: warp 0 places, warp 1 loads
 // ahead of it.  Bound by the chain of n dependent placements: a shared load of
 // the neighbours' sides (2: not placed), a warp reduction, a shared store.
-// Warp 1 fills the list of the next GREEDY_WIN vertices (vertex, row, first 64
-// entries) in shared memory while warp 0 works on this one; longer rows are
-// read in place.  SMEM: the sides live in shared memory, a byte per vertex, and
-// go to the run's part of `order` at the end, which it has consumed (4 n bytes of
-// stride); else (a graph whose sides do not fit) they are column b of z.
-// Measured, n = 5 000, degree 10, 256 runs: 0.49 ms; loading ahead from the same
-// warp 1.07, with the whole chain of loads in each placement 4.28.
-constexpr int GREEDY_WIN = 16;
+// Warp 1 fills the list of the next WIN vertices (vertex, row, first 64
+// entries) in shared memory while warp 0 works on this one; of longer rows the
+// rest is read in place, several loads at once.  The sides of a run are a byte
+// or two bits per vertex in shared memory, which go to the run's part of
+// `order` at the end (it has consumed it; 4 n bytes of stride), or column b of
+// z: greedy_plan.  Measured, degree 10, 256 runs of 5 000 vertices: 0.54 ms;
+// loading ahead from the same warp 1.07, with the whole chain of loads in each
+// placement 4.28.  Degree 300, one run: 4.0 ms; one load after another on long
+// rows 8.9.
+enum GreedySides : int { GREEDY_BYTES = 0, GREEDY_BITS = 1, GREEDY_COLUMN = 2 };
 
-template <bool WT>
+template <bool WT, int WIN>
 struct GreedyWindow {
-  int4 row[GREEDY_WIN];                                  // vertex, first entry, entries
-  int32_t u[GREEDY_WIN][64];                             // neighbours (-1: none)
-  int32_t w[WT ? GREEDY_WIN : 1][64];
+  int4 row[WIN];                                  // vertex, first entry, entries
+  int32_t u[WIN][64];                             // neighbours (-1: none)
+  int32_t w[WT ? WIN : 1][64];
 };
 
-template <bool WT, bool SMEM>
+template <bool WT, int SIDES, int WIN>
 __global__ void __launch_bounds__(64) k_greedy(int32_t n, int32_t B, const int32_t* __restrict__ row_ptr,
                                                const int32_t* __restrict__ col_idx, const int32_t* __restrict__ wint,
                                                int32_t* order, uint8_t* z) {
   extern __shared__ __align__(16) uint8_t sides[];
-  __shared__ GreedyWindow<WT> win[2];
+  __shared__ GreedyWindow<WT, WIN> win[2];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int32_t b = blockIdx.x;
   int32_t* const ord = order + (size_t)b * n;
-  if (SMEM)
-    for (int i = threadIdx.x; i < (n + 3) / 4; i += 64) reinterpret_cast<uint32_t*>(sides)[i] = 0x02020202u;
+  uint32_t* const words = reinterpret_cast<uint32_t*>(sides);
+  if (SIDES != GREEDY_COLUMN)
+    for (int i = threadIdx.x; i < (SIDES == GREEDY_BYTES ? (n + 3) / 4 : (n + 15) / 16); i += 64)
+      words[i] = SIDES == GREEDY_BYTES ? 0x02020202u : 0xAAAAAAAAu;
   // rows of the window after the next, one per lane (warp 1)
   int32_t v = -1, e0 = 0, d = 0;
   auto rows = [&](int32_t k) {
-    v = lane < GREEDY_WIN && k + lane < n ? ord[k + lane] : -1;
+    v = lane < WIN && k + lane < n ? ord[k + lane] : -1;
     e0 = v >= 0 ? __ldg(row_ptr + v) : 0;
     d = v >= 0 ? __ldg(row_ptr + v + 1) - e0 : 0;
   };
-  auto fill = [&](GreedyWindow<WT>& g) {
-    if (lane < GREEDY_WIN) g.row[lane] = make_int4(v, e0, d, 0);
-    int32_t u[GREEDY_WIN][2], w[WT ? GREEDY_WIN : 1][2];
+  auto fill = [&](GreedyWindow<WT, WIN>& g) {
+    if (lane < WIN) g.row[lane] = make_int4(v, e0, d, 0);
+    int32_t u[WIN][2], w[WT ? WIN : 1][2];
 #pragma unroll
-    for (int j = 0; j < GREEDY_WIN; ++j) {
+    for (int j = 0; j < WIN; ++j) {
       const int32_t ej = __shfl_sync(0xFFFFFFFFu, e0, j), dj = __shfl_sync(0xFFFFFFFFu, d, j);
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
@@ -147,7 +151,7 @@ __global__ void __launch_bounds__(64) k_greedy(int32_t n, int32_t B, const int32
       }
     }
 #pragma unroll
-    for (int j = 0; j < GREEDY_WIN; ++j)
+    for (int j = 0; j < WIN; ++j)
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         g.u[j][32 * h + lane] = u[j][h];
@@ -157,19 +161,22 @@ __global__ void __launch_bounds__(64) k_greedy(int32_t n, int32_t B, const int32
   if (warp == 1) {
     rows(0);
     fill(win[0]);
-    rows(GREEDY_WIN);
+    rows(WIN);
   }
   __syncthreads();
-  for (int32_t k0 = 0, s = 0; k0 < n; k0 += GREEDY_WIN, s ^= 1) {
+  for (int32_t k0 = 0, s = 0; k0 < n; k0 += WIN, s ^= 1) {
     if (warp == 1) {
       fill(win[s ^ 1]);
-      rows(k0 + 2 * GREEDY_WIN);
+      rows(k0 + 2 * WIN);
     } else {
-      const GreedyWindow<WT>& g = win[s];
-      const int cnt = min(GREEDY_WIN, n - k0);
+      const GreedyWindow<WT, WIN>& g = win[s];
+      const int cnt = min(WIN, n - k0);
       auto vote = [&](int32_t u, int32_t w) -> int32_t {
         // w if the neighbour is in S-bar (placing v in S cuts the edge), -w if in S, 0 if not placed
-        const int x = u >= 0 ? (SMEM ? sides[u] : z[(size_t)u * B + b]) : 2;
+        int x = 2;
+        if (u >= 0)
+          x = SIDES == GREEDY_BYTES ? sides[u] : SIDES == GREEDY_BITS ? (words[u >> 4] >> (2 * (u & 15))) & 3u
+                                                                        : z[(size_t)u * B + b];
         return x == 0 ? w : x == 1 ? -w : 0;
       };
       int4 r = g.row[0];
@@ -184,23 +191,43 @@ __global__ void __launch_bounds__(64) k_greedy(int32_t n, int32_t B, const int32
         if (WT) w0 = g.w[WT ? jn : 0][lane];
         if (cur.z > 32) {
           t += vote(g.u[j][32 + lane], WT ? g.w[WT ? j : 0][32 + lane] : 1);
-          for (int32_t x = 64 + lane; x < cur.z; x += 32)
-            t += vote(__ldg(col_idx + cur.y + x), WT ? __ldg(wint + cur.y + x) : 1);
+          // the entries from x on: 32 N at a time while more than `over` are left
+          int32_t x = 64;
+          auto tail = [&](auto count, int32_t over) {
+            constexpr int N = decltype(count)::value;
+            for (; cur.z - x > over; x += 32 * N) {
+              int32_t ux[N], wx[N];
+#pragma unroll
+              for (int q = 0; q < N; ++q) {
+                const int32_t at = x + 32 * q + lane;
+                ux[q] = at < cur.z ? __ldg(col_idx + cur.y + at) : -1;
+                wx[q] = WT && at < cur.z ? __ldg(wint + cur.y + at) : 1;
+              }
+#pragma unroll
+              for (int q = 0; q < N; ++q) t += vote(ux[q], wx[q]);
+            }
+          };
+          tail(std::integral_constant<int, 8>{}, 128);
+          tail(std::integral_constant<int, 4>{}, 64);
+          tail(std::integral_constant<int, 1>{}, 0);
         }
         // |sum| <= sum of the row's |w| <= 2^24 (checked when the graph is created)
         const int32_t sum = __reduce_add_sync(0xFFFFFFFFu, t);
         if (lane == 0) {
-          if (SMEM) sides[cur.x] = sum >= 0 ? 1 : 0;
-          else z[(size_t)cur.x * B + b] = sum >= 0 ? 1 : 0;
+          const uint32_t side = sum >= 0 ? 1u : 0u;
+          if (SIDES == GREEDY_BYTES) sides[cur.x] = (uint8_t)side;
+          else if (SIDES == GREEDY_BITS) atomicXor(words + (cur.x >> 4), (2u ^ side) << (2 * (cur.x & 15)));
+          else z[(size_t)cur.x * B + b] = (uint8_t)side;
         }
         __syncwarp();   // the next vertices read this side
       }
     }
     __syncthreads();
   }
-  if (SMEM) {
+  if (SIDES != GREEDY_COLUMN) {
     uint8_t* out = reinterpret_cast<uint8_t*>(ord);
-    for (int i = threadIdx.x; i < n; i += 64) out[i] = sides[i];
+    for (int i = threadIdx.x; i < n; i += 64)
+      out[i] = SIDES == GREEDY_BYTES ? sides[i] : (uint8_t)((words[i >> 4] >> (2 * (i & 15))) & 3u);
   }
 }
 
@@ -671,6 +698,62 @@ int launch_local_search(const deco_graph* g, int32_t B, uint32_t* zbits, int32_t
 
 using namespace deco;
 
+namespace {
+
+// Where the runs keep their sides, by the rounds of runs that each form takes
+// (some ten runs share an SM before they slow each other down) and its time
+// per placement: bytes 1, two bits 1.7 (weights: 1.2), a column of z 4.5 (2.7),
+// 7 (4.2) once the n x B bytes leave L2, or 0.0038 (0.0024) a run where the
+// memory is the limit.  ms, bytes / two bits / column: n = 20 000, degree 10,
+// B = 2 048 5.2 / 5.7 / 9.3; n = 40 000, B = 4 096 31 / 25 / 48; n = 200 000,
+// degree 6, B = 64 19 / 33 / 77, B = 1 024 147 / 101 / 130, B = 4 096 572 / 313
+// / 299; n = 400 000 (no bytes), B = 64 66 / 155, B = 2 048 469 / 312; weights,
+// n = 100 000, B = 256 36 / 22 / 49.  Columns of weighted graphs take windows of
+// 8 vertices where those of 16 hold too few runs on an SM (n = 200 000, B =
+// 4 096: 461 ms with 16, 346 with 8; n = 400 000, B = 1 024: 310 and 325).
+struct GreedyPlan {
+  int sides = GREEDY_COLUMN;
+  size_t smem = 0;       // dynamic shared memory
+  bool narrow = false;   // windows of 8
+};
+
+template <bool WT>
+GreedyPlan greedy_plan(int32_t n, int32_t B) {
+  constexpr size_t windows = 2 * sizeof(GreedyWindow<WT, 16>) + 1024;
+  const size_t limit = (size_t)block_smem_limit();
+  const int64_t sms = device_sm_count();
+  GreedyPlan p;
+  p.narrow = WT && B > sms * (int64_t)((limit + 1024) / windows);
+  double least = std::max((double)n * B > 1e8 ? (WT ? 4.2 : 7.0) : (WT ? 2.7 : 4.5), (WT ? 0.0024 : 0.0038) * B);
+  auto consider = [&](int sides, size_t smem, double placement) {
+    if (smem + windows > limit) return;
+    const int64_t runs = sms * std::min<int64_t>(10, (int64_t)((limit + 1024) / (smem + windows)));
+    const double cost = placement * (double)((B + runs - 1) / runs);
+    if (cost < least) { least = cost; p = GreedyPlan{sides, smem, false}; }
+  };
+  consider(GREEDY_BITS, ((size_t)n + 63) / 64 * 16, WT ? 1.2 : 1.7);
+  consider(GREEDY_BYTES, ((size_t)n + 15) / 16 * 16, 1.0);
+  return p;
+}
+
+// the placement of B runs in the order of `order`: sides in it (run-major), or in z where *columns
+template <bool WT>
+int launch_greedy(const deco_graph* g, int32_t B, int32_t* order, uint8_t* z, bool* columns, cudaStream_t st) {
+  const GreedyPlan p = greedy_plan<WT>(g->n, B);
+  auto fn = p.sides == GREEDY_BYTES  ? k_greedy<WT, GREEDY_BYTES, 16>
+            : p.sides == GREEDY_BITS ? k_greedy<WT, GREEDY_BITS, 16>
+            : WT && p.narrow         ? k_greedy<WT, GREEDY_COLUMN, WT ? 8 : 16>
+                                     : k_greedy<WT, GREEDY_COLUMN, 16>;
+  *columns = p.sides == GREEDY_COLUMN;
+  if (*columns) DECO_CUDA_TRY(cudaMemsetAsync(z, 2, (size_t)g->n * B, st));
+  DECO_CUDA_TRY(allow_smem(fn, 2 * sizeof(GreedyWindow<WT, 16>) + 1024));
+  fn<<<(unsigned)B, 64, p.smem, st>>>(g->n, B, g->row_ptr, g->col_idx, g->wint, order, z);
+  DECO_CUDA_TRY(cudaGetLastError());
+  return DECO_OK;
+}
+
+}  // namespace
+
 extern "C" int deco_greedy(const deco_graph* g, int32_t B, uint64_t seed, uint8_t* z, int64_t* cuts, void* stream) {
   clear_error();
   int rc = check_graph(g);
@@ -695,17 +778,10 @@ extern "C" int deco_greedy(const deco_graph* g, int32_t B, uint64_t seed, uint8_
   if (F.h <= ORDER_MAX_H) k_orders<true><<<ogrid, 256, sizeof(uint16_t) * (4u << F.h), st>>>(F, B, order);
   else k_orders<false><<<ogrid, 256, 0, st>>>(F, B, order);
   DECO_CUDA_TRY(cudaGetLastError());
-  const size_t smem = ((size_t)n + 15) / 16 * 16;
-  // the sides, beside the two windows of loaded rows
-  constexpr size_t windows = 2 * sizeof(GreedyWindow<true>) + 1024;
-  const bool fits = smem + windows <= (size_t)block_smem_limit();
-  auto fn = g->wint ? (fits ? k_greedy<true, true> : k_greedy<true, false>)
-                    : (fits ? k_greedy<false, true> : k_greedy<false, false>);
-  if (fits) DECO_CUDA_TRY(allow_smem(fn, windows));
-  else DECO_CUDA_TRY(cudaMemsetAsync(z, 2, (size_t)n * B, st));
-  fn<<<(unsigned)B, 64, fits ? smem : 0, st>>>(n, B, g->row_ptr, g->col_idx, g->wint, order, z);
-  DECO_CUDA_TRY(cudaGetLastError());
-  if (fits) {
+  bool columns = false;
+  if ((rc = g->wint ? launch_greedy<true>(g, B, order, z, &columns, st) : launch_greedy<false>(g, B, order, z, &columns, st)))
+    return rc;
+  if (!columns) {
     const int64_t tiles = (int64_t)((n + 31) / 32) * W;
     k_sides_out<<<(unsigned)std::min<int64_t>((tiles + 7) / 8, (int64_t)device_sm_count() * 16), 256, 0, st>>>(
         n, B, W, reinterpret_cast<const uint8_t*>(order), z, bits);

@@ -222,3 +222,38 @@ def test_local_search_bit_planes_match_oracle(name, B, rounds):
     np.testing.assert_array_equal(z.cpu().numpy().reshape(g.n, B), Zr)
     np.testing.assert_array_equal(cuts.cpu().numpy(), O.cut_values(g, Zr))
     assert r == rr
+
+
+# A run's sides as bytes, as two bits (several rounds of runs as bytes; graphs too large for bytes) and in the columns of
+# the result (graphs too large for two bits; with weights and many runs in windows of 8 vertices, not 16).
+@pytest.mark.parametrize("n,degree,B", [(7, 3.0, 3), (15, 4.0, 33), (16, 4.0, 33), (17, 4.0, 33), (20001, 6.0, 1024),
+                                        (180001, 3.0, 2560), (250007, 4.0, 2), (900001, 2.0, 1)])
+@pytest.mark.parametrize("weights", [False, True])
+def test_greedy_forms_of_the_sides(n, degree, B, weights):
+    g = gg.er_graph_avg_degree(n, degree, n)
+    if weights:
+        g = _sign(g, [-3.0, 2.0, 6.0])
+    G = deco.graph_from(g)
+    z = torch.zeros(n * B, dtype=torch.uint8, device=DEV)
+    cuts = torch.zeros(B, dtype=torch.int64, device=DEV)
+    deco.deco_greedy(G, B, 5, z, cuts)
+    Z = z.cpu().numpy().reshape(n, B)
+    for b in sorted({0, B - 1}):
+        np.testing.assert_array_equal(Z[:, b], O.greedy_maxcut(g, O.feistel_order(n, b, 5)))
+        assert cuts[b].item() == O.cut_value(g, Z[:, b])
+
+
+# Rows around the lengths at which the entries past the window's 64 are read 256, 128 and 32 at a time.
+@pytest.mark.parametrize("deg", [95, 96, 97, 128, 129, 192, 193, 321, 449, 705])
+@pytest.mark.parametrize("weights", [False, True])
+def test_greedy_tails_of_long_rows(deg, weights):
+    g = _hub_graph(1500, 4, deg, deg)
+    if weights:
+        g = _sign(g, [-3.0, 2.0, 6.0])
+    B = 5
+    z = torch.zeros(g.n * B, dtype=torch.uint8, device=DEV)
+    cuts = torch.zeros(B, dtype=torch.int64, device=DEV)
+    deco.deco_greedy(deco.graph_from(g), B, 3, z, cuts)
+    Zr, cr = O.greedy_batch(g, B, 3)
+    np.testing.assert_array_equal(z.cpu().numpy().reshape(g.n, B), Zr)
+    np.testing.assert_array_equal(cuts.cpu().numpy(), cr)
