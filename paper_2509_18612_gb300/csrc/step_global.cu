@@ -17,17 +17,21 @@
 // the warps that the registers allow, and by instruction issue (78 % with
 // 16-bit blocks before the mixed-precision adds).  So: few registers and many
 // warps; four gathers at once and the last one to three together, not one by
-// one; the own row and momentum loaded ahead of the gathers and the momentum
-// past L2 (evict-first); the sums of +-1 and unit graphs in 16 bits by
-// mixed-precision adds.  us per step, before and after:
+// one; the own row loaded ahead of the gathers, the momentum after them (held
+// through them it costs registers, and spills on +-1 graphs; read past L2,
+// evict-first, it left L2 where the whole block fits there); the sums of +-1
+// and unit graphs in 16 bits by mixed-precision adds; blocks of two warps.  us
+// per step, with eight gathers, a serial tail and the own row last, and here:
 //   n        degree  C    precision  weights   momentum
-//   200 003  12      100  FP32       general   0.9       195 -> 169
-//   200 003  12      128  BF16       unit      0          97 ->  64
-//   200 003  12      128  BF16       unit      0.9       127 ->  97
-//   200 003  12       60  FP32       unit      0          80 ->  54
-//   10^6      8      128  BF16       unit      0         531 -> 352
-//   10^6     10       64  FP32       unit      0.9       535 -> 451
-//   10^6      8       20  FP32       unit      0         248 -> 176
+//   200 003  12      100  FP32       general   0.9       189 -> 160
+//   200 003  12      128  BF16       unit      0          91 ->  61
+//   200 003  12      128  BF16       unit      0.9       121 ->  85
+//   200 003  12       60  FP32       unit      0          75 ->  51
+//   10^6      8      128  BF16       unit      0         522 -> 335
+//   10^6     10       64  FP32       unit      0.9       525 -> 437
+//   10^6      8       20  FP32       unit      0         239 -> 166
+//   700 000   5       40  FP32       +-1       0.9       236 -> 209 (momentum ahead and evict-first 271)
+//   700 000   5        3  BF16       general   0.9        91 ->  84 (99)
 // Eight gathers in flight without momentum cost 5 % on the second and fifth; a
 // loop over rows with the next row's indices prefetched took 136 and 649 us
 // (24 warps an SM); indices held a chunk ahead spill.
@@ -44,6 +48,7 @@ namespace {
 
 struct KArgs {
   int32_t n, C, ld, G, lg;   // G = 2^lg lanes per row
+  int32_t lr;                // 2^lr rows per block
   int32_t ch0;               // first column chunk of the launch
   const int32_t* row_ptr;
   const int32_t* col_idx;
@@ -62,10 +67,10 @@ struct KArgs {
   int32_t* flag;
 };
 
-// Gathers in flight per lane, and blocks per SM (registers): more of both at once does not fit.  With momentum more
-// gathers win over more warps (by 6 % on the sixth graph above; 206 319 nodes, 9 columns, 16-bit 31 against 26 us), and
-// without it on long rows and small grids (4 / 8 gathers: 4 096 nodes of degree 300 45 / 29 us, 8 000 of degree 20
-// 9.2 / 8.1; 200 000 of degree 24, 16-bit 88 / 96).
+// Gathers in flight per lane, and blocks of 256 threads per SM (registers): more of both at once does not fit.  With
+// momentum more gathers win over more warps (206 319 nodes, 9 columns, 16-bit 31 against 26 us), and without it on long
+// rows and small grids (4 / 8 gathers: 4 096 nodes of degree 300 45 / 29 us, 8 000 of degree 20 9.2 / 8.1; 200 000 of
+// degree 24, 16-bit 88 / 96).
 template <bool EIGHT>
 struct Shape {
   static constexpr int U = EIGHT ? 8 : 4;
@@ -104,15 +109,13 @@ __device__ __forceinline__ void add_entry(float (&acc)[VN], uint4 q, uint32_t x,
 // OVERLAP: launched to start while the step before it still runs (programmatic dependent launch).  It then reads the
 // graph ahead of waiting for that step, and the block by plain loads, since others still write it when this kernel
 // starts.  Saves the launch gap of the smaller steps; on large ones the wait ahead of the own row's loads costs 1 - 5 %.
-// us per step without and with: 8 000 nodes, degree 20, 128 columns, FP32 11.2 / 8.8; 5 000, degree 3, 8 columns 5.1 /
-// 4.2; 200 003, degree 12, 60 columns 62 / 54, 100 columns with momentum and general weights 169 / 174.
 template <int PREC, int WMODE, bool MOM, bool LAP, bool EIGHT, bool OVERLAP>
 __global__ void __launch_bounds__(256, Shape<EIGHT>::BLOCKS) k_step_global(const __grid_constant__ KArgs a) {
   using V = VecT<PREC>;
   constexpr int VN = V::N, U = Shape<EIGHT>::U;
   if (OVERLAP) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the next step's blocks may be placed
   const int gl = threadIdx.x & (a.G - 1);         // lane within the group
-  const int64_t row = ((int64_t)blockIdx.x << (8 - a.lg)) + (threadIdx.x >> a.lg);
+  const int64_t row = ((int64_t)blockIdx.x << a.lr) + (threadIdx.x >> a.lg);
   const int32_t c0 = ((a.ch0 + (int32_t)blockIdx.y) * a.G + gl) * VN;   // first column of this lane
   if (row >= a.n || c0 >= a.C) return;
   const int32_t r = (int32_t)row;
@@ -131,17 +134,12 @@ __global__ void __launch_bounds__(256, Shape<EIGHT>::BLOCKS) k_step_global(const
     const uint4* const q = reinterpret_cast<const uint4*>(at);
     return OVERLAP ? *q : __ldg(q);
   };
-  // own row and momentum ahead of the gathers, which hide their latency
+  // own row ahead of the gathers, which hide its latency
   const size_t base = (size_t)r * a.ld + c0;
   const uint4 own = vector(static_cast<const char*>(a.yin) + base * (16 / VN));
-  float vv[VN];
-  if (MOM) {
-#pragma unroll
-    for (int k = 0; k < VN; k += 4) {
-      const float4 q = __ldcs(reinterpret_cast<const float4*>(a.v + base + k));
-      vv[k] = q.x; vv[k + 1] = q.y; vv[k + 2] = q.z; vv[k + 3] = q.w;
-    }
-  }
+  // where it was measured to help (+-1, 16-bit: 2 000 nodes of degree 64, 40 columns 9.8 -> 8.1 us; 700 000 of degree 5,
+  // 3 columns 82 -> 94); general weights in 16 bits lose 13 %, FP32 up to 10 % on narrow blocks
+  if (MOM && PREC == DECO_PREC_BF16 && WMODE == W_SIGN) asm volatile("prefetch.global.L2 [%0];" ::"l"(a.v + base));
   const float dr = LAP ? __ldg(a.dnet + r) : 0.0f;
   const char* const yb = static_cast<const char*>(a.yin) + (size_t)c0 * (16 / VN);
   const uint32_t row_bytes = (uint32_t)a.ld * (16 / VN);
@@ -175,6 +173,15 @@ __global__ void __launch_bounds__(256, Shape<EIGHT>::BLOCKS) k_step_global(const
 #pragma unroll
   for (int q = 0; q < U - 1; ++q)
     if (e + q < e1) add_entry<PREC, WMODE>(acc, raw[q], x[q], w[q]);
+
+  float vv[VN];
+  if (MOM) {
+#pragma unroll
+    for (int k = 0; k < VN; k += 4) {
+      const float4 q = *reinterpret_cast<const float4*>(a.v + base + k);
+      vv[k] = q.x; vv[k + 1] = q.y; vv[k + 2] = q.z; vv[k + 3] = q.w;
+    }
+  }
 
   // ---- epilogue: gradient, momentum, step, projection
   float y[VN], out[VN];
@@ -210,7 +217,7 @@ __global__ void __launch_bounds__(256, Shape<EIGHT>::BLOCKS) k_step_global(const
     if (MOM) {
 #pragma unroll
       for (int k = 0; k < VN; k += 4)
-        __stcs(reinterpret_cast<float4*>(a.v + base + k), make_float4(vv[k], vv[k + 1], vv[k + 2], vv[k + 3]));
+        *reinterpret_cast<float4*>(a.v + base + k) = make_float4(vv[k], vv[k + 1], vv[k + 2], vv[k + 3]);
     }
   } else {
     // ragged last vector: only columns < C are written
@@ -228,7 +235,7 @@ __global__ void __launch_bounds__(256, Shape<EIGHT>::BLOCKS) k_step_global(const
 void launch_k(void (*fn)(const KArgs), const KArgs& a, bool overlap, dim3 grid, cudaStream_t st) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
-  cfg.blockDim = dim3(256, 1, 1);
+  cfg.blockDim = dim3(1u << (a.lr + a.lg), 1, 1);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -294,15 +301,28 @@ int launch_step_global(const StepLaunch& s, cudaStream_t st) {
   if (s.n == 0 || s.C == 0) return DECO_OK;
   const bool mom = s.mu != 0.0f;
   const bool lap = s.objective == DECO_OBJ_LAPLACIAN;
-  // long rows, and grids that leave warps' slots empty anyway: eight gathers in flight
-  const bool eight = s.nnz >= (int64_t)64 * s.n || (int64_t)s.n * s.C <= (int64_t)device_sm_count() * 2048 * VN;
   const int32_t nchunks = (nvec + G - 1) / G;
-  // steps of up to 64 MB of block and momentum (10 - 70 us): the gap between two launches is worth the wait.  Not rows of
-  // 1 024 entries and more, whose gathers the compiler overlaps better as read-only loads (4 096 nodes of degree 2 047,
-  // 128 columns, 16-bit: 205 us overlapping, 110 not; degree 300, FP32 29.5 and 31.8)
-  const bool overlap = s.overlap && nchunks <= 65535 && s.nnz < (int64_t)1024 * s.n &&
+  const int64_t threads = (int64_t)s.n * G * nchunks, sms = device_sm_count();
+  // long rows, and grids that leave warps' slots empty anyway: eight gathers in flight; not where the long rows fill one
+  // wave with four and a second, nearly empty one with eight (3 000 nodes of degree 300, 256 columns: 49 us, here 39)
+  const bool long_rows = s.nnz >= (int64_t)64 * s.n;
+  const bool eight = long_rows ? threads <= 1024 * sms || threads > 1536 * sms : (int64_t)s.n * s.C <= sms * 2048 * VN;
+  // steps of up to 64 MB of block and momentum (10 - 70 us): the gap between two launches is worth the wait.  Not on
+  // longer rows, whose lanes find most of their index words in L1: the waits of the blocks that come in drop them.  The
+  // fewer lanes a row has, the shorter the rows on which this costs more than the gap.  us per step, overlapping and
+  // not: 60 000 nodes of degree 32, 3 columns 27 / 16; 20 000 of degree 24, 11 columns, 16-bit 9.4 / 8.7; 3 000 of
+  // degree 300, 40 columns 37 / 21; 5 000 of degree 100, 40 columns, 16-bit 13 / 11; but 120 000 of degree 6, 3 columns
+  // 10.5 / 10.9; 60 000 of degree 48, 100 columns 62 / 64; 1 000 of degree 200, 40 columns 13.2 / 14.9
+  const int64_t longest = G >= 2 && threads <= 256 * sms                                       ? 1024
+                          : G >= 8 || s.n <= 64 * sms || (G == 4 && threads >= 1024 * sms) ? 80
+                          : G == 4 || (G == 2 && threads >= 1024 * sms)                     ? 28
+                                                                                            : 16;
+  const bool overlap = s.overlap && nchunks <= 65535 && s.nnz < longest * s.n &&
                        (int64_t)s.n * s.C * ((s.precision == DECO_PREC_BF16 ? 2 : 4) + (mom ? 8 : 0)) <= (64 << 20);
-  const unsigned rows = (unsigned)(((int64_t)s.n * G + 255) / 256);
+  // blocks of two warps free their slots sooner (eight warps: 200 003 nodes, 100 columns, momentum 172 us, two 160); where
+  // every block waits for the step before, fewer and larger ones
+  a.lr = (overlap ? (G == 1 ? 8 : 7) : 6) - a.lg;
+  const unsigned rows = (unsigned)(((int64_t)s.n + ((int64_t)1 << a.lr) - 1) >> a.lr);
   for (a.ch0 = 0; a.ch0 < nchunks; a.ch0 += 65535) {
     const dim3 grid(rows, (unsigned)std::min(nchunks - a.ch0, 65535));
     if (s.precision == DECO_PREC_BF16) launch_p<DECO_PREC_BF16>(a, s.wmode, mom, lap, eight, overlap, grid, st);

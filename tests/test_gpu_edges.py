@@ -361,3 +361,31 @@ def test_cuts_of_byte_vectors_match_oracle(name, B, how):
             deco.deco_debug_fail_scratch_alloc(0)
     torch.cuda.synchronize()
     np.testing.assert_array_equal(cuts.cpu().numpy(), O.cut_values(g, Z))
+
+
+# Steps of narrow blocks and long rows, whose launches overlap or not and come in blocks of 64, 128 and 256 threads,
+# against single steps.
+@pytest.mark.parametrize("n,degree,C", [(700, 90.0, 3), (700, 90.0, 9), (700, 90.0, 40), (1900, 200.0, 256), (3001, 40.0, 4),
+                                        (12001, 20.0, 5), (40009, 18.0, 11)])
+@pytest.mark.parametrize("weights", [None, "sign", "weights"])
+@pytest.mark.parametrize("precision", [deco.DECO_PREC_FP32, deco.DECO_PREC_BF16])
+@pytest.mark.parametrize("mu", [0.0, 0.9])
+def test_steps_of_long_rows_and_narrow_blocks_equal_single_steps(n, degree, C, weights, precision, mu):
+    g = gg.er_graph(n, degree / n, 3) if degree >= 90 else gg.er_graph_avg_degree(n, degree, 3)
+    if weights:
+        u, v, _ = g.edges()
+        choices = [-1.0, 1.0] if weights == "sign" else [-3.0, 2.0, 7.0]
+        g = gg.from_edges(g.n, u, v, np.random.default_rng(1).choice(np.array(choices), size=u.size))
+    G = deco.graph_from(g)
+    ld = (C + 7) // 8 * 8
+    y0 = ((torch.rand(n, ld, device=DEV) * 2 - 1) * 0.3).to(torch.bfloat16 if precision else torch.float32)
+    args = deco.step_args(1, precision, 0.0004, mu)
+    a, b, v = y0.clone(), y0.clone(), torch.zeros(n, ld, device=DEV)
+    for _ in range(9):
+        deco.deco_step(G, C, ld, a, b, v if mu else None, args)
+        torch.cuda.synchronize()
+        a, b = b, a
+    y, w = y0.clone(), torch.zeros(n, ld, device=DEV)
+    deco.deco_run_phase(G, C, ld, y, w if mu else None, 9, args, deco.DECO_KERNEL_GLOBAL)
+    assert torch.equal(y[:, :C], a[:, :C]) and torch.equal(y[:, C:], y0[:, C:])
+    assert mu == 0.0 or torch.equal(w, v)
