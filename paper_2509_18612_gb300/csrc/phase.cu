@@ -280,7 +280,7 @@ int plan_phase(const deco_graph* g, int32_t C, int32_t ld, int prec, int force, 
               (long long)g->nnz, ld);
     return DECO_ERR_UNSUPPORTED;
   }
-  if (any_form && aligned && (size_t)(g->n + 1) * 32 <= (size_t)max_smem) {
+  if (any_form && aligned && rows_smem_least(g->n, g->nnz, prec, g->wmode) <= (size_t)max_smem) {
     // the row-vector form, where its estimate is the lowest over its slab widths
     double least = plan->kernel == KERNEL_ONCHIP ? slab_best : step_cycles(g, C, prec);
     std::lock_guard<std::mutex> lock(g_image_mutex);

@@ -342,11 +342,19 @@ void sort_rows(const int32_t* row_ptr, const float* w, int wmode, int32_t row0, 
   }
   order->resize((size_t)n);
   std::iota(order->begin(), order->end(), 0);
-  auto deg = [&](int32_t r) { return row_ptr[row0 + r + 1] - row_ptr[row0 + r]; };
-  std::stable_sort(order->begin(), order->end(), [&](int32_t a, int32_t b) {
-    if (deg(a) != deg(b)) return deg(a) > deg(b);
-    return (*np)[(size_t)a] > (*np)[(size_t)b];
-  });
+  // counting sorts, the second key first: each keeps the order of equal keys
+  std::vector<int32_t> from, at;
+  auto by = [&](auto&& key) {
+    int32_t most = 0;
+    for (int32_t r = 0; r < n; ++r) most = std::max(most, key(r));
+    at.assign((size_t)most + 2, 0);
+    for (int32_t r = 0; r < n; ++r) ++at[(size_t)(most - key(r)) + 1];
+    for (int32_t k = 0; k <= most; ++k) at[(size_t)k + 1] += at[(size_t)k];
+    from = *order;
+    for (int32_t r : from) (*order)[(size_t)at[(size_t)(most - key(r))]++] = r;
+  };
+  if (wmode == W_SIGN) by([&](int32_t r) { return (*np)[(size_t)r]; });
+  by([&](int32_t r) { return row_ptr[row0 + r + 1] - row_ptr[row0 + r]; });
 }
 
 // slice table (4 words a slice) and the sizes of *im
@@ -377,6 +385,10 @@ void slice_table(const int32_t* row_ptr, int wmode, int32_t row0, const std::vec
 }
 
 }  // namespace
+
+size_t rows_smem_least(int32_t n, int64_t nnz, int prec, int wmode) {
+  return 2 * ((size_t)n + 1) * 16 + (size_t)nnz * (wmode == W_GENERAL ? 6 : 2) + (size_t)n * (4 + (prec == DECO_PREC_BF16 ? 32 : 16));
+}
 
 size_t rows_smem_bytes(const RowsImage& im, int prec, bool lap, bool mom) {   // mom: in shared memory
   const size_t rep = (size_t)(im.n + 1) * 16 * im.lpr;

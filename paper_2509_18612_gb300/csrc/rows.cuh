@@ -38,6 +38,8 @@ constexpr int ROWS_MAX_LPR = 8;
 
 // shared memory of a launch: the replicas, image, (lap) net degrees and (mom) momentum
 size_t rows_smem_bytes(const RowsImage& im, int prec, bool lap, bool mom);
+// a lower bound of it (gradients with net degrees, momentum) over all widths, known without the image
+size_t rows_smem_least(int32_t n, int64_t nnz, int prec, int wmode);
 // sizes and counts of the images of rows [row0, row0 + n) for every lpr, nothing uploaded
 void rows_measure(const int32_t* row_ptr, const float* w, int wmode, int32_t row0, int32_t n,
                   std::vector<RowsImage>* out);
