@@ -624,18 +624,40 @@ int deco_probe_wait_timeout(int32_t which, float* waited_ms, void* stream);
  * against concurrent calls.  No paper counterpart.  Errors: DECO_ERR_ARG. */
 int deco_debug_fail_scratch_alloc(int32_t k);
 
-/* Diagnostic for tests of allocation behaviour: the stream-ordered memory pool
- * from which every scratch buffer of the library is taken on the current
- * device.  It is the library's own pool, which keeps up to 256 MiB between
- * calls and gives them back when the last graph is destroyed; where the caller
- * has made another pool the device's current one (cudaDeviceSetMemPool), it is
- * that pool.  used_now (host, or NULL) receives the bytes of
- * the pool in use now, used_high (host, or NULL) the most bytes in use at once
- * since the high-water mark was last reset; reset != 0 then restarts the
- * high-water mark from the current use.  Process-wide (the pool is shared by
+/* Diagnostic for tests of allocation behaviour: the stream-ordered memory pools
+ * from which the scratch buffers of the library are taken on the current
+ * device.  That is the library's own pool, which keeps up to 256 MiB between
+ * calls and gives them back when the last graph is destroyed, and the device's
+ * current pool: where the caller has made another pool the current one
+ * (cudaDeviceSetMemPool), where an allocation from the library's fails, and on
+ * capturing streams.  used_now (host, or NULL) receives the bytes of both in
+ * use now, used_high (host, or NULL) the sum of the most bytes in use at once in
+ * each since the high-water marks were last reset; reset != 0 then restarts the
+ * high-water marks from the current use.  Process-wide (the pools are shared by
  * all calls in the process).  No paper counterpart.
  * Errors: CUDA. */
 int deco_debug_pool_usage(int64_t* used_now, int64_t* used_high, int32_t reset);
+
+/* Diagnostics for tests and profiles: the form in which a phase (or a batch's
+ * phases) of C columns with row stride ld would run under a selector.
+ *  per_column  nonzero: with alpha_cols or steps_cols.
+ *  form        host, receives DECO_FORM_*; a batch's STEPS are the kernels that
+ *              deco_debug_phase_form names for its union.
+ *  width       host or NULL: cluster size (SLAB), 16-byte vectors of a slab row
+ *              (ROWS, ROWS_REG), else 0.
+ * Nothing is built or launched.  No paper counterpart.
+ * Errors: as deco_run_phase. */
+#define DECO_FORM_STEPS 0      /* one launch per step */
+#define DECO_FORM_PIPELINED 1  /* one launch per step, pipelined form */
+#define DECO_FORM_SLAB 2       /* on chip, 128-byte column slabs */
+#define DECO_FORM_SLAB_LEAN 3  /* its lean form */
+#define DECO_FORM_ROWS 4       /* on chip, row-vector form */
+#define DECO_FORM_ROWS_REG 5   /* its form with a row's data in registers */
+#define DECO_FORM_DENSE 6      /* tensor cores */
+int deco_debug_phase_form(const deco_graph* g, int32_t C, int32_t ld, int32_t precision, int32_t per_column,
+                          int32_t kernel, int32_t* form, int32_t* width);
+int deco_debug_batch_form(const deco_batch* b, int32_t C, int32_t ld, int32_t precision, int32_t objective,
+                          int32_t kernel, int32_t* form, int32_t* width);
 
 /* Thread-local message of the last error on this thread ("" if none). */
 const char* deco_last_error(void);

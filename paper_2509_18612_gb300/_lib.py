@@ -53,10 +53,17 @@ DECO_KERNEL_PIPELINED = 1 << 22
 DECO_KERNEL_PIPE_MIXED_ADD = 1 << 30
 DECO_KERNEL_PIPE_L2_HINTS = 1 << 19
 DECO_KERNEL_PIPE_WIDE = 1 << 2
+DECO_FORM_STEPS = 0
+DECO_FORM_PIPELINED = 1
+DECO_FORM_SLAB = 2
+DECO_FORM_SLAB_LEAN = 3
+DECO_FORM_ROWS = 4
+DECO_FORM_ROWS_REG = 5
+DECO_FORM_DENSE = 6
 
 
 def DECO_KERNEL_PIPE_ENTRIES(e: int) -> int:
-    """Entries of a row per stage of the pipelined form: e = 0: 16, 1: 8, 2: 24, 3: 32."""
+    """Entries of a row per stage of the pipelined form: e = 0: 16, 1: 8, 2: 24, 3: 12."""
     return e << 23
 
 
@@ -84,6 +91,7 @@ EXPORTED = [
     "deco_mpnn_train_step", "deco_mpnn_train",
     "deco_idi_mean", "deco_dui_mean", "deco_solve", "deco_solve_budget", "deco_greedy", "deco_local_search",
     "deco_probe_mma_rate", "deco_probe_smem_rate", "deco_probe_wait_timeout", "deco_debug_fail_scratch_alloc", "deco_debug_pool_usage",
+    "deco_debug_phase_form", "deco_debug_batch_form",
     "deco_last_error", "deco_abi_version",
 ]
 
@@ -172,6 +180,8 @@ def _load():
         "deco_probe_wait_timeout": (ctypes.c_int, [I32, P, P]),
         "deco_debug_fail_scratch_alloc": (ctypes.c_int, [I32]),
         "deco_debug_pool_usage": (ctypes.c_int, [P, P, I32]),
+        "deco_debug_phase_form": (ctypes.c_int, [P, I32, I32, I32, I32, I32, P, P]),
+        "deco_debug_batch_form": (ctypes.c_int, [P, I32, I32, I32, I32, I32, P, P]),
         "deco_last_error": (ctypes.c_char_p, []),
         "deco_abi_version": (ctypes.c_int, []),
     }
@@ -383,12 +393,31 @@ def deco_debug_fail_scratch_alloc(k: int):
 
 
 def deco_debug_pool_usage(reset: bool = False):
-    """(bytes in use, high-water mark) of the stream-ordered memory pool that
-    the library's scratch buffers come from on the current device; with
-    reset the high-water mark then restarts from the current use."""
+    """(bytes in use, high-water mark) of the stream-ordered memory pools that
+    the library's scratch buffers come from on the current device (its own and
+    the device's current one); with reset the high-water mark then restarts
+    from the current use."""
     now, high = ctypes.c_int64(), ctypes.c_int64()
     _check(lib.deco_debug_pool_usage(ctypes.byref(now), ctypes.byref(high), 1 if reset else 0))
     return int(now.value), int(high.value)
+
+
+def deco_debug_phase_form(g: Graph, C: int, ld: int, precision: int = DECO_PREC_FP32, per_column: bool = False,
+                          kernel: int = DECO_KERNEL_AUTO):
+    """(DECO_FORM_*, width) in which a phase of C columns would run."""
+    form, width = ctypes.c_int32(), ctypes.c_int32()
+    _check(lib.deco_debug_phase_form(g, int(C), int(ld), int(precision), 1 if per_column else 0, int(kernel),
+                                     ctypes.byref(form), ctypes.byref(width)))
+    return form.value, width.value
+
+
+def deco_debug_batch_form(b: "Batch", C: int, ld: int, precision: int = DECO_PREC_FP32,
+                          objective: int = DECO_OBJ_MULTILINEAR01, kernel: int = DECO_KERNEL_AUTO):
+    """(DECO_FORM_*, width) in which a batch's phases of C columns would run."""
+    form, width = ctypes.c_int32(), ctypes.c_int32()
+    _check(lib.deco_debug_batch_form(b, int(C), int(ld), int(precision), int(objective), int(kernel),
+                                     ctypes.byref(form), ctypes.byref(width)))
+    return form.value, width.value
 
 
 def deco_set_tuning(g: Graph, C: int, precision: int, kernel: int):

@@ -51,17 +51,55 @@ extern "C" int deco_debug_fail_scratch_alloc(int32_t k) {
 
 extern "C" int deco_debug_pool_usage(int64_t* used_now, int64_t* used_high, int32_t reset) {
   clear_error();
-  cudaMemPool_t pool = nullptr;
-  DECO_CUDA_TRY(scratch_pool(&pool));
-  cuuint64_t now = 0, high = 0;
-  DECO_CUDA_TRY(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &now));
-  DECO_CUDA_TRY(cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemHigh, &high));
-  if (used_now) *used_now = (int64_t)now;
-  if (used_high) *used_high = (int64_t)high;
-  if (reset) {
-    cuuint64_t zero = 0;   // the high-water mark restarts from the current use
-    DECO_CUDA_TRY(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrUsedMemHigh, &zero));
+  cudaMemPool_t pools[2] = {nullptr, nullptr};
+  int dev = 0;
+  DECO_CUDA_TRY(scratch_pool(&pools[0]));
+  DECO_CUDA_TRY(cudaGetDevice(&dev));
+  DECO_CUDA_TRY(cudaDeviceGetMemPool(&pools[1], dev));
+  if (used_now) *used_now = 0;
+  if (used_high) *used_high = 0;
+  for (int i = 0; i < (pools[1] == pools[0] ? 1 : 2); ++i) {
+    cuuint64_t now = 0, high = 0;
+    DECO_CUDA_TRY(cudaMemPoolGetAttribute(pools[i], cudaMemPoolAttrUsedMemCurrent, &now));
+    DECO_CUDA_TRY(cudaMemPoolGetAttribute(pools[i], cudaMemPoolAttrUsedMemHigh, &high));
+    if (used_now) *used_now += (int64_t)now;
+    if (used_high) *used_high += (int64_t)high;
+    if (reset) {
+      cuuint64_t zero = 0;   // the high-water mark restarts from the current use
+      DECO_CUDA_TRY(cudaMemPoolSetAttribute(pools[i], cudaMemPoolAttrUsedMemHigh, &zero));
+    }
   }
+  return DECO_OK;
+}
+
+extern "C" int deco_debug_phase_form(const deco_graph* g, int32_t C, int32_t ld, int32_t precision,
+                                     int32_t per_column, int32_t kernel, int32_t* form, int32_t* width) {
+  clear_error();
+  deco_step_args a{};
+  a.precision = precision;
+  int rc = check_step_args(g, C, ld, &a);
+  if (rc) return rc;
+  if (!form) { set_error("form is NULL"); return DECO_ERR_ARG; }
+  if (!valid_selector(kernel)) { set_error("bad kernel selector 0x%x", kernel); return DECO_ERR_ARG; }
+  PhasePlan plan;
+  if ((rc = plan_phase(g, C, ld, precision, kernel, &plan))) return rc;
+  int w = 0;
+  switch (plan.kernel) {
+    case KERNEL_ONCHIP:
+      *form = plan.lean ? DECO_FORM_SLAB_LEAN : DECO_FORM_SLAB;
+      w = plan.k;
+      break;
+    case KERNEL_ROWS:
+      *form = !per_column && rows_in_registers(g, plan.rows_lpr) ? DECO_FORM_ROWS_REG : DECO_FORM_ROWS;
+      w = plan.rows_lpr;
+      break;
+    case KERNEL_DENSE:
+      *form = DECO_FORM_DENSE;
+      break;
+    default:
+      *form = plan.pipe ? DECO_FORM_PIPELINED : DECO_FORM_STEPS;
+  }
+  if (width) *width = w;
   return DECO_OK;
 }
 

@@ -8,8 +8,9 @@
 // [k B/P, (k+1) B/P) and runs T_k steps with alpha_k = 10^{e_k} through the
 // per-column step-size and step-budget arrays of the phase kernels (when
 // every graph's iterate slab fits in shared memory: one on-chip launch whose
-// items are (graph, 128-byte column slab), each graph's replica on chip;
-// otherwise the per-step kernels over the union).  Rounds
+// items are (graph, column slab), each graph's replica on chip, slabs of 1 - 8
+// vectors (k_rows) or of 128 bytes (k_slab); otherwise the per-step kernels
+// over the union).  Rounds
 // alternate the lift as listed (Alg. 3); after every round a device kernel
 // ranks the candidates (sum over graphs of the candidate's best cut) and
 // replaces the bottom half by perturbed copies of the top half, and the next
@@ -403,17 +404,17 @@ int batch_rows_prepare(const deco_batch* b, int32_t C, int32_t ld, int prec, voi
   return DECO_OK;
 }
 
-// ok stays false (nothing allocated) when a member does not fit on chip;
-// any_form: the row-vector form may be taken instead of k_slab
-int batch_slab_prepare(const deco_batch* b, int32_t C, int32_t ld, int prec, void* y, float* v, bool mom_needed,
-                       bool lap, bool any_form, const float* alpha_cols, const int32_t* steps_cols, BatchSlab* bs) {
+// The form of a batch's phases (DECO_FORM_*): per-step kernels over the union
+// where a member does not fit on chip.  any_form: the row-vector form may be
+// taken instead of k_slab (its shape in *bs); lean_ok: k_slab's lean form too.
+int batch_form(const deco_batch* b, int32_t C, int32_t ld, int prec, bool lean_ok, bool lap, bool any_form,
+               BatchSlab* bs) {
   const deco_graph* U = b->U;
-  const int cols = prec == DECO_PREC_BF16 ? 64 : 32;
-  if (ld % cols) return DECO_OK;
+  if (ld % (prec == DECO_PREC_BF16 ? 64 : 32)) return DECO_FORM_STEPS;
   const int max_smem = slab_max_smem();
   int32_t max_n = 0;
   for (int32_t i = 0; i < b->n_graphs; ++i) max_n = std::max(max_n, b->h_goff[i + 1] - b->h_goff[i]);
-  if ((size_t)max_n * 128 + 4096 > (size_t)max_smem) return DECO_OK;
+  if ((size_t)max_n * 128 + 4096 > (size_t)max_smem) return DECO_FORM_STEPS;
   // what k_slab would take: where it does not fit, the per-step kernels run
   int64_t max_words = 0;
   for (int32_t i = 0; i < b->n_graphs; ++i) {
@@ -422,12 +423,23 @@ int batch_slab_prepare(const deco_batch* b, int32_t C, int32_t ld, int prec, voi
     image_sizes(U, 1, &b->h_goff[i], &own, &words, &edges);
     max_words = std::max(max_words, words);
   }
-  if (max_words > (1 << 26)) return DECO_OK;
+  if (max_words > (1 << 26)) return DECO_FORM_STEPS;
+  bs->max_n = max_n;
   const bool staged = slab_smem_bytes(max_n, max_n, (int)max_words, prec) <= (size_t)max_smem;
-  if (!staged && (slab_smem_bytes(max_n, max_n, (int)max_words, prec, true) > (size_t)max_smem || (mom_needed && !v)))
-    return DECO_OK;
-  if (any_form && batch_rows_shape(b, C, prec, lap, bs))
-    return batch_rows_prepare(b, C, ld, prec, y, v, alpha_cols, steps_cols, bs);
+  if (!staged && (slab_smem_bytes(max_n, max_n, (int)max_words, prec, true) > (size_t)max_smem || !lean_ok))
+    return DECO_FORM_STEPS;
+  if (any_form && batch_rows_shape(b, C, prec, lap, bs)) return DECO_FORM_ROWS;
+  return staged ? DECO_FORM_SLAB : DECO_FORM_SLAB_LEAN;
+}
+
+// ok stays false (nothing allocated) when the per-step kernels run
+int batch_slab_prepare(const deco_batch* b, int32_t C, int32_t ld, int prec, void* y, float* v, bool mom_needed,
+                       bool lap, bool any_form, const float* alpha_cols, const int32_t* steps_cols, BatchSlab* bs) {
+  const deco_graph* U = b->U;
+  const int form = batch_form(b, C, ld, prec, !mom_needed || v, lap, any_form, bs);
+  if (form == DECO_FORM_STEPS) return DECO_OK;
+  if (form == DECO_FORM_ROWS) return batch_rows_prepare(b, C, ld, prec, y, v, alpha_cols, steps_cols, bs);
+  const int cols = prec == DECO_PREC_BF16 ? 64 : 32;
   std::vector<SlabGraph> hg((size_t)b->n_graphs);
   const int32_t slabs = (C + cols - 1) / cols;
   const size_t esz = elem_size(prec);
@@ -456,9 +468,8 @@ int batch_slab_prepare(const deco_batch* b, int32_t C, int32_t ld, int prec, voi
     sg.steps_cols = steps_cols;
   }
   const std::vector<int2> items = batch_items(b, C, cols);
-  bs->max_n = max_n;
   cudaError_t e = cudaSuccess;
-  if (!staged) {
+  if (form == DECO_FORM_SLAB_LEAN) {
     bs->lean = true;
     e = cudaMalloc((void**)&bs->xbuf, (size_t)2 * slabs * U->n * 128);
     if (e != cudaSuccess) {
@@ -561,6 +572,23 @@ extern "C" void deco_destroy_batch(deco_batch* b) {
   deco_destroy_graph(b->U);
   for (auto& br : b->rows) cudaFree(br.data);
   delete b;
+}
+
+extern "C" int deco_debug_batch_form(const deco_batch* b, int32_t C, int32_t ld, int32_t precision, int32_t objective,
+                                     int32_t kernel, int32_t* form, int32_t* width) {
+  clear_error();
+  int rc = 0;
+  if (!b || !form || C < 1 || ld < C) { set_error("bad arguments"); return DECO_ERR_ARG; }
+  if ((rc = check_prec(precision)) || (rc = check_obj(objective))) return rc;
+  if (!valid_selector(kernel)) { set_error("bad kernel selector 0x%x", kernel); return DECO_ERR_ARG; }
+  BatchSlab bs;
+  const int kind = kernel & 0x3;
+  *form = DECO_FORM_STEPS;
+  if (kind == DECO_KERNEL_AUTO || kind == DECO_KERNEL_ONCHIP)
+    *form = batch_form(b, C, ld, precision, true, objective == DECO_OBJ_LAPLACIAN,
+                       kernel == DECO_KERNEL_AUTO || kernel == DECO_KERNEL_ONCHIP, &bs);
+  if (width) *width = *form == DECO_FORM_ROWS ? bs.lpr : *form == DECO_FORM_STEPS ? 0 : 1;
+  return DECO_OK;
 }
 
 extern "C" int deco_batch_graph(const deco_batch* b, const deco_graph** out) {

@@ -329,6 +329,13 @@ static int plan_captured(const deco_graph* g, int32_t C, int32_t ld, int prec, i
   return plan_phase(g, C, ld, prec, chosen ? DECO_KERNEL_ONCHIP | DECO_KERNEL_THREADS_1024 : DECO_KERNEL_GLOBAL, plan);
 }
 
+bool rows_in_registers(const deco_graph* g, int lpr) {
+  std::lock_guard<std::mutex> lock(g_image_mutex);
+  for (const RowsImage& im : g->rows_sizes)
+    if (im.lpr == lpr) return rows_reg_fits(im, g->wmode);
+  return false;
+}
+
 int PhaseRunner::prepare(const deco_graph* g_, int32_t C_, int32_t ld_, int prec_, int force,
                          cudaStream_t st) {
   g = g_;

@@ -48,6 +48,9 @@ void record_tuning(const deco_graph* g, int32_t C, int prec, int kernel);
 // force: DECO_KERNEL_* optionally | DECO_KERNEL_CLUSTER(k)
 int plan_phase(const deco_graph* g, int32_t C, int32_t ld, int prec, int force, PhasePlan* plan);
 
+// the planned row-vector form of slab width lpr keeps its rows in registers (without per-column step sizes and budgets)
+bool rows_in_registers(const deco_graph* g, int lpr);
+
 struct PhaseRunner {
   const deco_graph* g = nullptr;
   int32_t C = 0, ld = 0;

@@ -153,3 +153,9 @@ def test_smem_probe_rejects_bad_arguments(deco):
     for width, iters in ((4, 64), (16, 0), (16, 12), (8, (1 << 24) + 8)):
         assert deco.lib.deco_probe_smem_rate(width, iters, ctypes.byref(gbs), None) == deco.DECO_ERR_ARG
     assert deco.lib.deco_probe_smem_rate(16, 64, None, None) == deco.DECO_ERR_ARG
+
+
+def test_form_queries_reject_bad_arguments(deco):
+    f = ctypes.c_int32()
+    assert deco.lib.deco_debug_phase_form(None, 8, 8, 0, 0, 0, ctypes.byref(f), None) == deco.DECO_ERR_ARG
+    assert deco.lib.deco_debug_batch_form(None, 8, 8, 0, 0, 0, ctypes.byref(f), None) == deco.DECO_ERR_ARG

@@ -628,11 +628,9 @@ def test_batch_kernels_and_replay_agree():
 @pytest.mark.parametrize("sizes", [(150, 300), (300, 1150)])
 def test_batch_onchip_items_equal_the_union_per_step_kernel(precision, sizes):
     # 40 graphs whose union does not fit in shared memory while every member
-    # does: the default runs one on-chip launch (row-pair form) with an item
-    # per (graph, 128-byte column slab) -- with graphs of up to 1 150 rows in
-    # the lean form (momentum in global memory, replica refreshed from L2); the
-    # per-step kernel over the union performs the same FP32 operations in the
-    # same order
+    # does: the default runs one on-chip launch with an item per (graph, column
+    # slab) in the form that the planner takes; the per-step kernel over the
+    # union performs the same FP32 operations in the same order
     rng = np.random.default_rng(77)
     graphs = [gg.ba_graph(int(n), 4, 700 + i) for i, n in enumerate(rng.integers(sizes[0], sizes[1], 40))]
     batch = deco.deco_create_batch([deco.graph_from(g) for g in graphs])

@@ -3,8 +3,8 @@ with short rows or few starts) against the per-step kernel: the same FP32
 operations in the same order, so the blocks are bit-identical.
 
 The planner takes slab widths of 1, 2, 4 or 8 vectors by the number of
-columns: on a graph of 100 rows 64, 1 024, 3 000 and 9 000 columns take one
-width each; more columns than the GPU holds at once run in several waves."""
+columns, and more columns than the GPU holds at once run in several waves; the
+tests ask the library which form and width a call takes."""
 import numpy as np
 import pytest
 
@@ -112,3 +112,66 @@ def test_batched_row_vector_form_equals_the_other_forms(precision, kind, objecti
             outs.append((best.tolist(), ex["assignment"].tobytes(), ex["round_cuts"].tobytes(),
                          ex["round_scores"].tobytes(), ex["final_T"].tobytes()))
     assert all(o == outs[0] for o in outs)
+
+
+FORM_COLUMNS = (64, 500, 800, 1024, 1300, 1600, 2000, 2400, 3000, 4000, 5000, 6000, 7000, 9000)
+
+
+# Every width of the form, for every storage of the weights, with a row's data in registers where the planner takes that
+# (not with per-column step sizes), against the per-step kernel.
+@pytest.mark.parametrize("name,registers", [("er100", True), ("isolated", True), ("sign", False), ("weights", False)])
+@pytest.mark.parametrize("precision", [deco.DECO_PREC_FP32, deco.DECO_PREC_BF16])
+@pytest.mark.parametrize("width", [1, 2, 4, 8])
+def test_every_width_of_the_row_vector_form_equals_the_per_step_kernel(name, registers, precision, width):
+    g = GRAPHS[name]()
+    G = deco.graph_from(g)
+
+    def form(C, cols):
+        return deco.deco_debug_phase_form(G, C, (C + 63) // 64 * 64, precision, cols)
+
+    taken = [C for C in FORM_COLUMNS if form(C, True) == (deco.DECO_FORM_ROWS, width)]
+    if name == "isolated" and width == 8:
+        assert not taken   # 90 rows of up to 2 entries: never worth more than 4 vectors at these columns
+        return
+    C = taken[0]
+    if registers:
+        assert form(C, False) == (deco.DECO_FORM_ROWS_REG, width)
+    else:
+        assert form(C, False)[0] in (deco.DECO_FORM_ROWS, deco.DECO_FORM_ROWS_REG)
+    ld = (C + 63) // 64 * 64
+    y0 = ((torch.rand(g.n, ld, device=DEV) * 2 - 1) * 0.3).to(torch.bfloat16 if precision else torch.float32)
+    alpha = torch.rand(C, device=DEV) * 0.02
+    budget = torch.randint(0, 8, (C,), device=DEV, dtype=torch.int32)
+    for cols in (False, True):
+        args = deco.step_args(1, precision, 0.01, 0.9, alpha_cols=alpha if cols else None,
+                              steps_cols=budget if cols else None)
+        out = []
+        for kernel in (deco.DECO_KERNEL_GLOBAL, deco.DECO_KERNEL_AUTO):
+            y, v = y0.clone(), torch.zeros(g.n, ld, device=DEV)
+            deco.deco_run_phase(G, C, ld, y, v, 7, args, kernel=kernel)
+            out.append((y, v))
+        assert torch.equal(out[1][0], out[0][0]) and torch.equal(out[1][1], out[0][1])
+
+
+# The batched forms by name: the planner's row-vector form, and k_slab (demanded by a modifier, which takes a union that
+# fits on chip as well) with its staging area or, for members of 620 rows, lean.  Four candidates of 32 columns: slabs
+# stop at budgets of their own.
+@pytest.mark.parametrize("precision", [deco.DECO_PREC_FP32, deco.DECO_PREC_BF16])
+@pytest.mark.parametrize("sizes,slab", [((200, 150, 33, 120), deco.DECO_FORM_SLAB), ((620, 200), deco.DECO_FORM_SLAB_LEAN)])
+@pytest.mark.parametrize("mu", [0.0, 0.9])
+@pytest.mark.parametrize("weights", [None, [-1.0, 1.0], [-3.0, 2.0, 7.0]])
+def test_batched_forms_equal_the_per_step_kernels(precision, sizes, slab, mu, weights):
+    graphs = [gg.ba_graph(n, 2, 800 + n) for n in sizes]
+    if weights:
+        graphs = [_weighted(g, weights, g.n) for g in graphs]
+    batch = deco.deco_create_batch([deco.graph_from(g) for g in graphs])
+    pairs = deco.DECO_KERNEL_ONCHIP | deco.DECO_KERNEL_ROW_PAIRS
+    assert deco.deco_debug_batch_form(batch, 128, 128, precision, kernel=pairs)[0] == slab
+    assert deco.deco_debug_batch_form(batch, 128, 128, precision)[0] == deco.DECO_FORM_ROWS
+    pop = deco.population(candidates=4, rounds=3, t_lo=1, t_hi=50, e_lo=-2.5, e_hi=-1.5, momentum=mu, lifts=(1, 2))
+    outs = []
+    for kernel in (deco.DECO_KERNEL_GLOBAL, pairs, deco.DECO_KERNEL_AUTO):
+        p = deco.params(objective=deco.DECO_OBJ_LAPLACIAN, init=deco.DECO_INIT_IDI, precision=precision, kernel=kernel)
+        _, best, ex = deco.deco_solve_batch(batch, 128, p, pop, 9, want_assignment=True, want_round_cuts=True)
+        outs.append((best.tolist(), ex["assignment"].tobytes(), ex["round_cuts"].tobytes(), ex["round_scores"].tobytes()))
+    assert outs[1] == outs[0] and outs[2] == outs[0]

@@ -164,7 +164,7 @@ def _hub_graph(n, hubs, deg, seed):
 @pytest.mark.parametrize("n", [2, 31, 32, 33, 40, 65])
 @pytest.mark.parametrize("weights", [False, True])
 def test_greedy_windows_of_vertices(n, weights):
-    # windows of 32 vertices, neighbours loaded 8 vertices ahead, across the ends of windows and orderings
+    # windows of 16 vertices, the next one loaded meanwhile, across the ends of windows and orderings
     g = signed_graph(n, 0.5, n) if weights else gg.er_graph(n, 0.5, n)
     B = 33
     z = torch.zeros(n * B, dtype=torch.uint8, device=DEV)
