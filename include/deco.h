@@ -83,12 +83,19 @@ typedef enum deco_status {
 #define DECO_INIT_MEAN 5
 
 /* Kernel used for the steps of a phase.
- *  AUTO    the persistent on-chip kernel when a 128-byte column slab of the
- *          graph (plus its share of the CSR) fits in shared memory, else one
- *          launch of the global-memory kernel per step
+ *  AUTO    what cost estimates put first: a persistent on-chip kernel (all
+ *          steps in one launch) where the graph fits, in one of two forms, else
+ *          one launch of the global-memory kernel per step.  The slab form
+ *          keeps 128-byte column slabs (and its share of the CSR) in shared
+ *          memory, over a cluster of CTAs where one does not hold them; the
+ *          row-vector form slabs of 1, 2, 4 or 8 16-byte vectors in one CTA
+ *          each (up to some 4 000 rows).  On a capturing stream, where nothing
+ *          may be allocated, a graph's first call of a form takes the
+ *          global-memory kernel
  *  GLOBAL  always the per-step global-memory kernel
- *  ONCHIP  always the persistent on-chip kernel (DECO_ERR_UNSUPPORTED if it
- *          does not fit)
+ *  ONCHIP  always a persistent on-chip kernel (DECO_ERR_UNSUPPORTED if the slab
+ *          form does not fit); without modifiers in the form that the
+ *          estimates put first, with one in the slab form
  *  DENSE   (BF16 blocks) the tensor-core kernel for dense graphs: A Y as a
  *          dense BF16 x BF16 -> FP32 product on the 5th-generation tensor
  *          cores (tcgen05, accumulator in tensor memory) with the update
@@ -138,7 +145,8 @@ typedef enum deco_status {
  * own row (every lane on 8 bytes of the 128-byte replica row), so a warp
  * advances two rows at a time and one shared load serves an entry of each.
  * Same iterates as the other forms.  DECO_KERNEL_AUTO without a recorded
- * tuning, and the batched on-chip launch of deco_solve_batch, use this form. */
+ * tuning, and the batched on-chip launch of deco_solve_batch, use this form
+ * where they take the slab form. */
 #define DECO_KERNEL_ROW_PAIRS (1 << 21)
 /* With DECO_KERNEL_GLOBAL (optionally with column slabs), the pipelined form
  * of the per-step kernel: rows sorted by degree in slices of 32 / G rows (G
@@ -264,16 +272,17 @@ int deco_step(const deco_graph* g, int32_t C, int32_t ld, const void* y_in, void
  *          gave up (the block is then unreliable).
  * Stream-ordered and asynchronous; scratch memory (exchange buffers, the
  * second block of the global kernel) is allocated and released in stream
- * order.  The first use of a graph with a given cluster size builds its
- * on-chip CSR image on the host (kept with the graph).
+ * order.  The first use of a graph with a given cluster size or slab width
+ * builds its on-chip image on the host (kept with the graph).
  * Errors: DECO_ERR_ARG, DECO_ERR_UNSUPPORTED (ONCHIP does not fit, DENSE
  * outside its limits), CUDA. */
 int deco_run_phase(const deco_graph* g, int32_t C, int32_t ld, void* y, float* v, int32_t steps,
                    const deco_step_args* a, int32_t kernel, int32_t* nonfinite_flag, void* stream);
 
 /* Autotuner: times every feasible launch shape of a phase on this graph --
- * the per-step global kernel, the on-chip kernel for each cluster size
- * (1, 2, 4, 8), CTA size (512, 1024) and exchange mode (DSMEM, L2), and, for
+ * the per-step global kernel, the on-chip form that the cost estimates put
+ * first, its slab form for each cluster size (1, 2, 4, 8), CTA size (512,
+ * 1024) and exchange mode (DSMEM, L2), and, for
  * BF16 blocks of graphs with nnz >= n^2 / 64 inside the DENSE limits, the
  * tensor-core kernel for each contraction split (1, 2, 4, 8) -- over
  * `probe_steps` steps of a C-column block with the given precision,

@@ -215,8 +215,7 @@ __global__ void __launch_bounds__(512) k_layer(const __grid_constant__ LayerArgs
       const int r = ty + 16 * i, v = v0 + r;
       float acc[4] = {0.f, 0.f, 0.f, 0.f};
       if (v < a.n) {
-        csr_gather_row<DECO_PREC_FP32, WMODE>(a.A, a.in1, H, 4 * tx, __ldg(a.row_ptr + v), __ldg(a.row_ptr + v + 1),
-                                              acc);
+        csr_gather_row<WMODE>(a.A, a.in1, H, 4 * tx, __ldg(a.row_ptr + v), __ldg(a.row_ptr + v + 1), acc);
         const float s = __ldg(a.dinv + v);
 #pragma unroll
         for (int c = 0; c < 4; ++c) acc[c] *= s;
@@ -338,7 +337,7 @@ __global__ void __launch_bounds__(512) k_back(const __grid_constant__ BackArgs a
 #pragma unroll
         for (int c = 0; c < 4; ++c) d[c] = s_dout[r] * __ldg(a.wo + 4 * tx + c);
       } else {
-        csr_gather_row<DECO_PREC_FP32, WMODE>(a.A, a.T, H, 4 * tx, __ldg(a.row_ptr + v), __ldg(a.row_ptr + v + 1), d);
+        csr_gather_row<WMODE>(a.A, a.T, H, 4 * tx, __ldg(a.row_ptr + v), __ldg(a.row_ptr + v + 1), d);
         const float4 s = *reinterpret_cast<const float4*>(a.S + (size_t)v * H + 4 * tx);
         d[0] += s.x; d[1] += s.y; d[2] += s.z; d[3] += s.w;
       }

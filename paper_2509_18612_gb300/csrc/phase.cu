@@ -1,7 +1,7 @@
 // One phase of projected gradient ascent (the step loop of Alg. 1 / Alg. 2): T steps
-// on a device block, by the persistent on-chip kernel (slab.cu) when one
-// column slab of the graph fits in shared memory, otherwise by one launch of
-// the global-memory kernel (step_global.cu) per step.
+// on a device block, by a persistent on-chip kernel (slab.cu, rows.cu,
+// rows_reg.cu) when a column slab of the graph fits in shared memory, otherwise
+// by one launch of the global-memory kernel (step_global.cu) per step.
 #include <algorithm>
 #include <mutex>
 #include <new>
