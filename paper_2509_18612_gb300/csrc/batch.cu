@@ -361,7 +361,7 @@ int batch_rows_images(const deco_batch* b, int lpr, const BatchRows** out) {
   }
   cudaError_t e = cudaMalloc((void**)&br.data, all.size() * 4);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(batch row images)");
-  e = cudaMemcpy(br.data, all.data(), all.size() * 4, cudaMemcpyHostToDevice);
+  e = upload(br.data, all.data(), all.size() * 4);
   if (e != cudaSuccess) {
     cudaFree(br.data);
     return cuda_fail(e, "cudaMemcpy(batch row images)");
@@ -393,8 +393,8 @@ int batch_rows_prepare(const deco_batch* b, int32_t C, int32_t ld, int prec, voi
   const std::vector<int2> items = batch_items(b, C, bs->lpr * (prec == DECO_PREC_BF16 ? 8 : 4));
   cudaError_t e = cudaMalloc((void**)&bs->d_rows, sizeof(RowsGraph) * hg.size());
   if (e == cudaSuccess) e = cudaMalloc((void**)&bs->d_items, sizeof(int2) * items.size());
-  if (e == cudaSuccess) e = cudaMemcpy(bs->d_rows, hg.data(), sizeof(RowsGraph) * hg.size(), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(bs->d_items, items.data(), sizeof(int2) * items.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = upload(bs->d_rows, hg.data(), sizeof(RowsGraph) * hg.size());
+  if (e == cudaSuccess) e = upload(bs->d_items, items.data(), sizeof(int2) * items.size());
   if (e != cudaSuccess) {
     bs->release();
     return cuda_fail(e, "batch on-chip parameters");
@@ -480,8 +480,8 @@ int batch_slab_prepare(const deco_batch* b, int32_t C, int32_t ld, int prec, voi
   }
   e = cudaMalloc((void**)&bs->d_graphs, sizeof(SlabGraph) * hg.size());
   if (e == cudaSuccess) e = cudaMalloc((void**)&bs->d_items, sizeof(int2) * items.size());
-  if (e == cudaSuccess) e = cudaMemcpy(bs->d_graphs, hg.data(), sizeof(SlabGraph) * hg.size(), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMemcpy(bs->d_items, items.data(), sizeof(int2) * items.size(), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = upload(bs->d_graphs, hg.data(), sizeof(SlabGraph) * hg.size());
+  if (e == cudaSuccess) e = upload(bs->d_items, items.data(), sizeof(int2) * items.size());
   if (e != cudaSuccess) {
     bs->release();
     return cuda_fail(e, "batch on-chip parameters");
@@ -541,7 +541,7 @@ extern "C" int deco_create_batch(const deco_graph* const* graphs, int32_t n_grap
   }
   auto up = [&](void** dst, const void* src, size_t bytes) -> cudaError_t {
     cudaError_t e2 = cudaMalloc(dst, bytes);
-    if (e2 == cudaSuccess) e2 = cudaMemcpy(*dst, src, bytes, cudaMemcpyHostToDevice);
+    if (e2 == cudaSuccess) e2 = upload(*dst, src, bytes);
     return e2;
   };
   cudaError_t e = up((void**)&b->gid, gid.data(), sizeof(int32_t) * (size_t)n);

@@ -67,6 +67,14 @@ cudaError_t allow_smem(F fn, size_t fixed = 1024) {
   return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, block_smem_limit() - (int)fixed);
 }
 
+// Host memory to the device, there for every stream on return.  A cudaMemcpy from pageable memory may return with the
+// data staged and not yet copied, in the order of the legacy default stream alone: a kernel on a non-blocking stream
+// could read the destination before it is written.
+inline cudaError_t upload(void* dst, const void* src, size_t bytes) {
+  const cudaError_t e = cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice);
+  return e != cudaSuccess ? e : cudaStreamSynchronize(cudaStreamLegacy);
+}
+
 #define DECO_CUDA_TRY(expr)                                   \
   do {                                                        \
     cudaError_t _e = (expr);                                  \

@@ -343,6 +343,9 @@ int deco::create_graph_impl(int32_t n, int64_t nnz, const int32_t* row_ptr, cons
       rc = DECO_ERR_GRAPH;
     }
   }
+  // the arrays are there for every stream (upload, deco_internal.cuh; once for all of them)
+  if (rc == DECO_OK)
+    if (cudaError_t e = cudaStreamSynchronize(cudaStreamLegacy)) rc = cuda_fail(e, "graph upload");
   if (rc != DECO_OK) {
     free_graph(g);
     return rc;

@@ -858,9 +858,9 @@ extern "C" int deco_mpnn_set_params(deco_mpnn* m, const float* host, int64_t cou
   int rc = check_model(m);
   if (rc) return rc;
   if (!host || count != m->n_params) { set_error("need a host buffer of %lld floats", (long long)m->n_params); return DECO_ERR_ARG; }
-  DECO_CUDA_TRY(cudaMemcpy(m->theta, host, sizeof(float) * count, cudaMemcpyHostToDevice));
   DECO_CUDA_TRY(cudaMemset(m->m, 0, sizeof(float) * count));
   DECO_CUDA_TRY(cudaMemset(m->v, 0, sizeof(float) * count));
+  DECO_CUDA_TRY(upload(m->theta, host, sizeof(float) * count));   // and the moments: there for every stream
   m->t = 0;
   return DECO_OK;
 }

@@ -461,7 +461,7 @@ int rows_image(deco_graph* g, int lpr, const RowsImage** out) {
              &im, &host);
   cudaError_t e = cudaMalloc((void**)&im.data, host.size() * 4);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(row image)");
-  e = cudaMemcpy(im.data, host.data(), host.size() * 4, cudaMemcpyHostToDevice);
+  e = upload(im.data, host.data(), host.size() * 4);
   if (e != cudaSuccess) {
     cudaFree(im.data);
     return cuda_fail(e, "cudaMemcpy(row image)");

@@ -675,7 +675,7 @@ int slab_image_rows(const int32_t* row_ptr, const int32_t* col, const float* w, 
   for (int i = k + 1; i <= SLAB_MAX_CLUSTER; ++i) im.off[i] = im.off[k];
   cudaError_t e = cudaMalloc((void**)&im.data, words.size() * 4);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(slab image)");
-  e = cudaMemcpy(im.data, words.data(), words.size() * 4, cudaMemcpyHostToDevice);
+  e = upload(im.data, words.data(), words.size() * 4);
   if (e != cudaSuccess) {
     cudaFree(im.data);
     return cuda_fail(e, "cudaMemcpy(slab image)");

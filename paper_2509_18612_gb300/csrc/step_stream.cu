@@ -237,7 +237,7 @@ int stream_image(deco_graph* g, const StreamShape& sh, const StreamImage** out) 
   cudaFree(d_order);
   cudaFree(d_srec);
   if (e == cudaSuccess) e = cudaMalloc((void**)&im.soff, soff.size() * 4);
-  if (e == cudaSuccess) e = cudaMemcpy(im.soff, soff.data(), soff.size() * 4, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = upload(im.soff, soff.data(), soff.size() * 4);
   if (e != cudaSuccess) {
     free_stream_image(im);
     return cuda_fail(e, "sliced record image");

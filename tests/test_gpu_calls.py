@@ -135,3 +135,27 @@ def test_phases_captured_before_their_images_are_built(n, degree, warm, C, kerne
         graph.replay()
         torch.cuda.synchronize()
         assert torch.equal(y, ref) and torch.equal(v, vref)
+
+
+# What a call uploads for its first launch (the graph's arrays, an image of its rows) is there for a stream that does not
+# wait for the default one.
+@pytest.mark.parametrize("n,degree,C,kernel", [
+    (800, 5.0, 64, deco.DECO_KERNEL_ONCHIP), (800, 48.0, 64, deco.DECO_KERNEL_AUTO),
+    (1200, 5.0, 64, SLAB), (30000, 40.0, 8, deco.DECO_KERNEL_GLOBAL), (30000, 12.0, 64, deco.DECO_KERNEL_AUTO)])
+def test_first_phase_on_a_non_blocking_stream(n, degree, C, kernel):
+    edges = gg.er_graph_avg_degree(n, degree, 1)
+    args = deco.step_args(0, deco.DECO_PREC_FP32, 0.01, 0.9)
+    y0 = torch.rand(n, C, device=DEV) - 0.5
+    ref, vref = y0.clone(), torch.zeros(n, C, device=DEV)
+    G = deco.graph_from(edges)
+    torch.cuda.synchronize()
+    deco.deco_run_phase(G, C, C, ref, vref, 5, args, deco.DECO_KERNEL_GLOBAL)
+    torch.cuda.synchronize()
+    stream = torch.cuda.Stream()
+    for _ in range(5):
+        y, v = y0.clone(), torch.zeros(n, C, device=DEV)
+        torch.cuda.synchronize()
+        first = deco.graph_from(edges)   # held until the stream has run
+        deco.deco_run_phase(first, C, C, y, v, 5, args, kernel, stream=stream.cuda_stream)
+        stream.synchronize()
+        assert torch.equal(y, ref) and torch.equal(v, vref)
