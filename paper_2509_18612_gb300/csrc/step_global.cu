@@ -319,9 +319,8 @@ int launch_step_global(const StepLaunch& s, cudaStream_t st) {
                                                                                             : 16;
   const bool overlap = s.overlap && nchunks <= 65535 && s.nnz < longest * s.n &&
                        (int64_t)s.n * s.C * ((s.precision == DECO_PREC_BF16 ? 2 : 4) + (mom ? 8 : 0)) <= (64 << 20);
-  // blocks of two warps free their slots sooner (200 003 nodes, 100 columns, momentum, multilinear: eight
-  // warps 172 us, two 160; with the Laplacian's degrees 170 and 170); where
-  // every block waits for the step before, fewer and larger ones
+  // blocks of two warps free their slots sooner (200 003 nodes, 100 columns, momentum, multilinear: eight warps 172 us,
+  // two 160; with the Laplacian's degrees 170 and 170); where every block waits for the step before, fewer and larger
   a.lr = (overlap ? (G == 1 ? 8 : 7) : 6) - a.lg;
   const unsigned rows = (unsigned)(((int64_t)s.n + ((int64_t)1 << a.lr) - 1) >> a.lr);
   for (a.ch0 = 0; a.ch0 < nchunks; a.ch0 += 65535) {
