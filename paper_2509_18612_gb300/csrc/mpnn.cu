@@ -34,7 +34,7 @@ struct deco_mpnn {
   int64_t n_params = 0;
   float* theta = nullptr;   // device parameters (flat, see mpnn oracle layout)
   float* m = nullptr;       // Adam first moment
-  float* v = nullptr;       // Adam second moment
+  float* v = nullptr;       // Adam second moment, behind the first
   int64_t t = 0;            // Adam step count
 };
 
@@ -782,12 +782,11 @@ extern "C" int deco_mpnn_create(int32_t hidden, int32_t layers, uint64_t seed, d
   const Layout lo = layout(hidden, layers);
   m->n_params = lo.total;
   cudaError_t e = cudaMalloc((void**)&m->theta, sizeof(float) * lo.total);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&m->m, sizeof(float) * lo.total);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&m->v, sizeof(float) * lo.total);
-  if (e == cudaSuccess) e = cudaMemset(m->m, 0, sizeof(float) * lo.total);
-  if (e == cudaSuccess) e = cudaMemset(m->v, 0, sizeof(float) * lo.total);
+  if (e == cudaSuccess) e = cudaMalloc((void**)&m->m, 2 * sizeof(float) * lo.total);   // both moments
+  if (e == cudaSuccess) e = cudaMemset(m->m, 0, 2 * sizeof(float) * lo.total);
+  if (e == cudaSuccess) m->v = m->m + lo.total;
   if (e != cudaSuccess) {
-    cudaFree(m->theta); cudaFree(m->m); cudaFree(m->v);
+    cudaFree(m->theta); cudaFree(m->m);
     delete m;
     return cuda_fail(e, "model allocation");
   }
@@ -819,7 +818,7 @@ extern "C" int deco_mpnn_create(int32_t hidden, int32_t layers, uint64_t seed, d
   cudaFree(dr);
   cudaFree(db);
   if (e != cudaSuccess) {
-    cudaFree(m->theta); cudaFree(m->m); cudaFree(m->v);
+    cudaFree(m->theta); cudaFree(m->m);
     delete m;
     return cuda_fail(e, "model initialisation");
   }
@@ -831,7 +830,6 @@ extern "C" void deco_mpnn_destroy(deco_mpnn* m) {
   if (!m) return;
   cudaFree(m->theta);
   cudaFree(m->m);
-  cudaFree(m->v);
   delete m;
 }
 
@@ -858,8 +856,7 @@ extern "C" int deco_mpnn_set_params(deco_mpnn* m, const float* host, int64_t cou
   int rc = check_model(m);
   if (rc) return rc;
   if (!host || count != m->n_params) { set_error("need a host buffer of %lld floats", (long long)m->n_params); return DECO_ERR_ARG; }
-  DECO_CUDA_TRY(cudaMemset(m->m, 0, sizeof(float) * count));
-  DECO_CUDA_TRY(cudaMemset(m->v, 0, sizeof(float) * count));
+  DECO_CUDA_TRY(cudaMemset(m->m, 0, 2 * sizeof(float) * count));
   DECO_CUDA_TRY(upload(m->theta, host, sizeof(float) * count));   // and the moments: there for every stream
   m->t = 0;
   return DECO_OK;
